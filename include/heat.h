@@ -166,13 +166,12 @@ typedef struct heat_opts {
                            128 cells x this; the operand ring holds 4 or 6 k-stages); 0 =
                            heat_autotune's choice, else 256.  Results do not depend on it        */
     int cooling;        /* HEAT_COOLING_CONTINUOUS (default) or HEAT_COOLING_DISCRETE          */
-    int build_prefetch; /* FP32 matrix build (more than 16 cells, not fused): 1: each segment step
-                           prefetches into L1 the pattern entry 32 entries past the segment's end;
-                           2: no prefetch; 0 (default): heat_autotune's choice if it made one, else
-                           1 on grids of at most 1024 wavelengths and 2 above (measured on a GB300:
-                           4.19 -> 3.89 ms per step of the 4096-cell x 64-grain x 1024-wavelength
-                           workload, 71.4 -> 86.9 ms of the 65536-cell x 32-grain x 2048-wavelength
-                           one).  Results do not depend on it                                 */
+    int build_prefetch; /* FP32 matrix build in one walk per task (more than 16 cells, not fused; run
+                           only where device memory has no room for the two-pass build's prefix
+                           table): 1: each segment step prefetches into L1 the pattern entry 32
+                           entries past the segment's end; 2: no prefetch; 0 (default):
+                           heat_autotune's choice if it made one, else 1 on grids of at most 1024
+                           wavelengths and 2 above.  Results do not depend on it              */
 } heat_opts;
 
 /* kernel classes reported by heat_get_timing */

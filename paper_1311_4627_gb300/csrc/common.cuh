@@ -111,6 +111,56 @@ __device__ __forceinline__ float e1f_small(float z) {
     return fmaf(p, z, 1.0f);
 }
 
+// Two FP32 values in one 64-bit register, for the packed FP32 instructions: each half is rounded as
+// the scalar instruction rounds it, one issue slot does the work of two.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ F2 f2(float a) { return f2(a, a); }
+__device__ __forceinline__ float lo(F2 a) { return __uint_as_float((unsigned)a.v); }
+__device__ __forceinline__ float hi(F2 a) { return __uint_as_float((unsigned)(a.v >> 32)); }
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, f2(-1.0f), a); }  // a - b, one rounding
+
+// The series of e1f, both halves (|z| < 0.5).
+__device__ __forceinline__ F2 e1f_series2(F2 z) {
+    F2 p = f2(1.0f / 40320.0f);
+    p = fma2(p, z, f2(1.0f / 5040.0f));
+    p = fma2(p, z, f2(1.0f / 720.0f));
+    p = fma2(p, z, f2(1.0f / 120.0f));
+    p = fma2(p, z, f2(1.0f / 24.0f));
+    p = fma2(p, z, f2(1.0f / 6.0f));
+    p = fma2(p, z, f2(0.5f));
+    return fma2(p, z, f2(1.0f));
+}
+__device__ __forceinline__ F2 e1f_small2(F2 z) {
+    F2 p = f2(1.0f / 720.0f);
+    p = fma2(p, z, f2(1.0f / 120.0f));
+    p = fma2(p, z, f2(1.0f / 24.0f));
+    p = fma2(p, z, f2(1.0f / 6.0f));
+    p = fma2(p, z, f2(0.5f));
+    return fma2(p, z, f2(1.0f));
+}
+
 // Whether a segment's elements may use e1f_small: every argument there is z = q t with
 // t in [0, dl] and q = su + sC + 2, so |z| <= |q| dl.
 __device__ __forceinline__ bool short_series(float su, float sC, float dl) {
@@ -179,6 +229,19 @@ struct Sum32 {
     }
     __device__ __forceinline__ float val() const { return __fadd_rn(s, c); }
     __device__ __forceinline__ double wide() const { return (double)s + (double)c; }
+};
+
+// Two such sums at once.
+struct Sum32x2 {
+    F2 s{0ull}, c{0ull};
+    __device__ __forceinline__ void add(F2 x) {
+        const F2 t = add2(s, x);
+        const F2 bp = sub2(t, s);
+        const F2 err = add2(sub2(s, sub2(t, bp)), sub2(x, bp));
+        s = t;
+        c = add2(c, err);
+    }
+    __device__ __forceinline__ F2 val() const { return add2(s, c); }
 };
 
 // Widen a non-negative finite float to double with integer operations only

@@ -404,6 +404,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
     std::vector<PatF64> pat64;
     std::vector<PatF32> pat32;
     std::vector<int> seg_ptr((size_t)G * (N + 1), 0);
+    std::vector<int4> pieces, pseg;
     std::vector<SoftF64> soft;
     std::vector<int> soft_off(G + 1, 0);
     std::vector<int> wmax(G, 1);
@@ -414,6 +415,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
     struct Ent {
         int n, e;
         double t;
+        bool diag;
     };
     std::vector<int> diag_e(nbt, 0), diag_ok(nbt, 0);
     std::vector<PointEnt> pent;  // point-rule entries (Eq. heating), column by column
@@ -457,6 +459,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
                 double lf = kHChost / (Elo[f] - E[j]);
                 Ent en;
                 en.e = (int)(band_total + band);
+                en.diag = j == f - 1;
                 RowEnt32 re;
                 re.n = N;  // no photon part unless the pattern loop below sets the segment
                 re.t = re.cat = re.zt = 0.0f;
@@ -502,13 +505,28 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
                 pent.push_back(pe);
             }
         }
-        // pattern: the grain's elements grouped by segment
-        std::stable_sort(ents.begin(), ents.end(), [](const Ent& a, const Ent& b) { return a.n < b.n; });
+        // pattern: the grain's elements grouped by segment, the diagonal ones (which also carry an
+        // intra-bin term) last in each
+        std::stable_sort(ents.begin(), ents.end(),
+                         [](const Ent& a, const Ent& b) { return a.n != b.n ? a.n < b.n : a.diag < b.diag; });
         size_t base = pat64.size();
         size_t k = 0;
         for (int n = 0; n <= N; ++n) {
             while (k < ents.size() && ents[k].n < n) ++k;
             seg_ptr[(size_t)g * (N + 1) + n] = (int)(base + k);
+        }
+        for (size_t b = 0; b < ents.size(); b += kPieceEntries) {
+            const size_t b1 = std::min(ents.size(), b + kPieceEntries);
+            const int s0 = (int)pseg.size();
+            for (size_t i = b; i < b1;) {
+                size_t d = i, e = i;
+                while (d < b1 && ents[d].n == ents[i].n && !ents[d].diag) ++d;
+                for (e = d; e < b1 && ents[e].n == ents[i].n;) ++e;
+                pseg.push_back(make_int4(ents[i].n, (int)(d - b), (int)(e - b), 0));
+                i = e;
+            }
+            pieces.push_back(make_int4(g, (int)(base + b), (int)(base + b1), 0));
+            pieces.push_back(make_int4(s0, (int)pseg.size(), 0, 0));
         }
         for (const Ent& en : ents) {
             size_t kk = (size_t)g * N + en.n;
@@ -574,6 +592,27 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
     }
     pat32.resize(pat32.size() + 64, PatF32{});  // the FP32 build prefetches 32 entries past a segment's end
     ctx->band_per_cell = band_total;
+    ctx->n_pieces = (int)(pieces.size() / 2);
+    std::vector<int4> soft32;
+    soft32.reserve(soft.size() + 1);
+    for (int g = 0; g < G; ++g)
+        for (int i = soft_off[g]; i < soft_off[g + 1]; ++i) {
+            const float t = (float)soft[i].t, ide = invdE32[bin_offset[g] + soft[i].j];
+            int4 r = make_int4(soft[i].n, soft[i].e_diag, 0, 0);
+            std::memcpy(&r.z, &t, 4);
+            std::memcpy(&r.w, &ide, 4);
+            soft32.push_back(r);
+        }
+    soft32.push_back(make_int4(-2, 0, 0, 0));
+    const int GP = (G + 1) / 2;
+    std::vector<float4> seg32(2 * (size_t)GP * N, make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+    for (int q = 0; q < GP; ++q)
+        for (int n = 0; n < N - 1; ++n) {
+            const size_t k = 2 * (size_t)q * N + n, k1 = 2 * q + 1 < G ? k + N : k;
+            const float on = 2 * q + 1 < G ? 1.0f : 0.0f;
+            seg32[(size_t)q * N + n] = make_float4(ca32[k], on * ca32[k1], sC32[k], sC32[k1]);
+            seg32[((size_t)GP + q) * N + n] = make_float4(ce32[k], on * ce32[k1], sC32[k], sC32[k1]);
+        }
     ctx->band_max = 0;
     ctx->wmax_all = *std::max_element(wmax.begin(), wmax.end());
     for (int g = 0; g < G; ++g) ctx->band_max = std::max(ctx->band_max, (int)ctx->grain_band[g]);
@@ -588,7 +627,9 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
         upload(ctx->d_invdE, invdE) || upload(ctx->d_invdE32, invdE32) || upload(ctx->d_Cact, Cact) ||
         upload(ctx->d_sC, sC) || upload(ctx->d_ca32, ca32) || upload(ctx->d_ce32, ce32) ||
         upload(ctx->d_sC32, sC32) || upload(ctx->d_rowptr, rowptr) || upload(ctx->d_wmax, wmax) || upload(ctx->d_pat64, pat64) ||
-        upload(ctx->d_pat32, pat32) || upload(ctx->d_seg_ptr, seg_ptr) || upload(ctx->d_soft, soft) || upload(ctx->d_soft_off, soft_off) ||
+        upload(ctx->d_pat32, pat32) || upload(ctx->d_seg_ptr, seg_ptr) || upload(ctx->d_seg32, seg32) ||
+        upload(ctx->d_soft32, soft32) ||
+        upload(ctx->d_pieces, pieces) || upload(ctx->d_pseg, pseg) || upload(ctx->d_soft, soft) || upload(ctx->d_soft_off, soft_off) ||
         upload(ctx->d_w, ctx->w) || upload(ctx->d_pent, pent) || upload(ctx->d_pcol, pcol) ||
         upload(ctx->d_rent, rent))
         return ctx->fail(HEAT_ENOMEM, "heat_set_grains: device allocation failed");
@@ -694,12 +735,13 @@ static bool uses_fused(const heat_ctx* ctx, const heat_opts& o, int count) {
 
 static int default_chunk(heat_ctx* ctx, int build, int count, int nslots, bool fused) {
     const size_t band_bytes = fused ? 0 : (size_t)ctx->band_per_cell * 32 * (build == 0 ? 8 : 4);
-    const size_t per_group = band_bytes + (size_t)ctx->nbt * 32 * 10 + (size_t)ctx->N * 32 * 16;
+    const size_t phi_bytes = fused ? 0 : (size_t)ctx->G * ctx->N * 32 * (build == 0 ? 8 : 4);
+    const size_t per_group = band_bytes + phi_bytes + (size_t)ctx->nbt * 32 * 10 + (size_t)ctx->N * 32 * 16;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = size_t(16) << 30;
     size_t held = 0;
-    for (auto& sl : ctx->slots) held += sl.ua64.cap + sl.su64.cap + sl.ua32.cap + sl.Bb64.cap + sl.Bb32.cap + sl.xs.cap +
-                                        sl.ep.cap;
+    for (auto& sl : ctx->slots) held += sl.ua64.cap + sl.su64.cap + sl.ua32.cap + sl.Bb64.cap + sl.Bb32.cap + sl.phi.cap +
+                                        sl.xs.cap + sl.ep.cap;
     const size_t budget = std::max<size_t>(size_t(2) << 30, (size_t)(0.45 * (double)(free_b + held)));
     size_t groups = std::max<size_t>(1, budget / (size_t)nslots / per_group);
     size_t want = ((size_t)count + 31) / 32;
@@ -829,6 +871,10 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
     // the recursion's epilogue packs the tensor-core operand (per-grain output, lane-per-cell
     // kernels); P then goes to memory only where the caller asked for it
     const bool pack_in_recur = tc && !si && !fused && count > kSmallCells && !discrete;
+    // the integral form's matrix build in two passes (photon prefixes, then the elements): needs the
+    // prefix table
+    const bool two_pass = !discrete && !fused && count > kSmallCells && o.heating == HEAT_HEATING_INTEGRAL;
+    bool phi_ok[heat_ctx::kMaxSlots] = {};
     // scratch of every slot in use
     bool internal_P = (P_out == nullptr) || o.host_io;
     const bool async_io = o.host_io == 2;
@@ -868,6 +914,9 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
             ok &= !sl.rowscale.ensure(sizeof(float) * (size_t)Cc * Gt);
         }
         if (!ok) return ctx->fail(HEAT_ENOMEM, "heat_solve: scratch allocation failed");
+        // without room for the prefix table the build walks every task's segments once instead
+        phi_ok[k] = two_pass && sl.phi.ensure((build == 0 ? 8 : 4) * (size_t)G * N * Cc) == cudaSuccess;
+        if (two_pass && !phi_ok[k]) (void)cudaGetLastError();
         if (nslots > 1 && !sl.stream) {
             CKR(cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking));
             CKR(cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming));
@@ -912,6 +961,11 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
     gd.band_max = ctx->band_max;
     gd.wmax_all = ctx->wmax_all;
     gd.seg_ptr = ctx->d_seg_ptr.as<int>();
+    gd.seg32 = ctx->d_seg32.as<float4>();
+    gd.soft32 = ctx->d_soft32.as<int4>();
+    gd.pieces = ctx->d_pieces.as<int4>();
+    gd.pseg = ctx->d_pseg.as<int4>();
+    gd.n_pieces = ctx->n_pieces;
     gd.pat64 = ctx->d_pat64.as<PatF64>();
     gd.pat32 = ctx->d_pat32.as<PatF32>();
     gd.soft = ctx->d_soft.as<SoftF64>();
@@ -947,6 +1001,10 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
         ch.ua32 = sl.ua32.as<float>();
         ch.Bb64 = sl.Bb64.as<double>();
         ch.Bb32 = sl.Bb32.as<float>();
+        if (phi_ok[ci % nslots]) {
+            ch.phi64 = build == 0 ? sl.phi.as<double>() : nullptr;
+            ch.phi32 = build == 0 ? nullptr : sl.phi.as<float>();
+        }
         ch.xs = sl.xs.as<double>();
         ch.ep = sl.ep.as<unsigned short>();
         ch.pabs = sl.pabs.as<double>();
@@ -1374,13 +1432,13 @@ void heat_destroy(heat_ctx* ctx) {
     DevBuf* bufs[] = {&ctx->d_lam, &ctx->d_dln, &ctx->d_lam32, &ctx->d_dln32, &ctx->d_bin_off, &ctx->d_cabs,
                       &ctx->d_T, &ctx->d_E, &ctx->d_Cf, &ctx->d_invC, &ctx->d_invdE, &ctx->d_invdE32, &ctx->d_Cact,
                       &ctx->d_sC, &ctx->d_ca32, &ctx->d_ce32, &ctx->d_sC32, &ctx->d_rowptr, &ctx->d_wmax, &ctx->d_seg_ptr,
-                      &ctx->d_pat64, &ctx->d_pat32, &ctx->d_soft, &ctx->d_soft_off, &ctx->d_K, &ctx->d_Kw, &ctx->d_w,
+                      &ctx->d_seg32, &ctx->d_soft32, &ctx->d_pieces, &ctx->d_pseg, &ctx->d_pat64, &ctx->d_pat32, &ctx->d_soft, &ctx->d_soft_off, &ctx->d_K, &ctx->d_Kw, &ctx->d_w,
                       &ctx->d_koff_all, &ctx->d_cde, &ctx->d_pent, &ctx->d_pcol, &ctx->d_kexp, &ctx->d_rent, &ctx->d_gl, &ctx->d_Dtd, &ctx->d_Dtd_off, &ctx->d_Dtd_woff, &ctx->d_Dtd_order, &ctx->d_u_own, &ctx->s_tasks, &ctx->s_tasks_tail, &ctx->d_status};
     for (DevBuf* b : bufs) b->release();
     for (auto& sl : ctx->slots) {
         DevBuf* sb[] = {&sl.ua64, &sl.su64, &sl.ua32, &sl.Bb64, &sl.Bb32, &sl.xs, &sl.ep,   &sl.pabs,
                         &sl.P,    &sl.j,    &sl.led,  &sl.A,    &sl.rowscale, &sl.work, &sl.P_alt, &sl.j_alt,
-                        &sl.led_alt, &sl.phs, &sl.tdq};
+                        &sl.led_alt, &sl.phs, &sl.tdq,  &sl.phi};
         for (DevBuf* b : sb) b->release();
         if (sl.stream) cudaStreamDestroy(sl.stream);
         if (sl.done) cudaEventDestroy(sl.done);

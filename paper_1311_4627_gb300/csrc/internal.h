@@ -51,9 +51,18 @@ struct GrainDev {
     int pat_prefetch;       // nonzero: the FP32 build prefetches into L1 the pattern entry 32 past each segment
     const int* seg_ptr;     // [G][N+1] pattern entries of grain g in segment n at
                             //   seg_ptr[g*(N+1)+n] .. seg_ptr[g*(N+1)+n+1]
+    const float4* seg32;    // [2][ceil(G/2)][N] of two grains (0 in place of a grain past the last): (ca32 of
+                            //   both, sC32 of both), then (ce32 of both, sC32 of both)
+    const int4* pieces;     // [2 n_pieces] runs of pattern entries: (grain, entry begin, entry end, 0),
+                            //   (first and last + 1 of its segment records, 0, 0)
+    const int4* pseg;       // segment records: (segment, first diagonal entry, end), entries counted from the
+                            //   piece's begin; a segment's diagonal elements come last in it
+    int n_pieces;
     const PatF64* pat64;    // pattern entries (FP64 build)
     const PatF32* pat32;    // pattern entries (FP32 build), then 64 zero entries (prefetch margin)
     const SoftF64* soft;    // [nbt - G] per grain, sorted by segment (descending)
+    const int4* soft32;     // the same list for the FP32 walk: (segment, diagonal element, t and 1/(E_{j+1}-E_j) as
+                            //   FP32 bits), then one entry of segment -2
     const int* soft_off;    // [G+1] start of each grain's soft list
     const PointEnt* pent;   // point-rule entries, column by column (u descending within a column)
     const int* pcol;        // [nbt + 1] entries of column j of grain g at pcol[off_g + j] .. pcol[off_g + j + 1]
@@ -75,6 +84,10 @@ struct ChunkDev {
     // band of B, [NG][band_total][32]: element e of group grp, lane l at (grp*band_total + e)*32 + l
     double* Bb64;
     float* Bb32;
+    // photon prefix Phi at every wavelength node, [G][N][Cc], in the build's precision (null: the
+    // one-walk build, which keeps it in registers)
+    double* phi64;
+    float* phi32;
     // per-group bin arrays [NG][nbt][32]
     double* xs;         // X history of the recursion
     unsigned short* ep; // rescale epoch at which each stored X was last written
@@ -101,6 +114,11 @@ struct ChunkDev {
     float* pack_rowscale;
     int pack_tf32, pack_split;
 };
+
+// Pattern entries per piece of the element pass (k_elem): a warp's share of a (grain, 32-cell
+// group).  Short enough that a solve of one group of cells still fills the device (the
+// 64-grain set has about 1700 pieces), long enough that the piece's start costs little.
+constexpr int kPieceEntries = 384;
 
 // Solves of at most this many cells use the element-parallel build and recursion (a block
 // per (cell, grain) for the build, a warp per spectrum with lanes over the band for the

@@ -255,6 +255,351 @@ __global__ void __launch_bounds__(128) k_build(GrainDev gd, ChunkDev ch) {
 }
 
 // ---------------------------------------------------------------------------
+// The build in two passes.  One walk per (grain, 32-cell group) leaves the device to the tasks
+// with the most elements once the others are done (on average 19 of the 48 warps an SM holds were
+// active), and takes as long as its longest task however few the cells.  So:
+//   k_prefix  the walks alone, one warp per (grain, group, direction): forward, Phi at every
+//             wavelength node into phi[g][n][cell]; backward, the intra-bin terms, parked in the
+//             diagonal elements' places of the band, and the absorbed power;
+//   k_elem    the band elements in pieces of kPieceEntries pattern entries: any number of warps,
+//             all alike.  A diagonal element adds the term it finds in its place.
+// The sums run in k_build's order and every expression is k_build's, so B is bit for bit the same.
+// Measured (FP32 build, one walk -> two passes): 4096 cells x 64 grains x 1024 wavelengths 3.88 -> 3.10 ms
+// (elements 2.0 ms, 5.5 TB/s, what the band's 10.2 GB of stores leaves; walks 1.1 ms); 1003 x 37 x 771
+// 2.95 -> 0.75 ms; 4096 x 32 x 2048 with 512 bins 19.9 -> 3.4 ms; 4096 x 80 x 1024 with 512 bins 37.6 -> 11.0 ms.
+// The prefix table costs 4 (8) bytes per grain, wavelength and cell; without room for it the one walk runs.
+// FP64 walks: a warp per (direction, group, grain).
+__global__ void __launch_bounds__(128) k_prefix64(GrainDev gd, ChunkDev ch) {
+    const int N = gd.N, Cc = ch.Cc, lane = threadIdx.x & 31;
+    // the grains of one group and direction in turn, so that the warps of a block read the same fields
+    long long w = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int g = (int)(w % gd.G);
+    w /= gd.G;
+    const int grp = (int)(w % ch.NG), back = (int)(w / ch.NG);
+    if (back > 1) return;
+    const int off = gd.bin_off[g], cc = grp * 32 + lane;
+    const size_t bb = (size_t)grp * gd.band_total * 32 + lane;
+    constexpr int U = 4;  // segments whose loads are in flight together
+    const double* __restrict__ Cact = gd.Cact + (size_t)g * N;
+    const double* __restrict__ sC = gd.sC + (size_t)g * N;
+    const double* __restrict__ ua = ch.ua64 + cc;
+    const double* __restrict__ su = ch.su64 + cc;
+    if (!back) {
+        double* phi = ch.phi64 + (size_t)g * N * Cc + cc;
+        double Phi = 0.0;
+        for (int n0 = 0; n0 < N - 1; n0 += U) {
+            double m[U], e[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                const int n = min(n0 + k, N - 2);
+                const double om = ua[(size_t)n * Cc] * Cact[n], q1 = su[(size_t)n * Cc] + sC[n] + 2.0;
+                const double ln = gd.lam[n], dl = gd.dln[n];
+                const int cls = series_class64(q1, dl);
+                m[k] = om > 0.0 ? om * ln * ln / kH * dl : 0.0;
+                e[k] = om > 0.0 ? (cls ? e1d_by_class(cls, q1 * dl) : e1d(q1 * dl)) : 0.0;
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k)
+                if (n0 + k < N - 1) {
+                    phi[(size_t)(n0 + k) * Cc] = Phi;
+                    Phi = fma(m[k], e[k], Phi);
+                }
+        }
+        phi[(size_t)(N - 1) * Cc] = Phi;
+        return;
+    }
+    const SoftF64* __restrict__ soft = gd.soft;
+    int p = gd.soft_off[g];
+    const int p1 = gd.soft_off[g + 1];
+    while (p < p1 && soft[p].n == N - 1) ++p;  // no photon is too soft: nothing to add
+    int pn = p < p1 ? soft[p].n : -2;
+    double Psi = 0.0;
+    for (int n0 = N - 2; n0 >= 0; n0 -= U) {
+        double m[U], e[U], om[U], q0[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const int n = max(n0 - k, 0);
+            om[k] = ua[(size_t)n * Cc] * Cact[n];
+            q0[k] = su[(size_t)n * Cc] + sC[n] + 1.0;
+            const double dl = gd.dln[n];
+            m[k] = om[k] > 0.0 ? om[k] * gd.lam[n] * dl : 0.0;
+            e[k] = om[k] > 0.0 ? e1d(q0[k] * dl) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const int n = n0 - k;
+            if (n < 0) break;
+            while (pn == n) {
+                const SoftF64 sf = soft[p];
+                double part = 0.0;
+                if (om[k] > 0.0) {
+                    const double L = gd.dln[n] - sf.t;
+                    part = om[k] * gd.lam[n] * exp(q0[k] * sf.t) * L * e1d(q0[k] * L);
+                }
+                ch.Bb64[bb + (size_t)sf.e_diag * 32] = kC * (part + Psi) * gd.invdE[off + sf.j];
+                ++p;
+                pn = p < p1 ? soft[p].n : -2;
+            }
+            Psi = fma(m[k], e[k], Psi);
+        }
+    }
+    for (; p < p1; ++p) ch.Bb64[bb + (size_t)soft[p].e_diag * 32] = kC * Psi * gd.invdE[off + soft[p].j];
+    if (ch.pabs) ch.pabs[(size_t)cc * gd.G + g] = kC * Psi;
+}
+
+// FP32 walks: a warp takes two grains, one direction, one group of cells.  The two grains share the
+// field loads and run through the packed FP32 instructions (each half rounds as the scalar one).
+// Bound by issue and by the few warps a walk has (2048 cells: 44 % of the issue slots, 76
+// instructions per segment and pair); four grains a warp, or scalar instructions with one grain, took
+// 1.06 ms at 2048 cells against 0.62.
+__global__ void __launch_bounds__(128) k_prefix32(GrainDev gd, ChunkDev ch) {
+    const int N = gd.N, Cc = ch.Cc, lane = threadIdx.x & 31, GP = (gd.G + 1) / 2;
+    // the groups of one pair of grains in turn: a block's warps read the same segment table
+    long long w = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int grp = (int)(w % ch.NG);
+    w /= ch.NG;
+    const int q = (int)(w % GP), back = (int)(w / GP), g0 = 2 * q;
+    if (back > 1) return;
+    const bool two = g0 + 1 < gd.G;
+    const int cc = grp * 32 + lane;
+    const int last = N - 2, dir = back ? -1 : 1;
+    const ptrdiff_t cstep = (ptrdiff_t)Cc * dir;
+    // the next segment to load, in the walk's direction
+    const float2* us_p = (const float2*)ch.ua32 + cc + (back ? (size_t)last * Cc : 0);
+    const float4* tab = gd.seg32 + ((size_t)back * GP + q) * N + (back ? last : 0);
+    const float* dln = gd.dln32 + (back ? last : 0);
+    constexpr int U = 4;  // segments loaded together, a batch ahead of their use
+    float2 us[U], us_n[U];
+    float4 c[U], c_n[U];
+    float dl[U], dl_n[U];
+    Sum32x2 S;
+    auto load = [&](int i0, float2(&u)[U], float4(&t)[U], float(&d)[U]) {  // steps i0 .. i0 + U - 1
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (i0 + k <= last) {
+                u[k] = us_p[k * cstep];
+                t[k] = __ldg(tab + k * dir);
+                d[k] = __ldg(dln + k * dir);
+            }
+        us_p += U * cstep;
+        tab += U * dir;
+        dln += U * dir;
+    };
+    // a step's increments v dl E1((su + sC + p + 1) dl) of both grains (0 where v is 0)
+    auto increment = [&](F2 v, F2 qv, F2 d2) {
+        const F2 z = mul2(qv, d2), m = mul2(v, d2);
+        if (fmaxf(fabsf(lo(z)), fabsf(hi(z))) < 0.5f) return mul2(m, e1f_series2(z));
+        return f2(lo(v) > 0.0f ? lo(m) * e1f(lo(z)) : 0.0f, hi(v) > 0.0f ? hi(m) * e1f(hi(z)) : 0.0f);
+    };
+    load(0, us, c, dl);
+    if (!back) {
+        float* phi0 = ch.phi32 + (size_t)g0 * N * Cc + cc;
+        float* phi1 = two ? phi0 + (size_t)N * Cc : phi0;
+        for (int n0 = 0; n0 < N - 1; n0 += U) {
+            load(n0 + U, us_n, c_n, dl_n);
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                if (n0 + k > last) break;
+                const F2 v = S.val();
+                if (two) *phi1 = hi(v);
+                *phi0 = lo(v);
+                phi0 += Cc;
+                phi1 += Cc;
+                const F2 a = mul2(f2(us[k].x), f2(c[k].x, c[k].y));
+                S.add(increment(a, add2(add2(f2(us[k].y), f2(c[k].z, c[k].w)), f2(2.0f)), f2(dl[k])));
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k) us[k] = us_n[k], c[k] = c_n[k], dl[k] = dl_n[k];
+        }
+        if (two) *phi1 = hi(S.val());
+        *phi0 = lo(S.val());
+        return;
+    }
+    float* Bb = ch.Bb32 + (size_t)grp * gd.band_total * 32 + lane;
+    int p[2], p1[2];
+    int4 sf[2], sf_n[2];  // each grain's next two soft-photon records (loaded a record ahead of the test)
+    auto next = [&](int i) {
+        sf[i] = sf_n[i];
+        sf_n[i] = __ldg(gd.soft32 + min(p[i] + 1, p1[i]));
+        if (p[i] >= p1[i]) sf[i].x = -2;
+    };
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int g = min(g0 + i, gd.G - 1);
+        p1[i] = gd.soft_off[g + 1];
+        p[i] = g0 + i < gd.G ? gd.soft_off[g] : p1[i];
+        while (p[i] < p1[i] && gd.soft32[p[i]].x == N - 1) ++p[i];  // no photon is too soft: nothing to add
+        sf_n[i] = __ldg(gd.soft32 + p[i]);
+        next(i);
+    }
+    for (int i0 = 0; i0 < N - 1; i0 += U) {
+        load(i0 + U, us_n, c_n, dl_n);
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            if (i0 + k > last) break;
+            const int n = last - i0 - k;
+            const F2 b = mul2(f2(us[k].x), f2(c[k].x, c[k].y));
+            const F2 q0 = add2(add2(f2(us[k].y), f2(c[k].z, c[k].w)), f2(1.0f));
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                while (sf[i].x == n) {
+                    const int4 r = sf[i];
+                    ++p[i];
+                    next(i);
+                    const float bi = i ? hi(b) : lo(b), qi = i ? hi(q0) : lo(q0);
+                    float part = 0.0f;
+                    if (bi > 0.0f) {
+                        const float ts = __int_as_float(r.z), L = dl[k] - ts;
+                        part = bi * __expf(qi * ts) * L * e1f(qi * L);
+                    }
+                    const float psi = i ? hi(S.val()) : lo(S.val());
+                    Bb[(size_t)r.y * 32] = __fmul_rn(__fadd_rn(part, psi), __int_as_float(r.w));
+                }
+            S.add(increment(b, q0, f2(dl[k])));
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) us[k] = us_n[k], c[k] = c_n[k], dl[k] = dl_n[k];
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        if (g0 + i >= gd.G) break;
+        const float psi_end = i ? hi(S.val()) : lo(S.val());
+        for (; p[i] < p1[i]; ++p[i]) {  // no photon on the grid reaches the next bin: all absorbed power counts
+            const int4 r = __ldg(gd.soft32 + p[i]);
+            Bb[(size_t)r.y * 32] = __fmul_rn(psi_end, __int_as_float(r.w));
+        }
+        if (ch.pabs)
+            ch.pabs[(size_t)cc * gd.G + g0 + i] =
+                i ? (double)hi(S.s) + (double)hi(S.c) : (double)lo(S.s) + (double)lo(S.c);
+    }
+}
+
+// One piece of a grain's pattern entries for up to 8 warps' cells.  The piece's entries and segment
+// records are staged in shared memory, where all warps read them as broadcasts; what a warp loads
+// from memory is its cells' prefix and field values, a segment ahead.
+// FP64: a warp per group of 32 cells, lane = cell.
+__global__ void __launch_bounds__(256) k_elem64(GrainDev gd, ChunkDev ch, int gblocks) {
+    __shared__ __align__(16) PatF64 pat[kPieceEntries];
+    __shared__ __align__(16) int4 seg[kPieceEntries];
+    const int piece = blockIdx.x / gblocks;
+    const int4 pc = gd.pieces[2 * piece], ps = gd.pieces[2 * piece + 1];
+    const int N = gd.N, Cc = ch.Cc, g = pc.x, ne = pc.z - pc.y, ns = ps.y - ps.x;
+    for (int i = threadIdx.x; i < ne; i += blockDim.x) ((int4*)pat)[i] = __ldg((const int4*)(gd.pat64 + pc.y) + i);
+    for (int i = threadIdx.x; i < ns; i += blockDim.x) seg[i] = __ldg(gd.pseg + ps.x + i);
+    __syncthreads();
+    const int grp = (blockIdx.x % gblocks) * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (grp >= ch.NG) return;
+    const int cc = grp * 32 + lane;
+    int k = 0;
+    const double* __restrict__ phi = ch.phi64 + (size_t)g * N * Cc + cc;
+    double* Bb = ch.Bb64 + (size_t)grp * gd.band_total * 32 + lane;
+    for (int s = 0; s < ns; ++s) {
+        const int4 r = seg[s];
+        const int n = r.x;
+        const double Phi = phi[(size_t)n * Cc];
+        if (n == N - 1) {  // at or beyond the last node: the whole grid's prefix
+            for (; k < r.z; ++k) Bb[(size_t)pat[k].e * 32] = Phi;
+            break;
+        }
+        const double om = ch.ua64[(size_t)n * Cc + cc] * gd.Cact[(size_t)g * N + n];
+        const double q1 = ch.su64[(size_t)n * Cc + cc] + gd.sC[(size_t)g * N + n] + 2.0;
+        const double ln = gd.lam[n], a = om * ln * ln / kH;
+        const int cls = series_class64(q1, gd.dln[n]);
+        const double aq = (q1 != 0.0) ? a / q1 : a;
+        auto elem = [&](double t) {
+            if (cls) return Phi + (a * t) * e1d_by_class(cls, q1 * t);
+            return Phi + (q1 != 0.0 ? aq * expm1(q1 * t) : aq * t);
+        };
+        for (; k < r.y; ++k) Bb[(size_t)pat[k].e * 32] = elem(pat[k].t);
+        for (; k < r.z; ++k) {
+            double* q = Bb + (size_t)pat[k].e * 32;
+            *q = elem(pat[k].t) + *q;
+        }
+    }
+}
+
+// FP32: a warp per two groups (64 cells), lane = a cell of each, the two in the halves of the packed
+// FP32 instructions: an entry's constants, its address and every operation serve both.
+__global__ void __launch_bounds__(256) k_elem32(GrainDev gd, ChunkDev ch, int gblocks) {
+    __shared__ __align__(16) PatF32 pat[kPieceEntries];
+    __shared__ __align__(16) int4 seg[kPieceEntries];
+    __shared__ float2 sq[kPieceEntries];  // (sC, dln) of the segments
+    const int piece = blockIdx.x / gblocks;
+    const int4 pc = gd.pieces[2 * piece], ps = gd.pieces[2 * piece + 1];
+    const int N = gd.N, Cc = ch.Cc, g = pc.x, ne = pc.z - pc.y, ns = ps.y - ps.x;
+    for (int i = threadIdx.x; i < ne; i += blockDim.x) ((int4*)pat)[i] = __ldg((const int4*)(gd.pat32 + pc.y) + i);
+    for (int i = threadIdx.x; i < ns; i += blockDim.x) {
+        const int4 r = __ldg(gd.pseg + ps.x + i);
+        seg[i] = r;
+        sq[i] = r.x < N - 1 ? make_float2(gd.sC32[(size_t)g * N + r.x], gd.dln32[r.x]) : make_float2(0.0f, 0.0f);
+    }
+    __syncthreads();
+    const int grp = 2 * ((blockIdx.x % gblocks) * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+    if (grp >= ch.NG) return;
+    const bool two = grp + 1 < ch.NG;  // else the second half repeats the first and is not stored
+    const int cc = grp * 32 + lane, c1 = two ? 32 : 0;
+    const float* __restrict__ phis = ch.phi32 + (size_t)g * N * Cc + cc;
+    const float2* __restrict__ uasu = (const float2*)ch.ua32 + cc;
+    float* B0 = ch.Bb32 + (size_t)grp * gd.band_total * 32 + lane;
+    float* B1 = B0 + (two ? (size_t)gd.band_total * 32 : 0);
+    int k = 0;
+    int4 r = seg[0];
+    float2 ph, ua, ub;  // the next segment's prefix and (u, slope) of both cells
+    auto load = [&] {
+        const size_t n = (size_t)r.x * Cc;
+        ph = make_float2(phis[n], phis[n + c1]);
+        ua = uasu[n];
+        ub = uasu[n + c1];
+    };
+    load();
+    for (int s = 0; s < ns; ++s) {
+        const int n = r.x, kd = r.y, ke = r.z;
+        const F2 phi = f2(ph.x, ph.y), u = f2(ua.x, ub.x), su = f2(ua.y, ub.y);
+        const float2 sc = sq[s];
+        if (s + 1 < ns) {
+            r = seg[s + 1];
+            load();
+        }
+        if (n == N - 1) {  // at or beyond the last node: the whole grid's prefix
+            for (; k < ke; ++k) {
+                const size_t o = (size_t)pat[k].e * 32;
+                __stcs(B0 + o, lo(phi));
+                if (two) __stcs(B1 + o, hi(phi));
+            }
+            break;
+        }
+        // the series is chosen per cell (lanes and halves normally agree), so that a cell's values do not
+        // depend on the cells beside it
+        const bool s0 = short_series(lo(su), sc.x, sc.y), s1 = short_series(hi(su), sc.x, sc.y);
+        auto run = [&](auto e1) {
+            auto elem = [&](const PatF32& a) {
+                return fma2(mul2(u, f2(a.cat)), e1(fma2(su, f2(a.t), f2(a.zt))), phi);
+            };
+#pragma unroll 4
+            for (; k < kd; ++k) {
+                const PatF32 a = pat[k];
+                const F2 b = elem(a);
+                const size_t o = (size_t)a.e * 32;
+                __stcs(B0 + o, lo(b));
+                if (two) __stcs(B1 + o, hi(b));
+            }
+            for (; k < ke; ++k) {  // diagonal elements: plus the intra-bin term parked in their place
+                const PatF32 a = pat[k];
+                const size_t o = (size_t)a.e * 32;
+                const F2 b = add2(elem(a), f2(B0[o], B1[o]));
+                __stcs(B0 + o, lo(b));
+                if (two) __stcs(B1 + o, hi(b));
+            }
+        };
+        if (s0 && s1)
+            run([](F2 z) { return e1f_small2(z); });
+        else
+            run([&](F2 z) { return f2(s0 ? e1f_small(lo(z)) : e1f(lo(z)), s1 ? e1f_small(hi(z)) : e1f(hi(z))); });
+        k = ke;
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Element-parallel build for solves of few cells (ChunkDev::small): the same quantities as
 // k_build with the same expressions; the cumulative sums run in the same order (one thread),
 // so B is bit-identical.
@@ -602,6 +947,21 @@ cudaError_t launch_build(const GrainDev& g, const ChunkDev& ch, int build, cudaS
         return cudaGetLastError();
     }
     if (ch.n_tasks == 0) return cudaSuccess;
+    if (ch.phi64 || ch.phi32) {
+        const long long walks = 2LL * ch.NG * (build == 0 ? g.G : (g.G + 1) / 2);
+        const unsigned wblocks = (unsigned)((walks + 3) / 4);
+        const int units = build == 0 ? ch.NG : (ch.NG + 1) / 2;  // a warp's cells: one group, or two
+        const int warps = std::min(units, 8), gblocks = (units + warps - 1) / warps;
+        const unsigned eblocks = (unsigned)((long long)g.n_pieces * gblocks);
+        if (build == 0) {
+            k_prefix64<<<wblocks, 128, 0, st>>>(g, ch);
+            if (eblocks) k_elem64<<<eblocks, warps * 32, 0, st>>>(g, ch, gblocks);
+        } else {
+            k_prefix32<<<wblocks, 128, 0, st>>>(g, ch);
+            if (eblocks) k_elem32<<<eblocks, warps * 32, 0, st>>>(g, ch, gblocks);
+        }
+        return cudaGetLastError();
+    }
     // one warp per task (measured: a persistent launch with a task counter is no faster)
     auto kern = build == 0 ? k_build<0> : (g.pat_prefetch ? k_build<1, true> : k_build<1, false>);
     kern<<<(unsigned)((ch.n_tasks + 3) / 4), 128, 0, st>>>(g, ch);
