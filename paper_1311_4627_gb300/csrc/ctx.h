@@ -49,7 +49,7 @@ struct heat_ctx {
     int G = 0, nbt = 0;
     std::vector<int> bin_off;
     std::vector<double> w;
-    bool has_w = false;
+    bool has_w = false, w_nonneg = true;  // size weights given; none negative
     long long band_per_cell = 0;
     int max_bins = 0;
     int band_max = 0;  // largest band (elements per cell) of one grain

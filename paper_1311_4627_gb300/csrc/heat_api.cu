@@ -368,6 +368,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
     ctx->has_w = size_weight != nullptr;
     ctx->w.assign(G, 0.0);
     if (size_weight) std::copy(size_weight, size_weight + G, ctx->w.begin());
+    ctx->w_nonneg = std::all_of(ctx->w.begin(), ctx->w.end(), [](double v) { return v >= 0.0; });
     ctx->tasks_NG = -1;
     ctx->tail_NG = -1;
     ctx->tuned_streams = ctx->tuned_chunk = 0;
@@ -1065,10 +1066,10 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
                 if (hs != HEAT_OK) return hs;
             } else if (si)
                 CKR(launch_gemm_f64(cells, N, 1, ctx->d_koff_all.as<int>(), ch.P, nbt, ctx->d_Kw.as<double>(), N, jdst,
-                                    N, 0, o.j_dtype == HEAT_F32, cs));
+                                    N, 0, o.j_dtype == HEAT_F32, ctx->w_nonneg, cs));
             else
                 CKR(launch_gemm_f64(cells, N, G, ctx->d_bin_off.as<int>(), ch.P, nbt, ctx->d_K.as<double>(), N, jdst,
-                                    (long long)G * N, N, o.j_dtype == HEAT_F32, cs));
+                                    (long long)G * N, N, o.j_dtype == HEAT_F32, 1, cs));
             if (o.timing) {
                 cudaEvent_t tb = ctx->take_event();
                 CKR(cudaEventRecord(tb, cs));

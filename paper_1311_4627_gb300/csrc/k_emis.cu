@@ -1,11 +1,11 @@
 // Emissivity contraction (Eq. emission, Eq. emission-lambda) in FP64:
 //   j[c][g][n] = sum_i P[c][off_g + i] K[off_g + i][n],   K = C_abs B_lambda(T_i) [E_i >= hc/lambda_n],
 // and the size-integrated form over the concatenated bins with K scaled by w_g (Eq. convolution).
-// Register-tiled SIMT GEMM on the FP64 FMA pipe: 64 x 64 output tile per block,
-// 16-deep k slices staged in shared memory, 4 x 4 outputs per thread; a thread-per-output
-// form for few rows.
+// Three forms: sums in 64-bit fixed point on the integer pipes (k_gemm_i64), a register-tiled SIMT
+// GEMM on the FP64 FMA pipe for kernels that may be negative, and a thread per output for few rows.
 #include "common.cuh"
 #include "internal.h"
+#include "isum.cuh"
 
 namespace heat {
 
@@ -66,6 +66,141 @@ __global__ void __launch_bounds__(256, 2) k_gemm_f64(int M, int N, const int* __
     }
 }
 
+// The contraction of non-negative operands without the FP64 unit, which takes 64 cycles per warp-wide
+// multiply-add: the sums run in 64-bit fixed point on the integer pipes (isum.cuh), four bins at a time.
+//   * Four bins whose K values lie within a factor of 2^4 in every column of the tile: both operands are
+//     aligned to the largest of their four (at staging, once per 32 or 64 outputs), a product is three
+//     multiply-adds, and one shift per four products brings them to the sum's exponent: about 18 cycles a
+//     product.  What the alignment drops is below 2^-57 of the largest operands' product, 2^-53 of the
+//     four's sum.
+//   * Otherwise (the Wien side, where K climbs steeply) each product is aligned by itself: 36 cycles.
+//   * Four bins without any emission in the tile's columns (K = 0: the bin's energy or temperature is too low)
+//     are left out.
+// Which form a column's bins take depends on K alone, so a cell's result does not depend on the others'.
+// Errors are below the FMA chain's (each row is rounded to FP64 once).  Measured at 512 cells x 64 grains x
+// 1024 wavelengths (36864 bins): MEASURED_GEMM.
+// Tile 64 rows x 32 columns per 256 threads, 4 x 2 outputs a thread, 16 bins staged at a time.
+template <typename TC>
+__global__ void __launch_bounds__(256, 2) k_gemm_i64(int M, int N, const int* __restrict__ koff,
+                                                     const double* __restrict__ A, long long lda,
+                                                     const double* __restrict__ B, long long ldb, TC* __restrict__ C,
+                                                     long long ldc, long long zs) {
+    constexpr int KB = 4;  // fours of bins per stage
+    __shared__ uint4 Ah[KB][64], Al[KB][64], Bh[KB][32], Bl[KB][32];
+    __shared__ int Ae[KB][64], Be[KB][32];
+    __shared__ Mant Am[KB][4][64], Bm[KB][4][32];  // for the one-by-one form
+    __shared__ int flag[KB];  // 0: no emission, 1: aligned, 3: one by one
+    __shared__ int bad[64];   // rows with a NaN or an infinity
+    const int z = blockIdx.z;
+    const int k0 = koff[z], k1 = koff[z + 1];
+    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 32;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    if (tid < 64) bad[tid] = 0;
+    ISum S[4][2];
+    for (int kb = k0; kb < k1; kb += 4 * KB) {
+        if (tid < KB) flag[tid] = 0;
+        __syncthreads();
+        if (tid < 32 * KB) {
+            const int c = tid & 31, q = tid >> 5, n = n0 + c;
+            double x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = kb + 4 * q + u;
+                x[u] = (k < k1 && n < N) ? B[(size_t)k * ldb + n] : 0.0;
+            }
+            const Align4 a = align4(x);
+            Bh[q][c] = make_uint4(a.h[0], a.h[1], a.h[2], a.h[3]);
+            Bl[q][c] = make_uint4(a.l[0], a.l[1], a.l[2], a.l[3]);
+            Be[q][c] = a.E;
+            // compared as integers: the values are not negative (the FP64 unit takes 64 cycles a comparison)
+            const int kn = k1 - (kb + 4 * q);  // bins of this four
+            long long lo = __double_as_longlong(x[0]), hi = lo;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                Bm[q][u][c] = mant(x[u]);
+                if (u < kn) {
+                    lo = min(lo, __double_as_longlong(x[u]));
+                    hi = max(hi, __double_as_longlong(x[u]));
+                }
+            }
+            const int f = hi > 0 ? (hi - lo > (3LL << 52) ? 3 : 1) : 0;  // (a difference of 3 exponents: 2^3 to 2^4)
+            const int any = __reduce_or_sync(0xffffffffu, f);
+            if (c == 0) flag[q] = any;
+        }
+        __syncthreads();
+        // nothing to add (the last stage is kept: it carries a row's NaN into columns without emission)
+        if ((flag[0] | flag[1] | flag[2] | flag[3]) == 0 && kb + 4 * KB < k1) continue;
+        {
+            const int r = tid >> 2, q = tid & 3, m = m0 + r;  // consecutive threads: consecutive fours of a row
+            double x[4];
+            bool nan = false;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = kb + 4 * q + u;
+                x[u] = (m < M && k < k1) ? A[(size_t)m * lda + k] : 0.0;
+                nan |= (__double2hiint(x[u]) & 0x7ff00000) == 0x7ff00000;
+            }
+            const Align4 a = align4(x);
+            Ah[q][r] = make_uint4(a.h[0], a.h[1], a.h[2], a.h[3]);
+            Al[q][r] = make_uint4(a.l[0], a.l[1], a.l[2], a.l[3]);
+            Ae[q][r] = a.E;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) Am[q][u][r] = mant(x[u]);
+            if (nan) bad[r] = 1;
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int q = 0; q < KB; ++q) {
+            const int f = flag[q];
+            if (f == 1) {
+                uint32_t bh[2][4], bl[2][4];
+                int be[2];
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const uint4 h = Bh[q][tx + 16 * s], l = Bl[q][tx + 16 * s];
+                    bh[s][0] = h.x, bh[s][1] = h.y, bh[s][2] = h.z, bh[s][3] = h.w;
+                    bl[s][0] = l.x, bl[s][1] = l.y, bl[s][2] = l.z, bl[s][3] = l.w;
+                    be[s] = Be[q][tx + 16 * s];
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint4 h = Ah[q][ty + 16 * r], l = Al[q][ty + 16 * r];
+                    const uint32_t ah[4] = {h.x, h.y, h.z, h.w}, al[4] = {l.x, l.y, l.z, l.w};
+                    const int ae = Ae[q][ty + 16 * r];
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) add_aligned4(S[r][s], ah, al, ae, bh[s], bl[s], be[s]);
+                }
+            } else if (f) {
+                Mant b[2][4];
+#pragma unroll
+                for (int s = 0; s < 2; ++s)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) b[s][u] = Bm[q][u][tx + 16 * s];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    Mant a[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) a[u] = Am[q][u][ty + 16 * r];
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) add_each4(S[r][s], a, b[s]);
+                }
+            }
+        }
+        __syncthreads();
+    }
+    TC* Cz = C + (size_t)z * zs;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int m = m0 + ty + 16 * r;
+        if (m >= M) continue;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const int n = n0 + tx + 16 * s;
+            if (n < N) Cz[(size_t)m * ldc + n] = bad[ty + 16 * r] ? (TC)NAN : (TC)S[r][s].value<0>();
+        }
+    }
+}
+
 // Few rows (solves of few cells): a thread per output, threads along n (coalesced rows of K),
 // one accumulator in ascending k as in k_gemm_f64, so both give the same bits; the 64-row
 // tile above would spend 64 FMAs per useful one on a single cell.
@@ -83,7 +218,8 @@ __global__ void __launch_bounds__(128) k_gemv_f64(int N, const int* __restrict__
 }
 
 cudaError_t launch_gemm_f64(int M, int N, int nz, const int* koff, const double* A, long long lda, const double* B,
-                            long long ldb, void* C, long long ldc, long long zstride_c, int c_is_f32, cudaStream_t st) {
+                            long long ldb, void* C, long long ldc, long long zstride_c, int c_is_f32, int b_nonneg,
+                            cudaStream_t st) {
     if (M <= 0 || N <= 0 || nz <= 0) return cudaSuccess;
     if (M <= kSmallCells) {
         dim3 g1((N + 127) / 128, M, nz);
@@ -91,6 +227,14 @@ cudaError_t launch_gemm_f64(int M, int N, int nz, const int* koff, const double*
             k_gemv_f64<float><<<g1, 128, 0, st>>>(N, koff, A, lda, B, ldb, (float*)C, ldc, zstride_c);
         else
             k_gemv_f64<double><<<g1, 128, 0, st>>>(N, koff, A, lda, B, ldb, (double*)C, ldc, zstride_c);
+        return cudaGetLastError();
+    }
+    if (b_nonneg) {
+        dim3 grid((N + 31) / 32, (M + 63) / 64, nz);
+        if (c_is_f32)
+            k_gemm_i64<float><<<grid, 256, 0, st>>>(M, N, koff, A, lda, B, ldb, (float*)C, ldc, zstride_c);
+        else
+            k_gemm_i64<double><<<grid, 256, 0, st>>>(M, N, koff, A, lda, B, ldb, (double*)C, ldc, zstride_c);
         return cudaGetLastError();
     }
     dim3 grid((N + 63) / 64, (M + 63) / 64, nz);
