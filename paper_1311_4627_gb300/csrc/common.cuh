@@ -21,10 +21,13 @@ constexpr int kStatTimeout = 4;   // bounded wait gave up
 // the segments in order and fills every element whose transition wavelength
 // hc/(Elo_f - E_j) lies in the current one).  e is the element's index in the band
 // storage (row-major over f, then j); t = ln(lambda_fj / lambda_n), 0 past the last node.
-struct __align__(16) PatF64 {
+// tau = t / ln(lambda_{n+1}/lambda_n) in Q60 (fix60.cuh).  A diagonal element (f = j + 1) has in j its lower
+// bin's index over all grains.
+struct __align__(8) PatF64 {
     int e;
-    int pad;
+    int j;
     double t;
+    int64_t tau;
 };
 
 // FP32 build: with a_n = u_n ca_n and z = (su_n + sC_n + 2) t,
@@ -60,6 +63,7 @@ struct __align__(8) PointEnt {
     int n;
     double t;
     double fac;
+    int64_t tau;  // t / ln(lambda_{n+1}/lambda_n) in Q60
 };
 
 // Soft-photon abscissa for the intra-bin term of row j+1:
@@ -74,6 +78,7 @@ struct SoftF64 {
     double t;
     int e_diag;
     int diag_in_band;
+    int64_t tau;  // t / ln(lambda_{n+1}/lambda_n) in Q60
 };
 
 // X > 2^800 for a positive finite double, tested on the exponent bits (integer pipe).
@@ -169,48 +174,6 @@ __device__ __forceinline__ bool short_series(float su, float sC, float dl) {
 
 __device__ __forceinline__ double e1d(double z) {
     return z == 0.0 ? 1.0 : expm1(z) / z;
-}
-
-// E1(z) in FP64 for |z| <= 1/4 from its Taylor series sum_{k>=0} z^k / (k+1)!, to k = 12
-// (the first dropped term is below 2e-19 relative): 12 FMAs instead of expm1 and a divide.
-__device__ __forceinline__ double e1d_series(double z) {
-    double p = 1.0 / 6227020800.0;  // 1/13!
-    p = fma(p, z, 1.0 / 479001600.0);
-    p = fma(p, z, 1.0 / 39916800.0);
-    p = fma(p, z, 1.0 / 3628800.0);
-    p = fma(p, z, 1.0 / 362880.0);
-    p = fma(p, z, 1.0 / 40320.0);
-    p = fma(p, z, 1.0 / 5040.0);
-    p = fma(p, z, 1.0 / 720.0);
-    p = fma(p, z, 1.0 / 120.0);
-    p = fma(p, z, 1.0 / 24.0);
-    p = fma(p, z, 1.0 / 6.0);
-    p = fma(p, z, 0.5);
-    return fma(p, z, 1.0);
-}
-
-// The same for |z| <= 1/16, to k = 8 (first dropped term below 5e-18 relative): 8 FMAs.
-__device__ __forceinline__ double e1d_series_short(double z) {
-    double p = 1.0 / 362880.0;  // 1/9!
-    p = fma(p, z, 1.0 / 40320.0);
-    p = fma(p, z, 1.0 / 5040.0);
-    p = fma(p, z, 1.0 / 720.0);
-    p = fma(p, z, 1.0 / 120.0);
-    p = fma(p, z, 1.0 / 24.0);
-    p = fma(p, z, 1.0 / 6.0);
-    p = fma(p, z, 0.5);
-    return fma(p, z, 1.0);
-}
-
-// Which FP64 form serves every argument z = q t with t in [0, dl] (per cell): 2 = the short
-// series (|z| <= 1/16), 1 = the series (|z| <= 1/4), 0 = the library expm1.
-__device__ __forceinline__ int series_class64(double q, double dl) {
-    const double zmax = fabs(q) * dl;
-    return zmax <= 0.0625 ? 2 : (zmax <= 0.25 ? 1 : 0);
-}
-__device__ __forceinline__ bool short_series64(double q, double dl) { return series_class64(q, dl) != 0; }
-__device__ __forceinline__ double e1d_by_class(int cls, double z) {
-    return cls == 2 ? e1d_series_short(z) : e1d_series(z);
 }
 
 // Compensated FP32 running sum (Knuth's TwoSum error term collected in c): s + c carries the

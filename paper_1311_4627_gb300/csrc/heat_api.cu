@@ -84,6 +84,13 @@ int segment_of(const std::vector<double>& lam, double x) {
     return lo;
 }
 
+// offset t in segment n as a fraction of the segment, in Q60 (0 outside the grid's segments)
+int64_t tau_q60(const std::vector<double>& lam, int n, double t) {
+    if (n < 0 || n + 1 >= (int)lam.size()) return 0;
+    const double tau = t / std::log(lam[n + 1] / lam[n]);
+    return (int64_t)(std::min(std::max(tau, 0.0), 1.0) * 0x1p60);
+}
+
 template <typename T>
 cudaError_t upload(DevBuf& b, const std::vector<T>& v) {
     size_t bytes = std::max<size_t>(v.size() * sizeof(T), 16);
@@ -383,6 +390,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
 
     // per-grain cross-section tables
     std::vector<double> Cact((size_t)G * N, 0.0), sC((size_t)G * N, 0.0);
+    std::vector<double> ca64((size_t)G * N, 0.0), ce64((size_t)G * N, 0.0);
     std::vector<float> ca32((size_t)G * N, 0.0f), ce32((size_t)G * N, 0.0f), sC32((size_t)G * N, 0.0f);
     for (int g = 0; g < G; ++g) {
         const double* C = c_abs_cm2 + (size_t)g * N;
@@ -391,6 +399,8 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
                 size_t k = (size_t)g * N + n;
                 Cact[k] = C[n];
                 sC[k] = std::log(C[n + 1] / C[n]) / std::log(lam[n + 1] / lam[n]);
+                ca64[k] = C[n] * lam[n] * lam[n] / kHhost;
+                ce64[k] = C[n] * lam[n];
                 ca32[k] = (float)(C[n] * lam[n] * lam[n] / kHhost);
                 ce32[k] = (float)(kChost * C[n] * lam[n]);
                 sC32[k] = (float)sC[k];
@@ -405,7 +415,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
     std::vector<PatF64> pat64;
     std::vector<PatF32> pat32;
     std::vector<int> seg_ptr((size_t)G * (N + 1), 0);
-    std::vector<int4> pieces, pseg;
+    std::vector<int4> pieces, pseg, cpieces;
     std::vector<SoftF64> soft;
     std::vector<int> soft_off(G + 1, 0);
     std::vector<int> wmax(G, 1);
@@ -416,7 +426,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
     struct Ent {
         int n, e;
         double t;
-        bool diag;
+        int diag;  // for a diagonal element, 1 + the lower bin's index over all grains, else 0
     };
     std::vector<int> diag_e(nbt, 0), diag_ok(nbt, 0);
     std::vector<PointEnt> pent;  // point-rule entries (Eq. heating), column by column
@@ -460,7 +470,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
                 double lf = kHChost / (Elo[f] - E[j]);
                 Ent en;
                 en.e = (int)(band_total + band);
-                en.diag = j == f - 1;
+                en.diag = j == f - 1 ? off + j + 1 : 0;
                 RowEnt32 re;
                 re.n = N;  // no photon part unless the pattern loop below sets the segment
                 re.t = re.cat = re.zt = 0.0f;
@@ -485,7 +495,13 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
         // jlo(f) does not decrease with f; every element the point rule can make non-zero
         // (E_u - E_j <= hc/lambda_0) lies in the band, and the band's other elements take the
         // column's suffix sum with T = 0
+        int cp0 = 0, ce0 = (int)pent.size();  // the current run of columns
         for (int j = 0; j < nb; ++j) {
+            if ((int)pent.size() - ce0 >= kPointEntries) {
+                cpieces.push_back(make_int4(g, cp0, j, 0));
+                cp0 = j;
+                ce0 = (int)pent.size();
+            }
             pcol[off + j] = (int)pent.size();
             int F = j;
             while (F + 1 <= M && row_jlo[F + 1] <= j) ++F;
@@ -498,18 +514,21 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
                     pe.n = segment_of(lam, x);
                     pe.t = std::log(x / lam[pe.n]);
                     pe.fac = x * x * x * dE / (kHhost * kHhost * kChost);
+                    pe.tau = tau_q60(lam, pe.n, pe.t);
                 } else {
                     pe.n = -1;
+                    pe.tau = 0;
                     pe.t = 0.0;
                     pe.fac = 0.0;
                 }
                 pent.push_back(pe);
             }
         }
+        cpieces.push_back(make_int4(g, cp0, nb, 0));
         // pattern: the grain's elements grouped by segment, the diagonal ones (which also carry an
         // intra-bin term) last in each
         std::stable_sort(ents.begin(), ents.end(),
-                         [](const Ent& a, const Ent& b) { return a.n != b.n ? a.n < b.n : a.diag < b.diag; });
+                         [](const Ent& a, const Ent& b) { return a.n != b.n ? a.n < b.n : (a.diag > 0) < (b.diag > 0); });
         size_t base = pat64.size();
         size_t k = 0;
         for (int n = 0; n <= N; ++n) {
@@ -535,8 +554,9 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
             double s2 = (en.n < N - 1) ? sC[kk] + 2.0 : 0.0;
             PatF64 a;
             a.e = en.e;
-            a.pad = en.n;
+            a.j = en.diag - 1;
             a.t = en.t;
+            a.tau = tau_q60(lam, en.n, en.t);
             PatF32 b;
             b.e = en.e;
             b.t = (float)en.t;
@@ -569,6 +589,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
                 sf.n = segment_of(lam, ls);
                 sf.t = std::log(ls / lam[sf.n]);
             }
+            sf.tau = tau_q60(lam, sf.n, sf.t);
             sg.push_back(sf);
         }
         std::stable_sort(sg.begin(), sg.end(), [](const SoftF64& a, const SoftF64& b) { return a.n > b.n; });
@@ -594,6 +615,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
     pat32.resize(pat32.size() + 64, PatF32{});  // the FP32 build prefetches 32 entries past a segment's end
     ctx->band_per_cell = band_total;
     ctx->n_pieces = (int)(pieces.size() / 2);
+    ctx->n_cpieces = (int)cpieces.size();
     std::vector<int4> soft32;
     soft32.reserve(soft.size() + 1);
     for (int g = 0; g < G; ++g)
@@ -629,6 +651,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
         upload(ctx->d_sC, sC) || upload(ctx->d_ca32, ca32) || upload(ctx->d_ce32, ce32) ||
         upload(ctx->d_sC32, sC32) || upload(ctx->d_rowptr, rowptr) || upload(ctx->d_wmax, wmax) || upload(ctx->d_pat64, pat64) ||
         upload(ctx->d_pat32, pat32) || upload(ctx->d_seg_ptr, seg_ptr) || upload(ctx->d_seg32, seg32) ||
+        upload(ctx->d_ca64, ca64) || upload(ctx->d_ce64, ce64) || upload(ctx->d_cpieces, cpieces) ||
         upload(ctx->d_soft32, soft32) ||
         upload(ctx->d_pieces, pieces) || upload(ctx->d_pseg, pseg) || upload(ctx->d_soft, soft) || upload(ctx->d_soft_off, soft_off) ||
         upload(ctx->d_w, ctx->w) || upload(ctx->d_pent, pent) || upload(ctx->d_pcol, pcol) ||
@@ -945,6 +968,10 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
     gd.bin_off = ctx->d_bin_off.as<int>();
     gd.Cact = ctx->d_Cact.as<double>();
     gd.sC = ctx->d_sC.as<double>();
+    gd.ca64 = ctx->d_ca64.as<double>();
+    gd.ce64 = ctx->d_ce64.as<double>();
+    gd.cpieces = ctx->d_cpieces.as<int4>();
+    gd.n_cpieces = ctx->n_cpieces;
     gd.lam32 = ctx->d_lam32.as<float>();
     gd.dln32 = ctx->d_dln32.as<float>();
     gd.ca32 = ctx->d_ca32.as<float>();
@@ -1433,7 +1460,7 @@ void heat_destroy(heat_ctx* ctx) {
     DevBuf* bufs[] = {&ctx->d_lam, &ctx->d_dln, &ctx->d_lam32, &ctx->d_dln32, &ctx->d_bin_off, &ctx->d_cabs,
                       &ctx->d_T, &ctx->d_E, &ctx->d_Cf, &ctx->d_invC, &ctx->d_invdE, &ctx->d_invdE32, &ctx->d_Cact,
                       &ctx->d_sC, &ctx->d_ca32, &ctx->d_ce32, &ctx->d_sC32, &ctx->d_rowptr, &ctx->d_wmax, &ctx->d_seg_ptr,
-                      &ctx->d_seg32, &ctx->d_soft32, &ctx->d_pieces, &ctx->d_pseg, &ctx->d_pat64, &ctx->d_pat32, &ctx->d_soft, &ctx->d_soft_off, &ctx->d_K, &ctx->d_Kw, &ctx->d_w,
+                      &ctx->d_seg32, &ctx->d_soft32, &ctx->d_ca64, &ctx->d_ce64, &ctx->d_cpieces, &ctx->d_pieces, &ctx->d_pseg, &ctx->d_pat64, &ctx->d_pat32, &ctx->d_soft, &ctx->d_soft_off, &ctx->d_K, &ctx->d_Kw, &ctx->d_w,
                       &ctx->d_koff_all, &ctx->d_cde, &ctx->d_pent, &ctx->d_pcol, &ctx->d_kexp, &ctx->d_rent, &ctx->d_gl, &ctx->d_Dtd, &ctx->d_Dtd_off, &ctx->d_Dtd_woff, &ctx->d_Dtd_order, &ctx->d_u_own, &ctx->s_tasks, &ctx->s_tasks_tail, &ctx->d_status};
     for (DevBuf* b : bufs) b->release();
     for (auto& sl : ctx->slots) {
@@ -1484,6 +1511,8 @@ __attribute__((visibility("hidden"))) heat_status heat_internal_grain_view(heat_
     gd->bin_off = ctx->d_bin_off.as<int>();
     gd->Cact = ctx->d_Cact.as<double>();
     gd->sC = ctx->d_sC.as<double>();
+    gd->ca64 = ctx->d_ca64.as<double>();
+    gd->ce64 = ctx->d_ce64.as<double>();
     gd->lam32 = ctx->d_lam32.as<float>();
     gd->dln32 = ctx->d_dln32.as<float>();
     gd->ca32 = ctx->d_ca32.as<float>();

@@ -31,6 +31,8 @@ struct GrainDev {
     const int* bin_off; // [G+1]
     const double* Cact;     // [G][N] C_n if the C segment n is active (both ends > 0), else 0
     const double* sC;       // [G][N] log-log slope of C on segment n (0 if inactive)
+    const double* ca64;     // [G][N] C_n lambda_n^2 / h on active C segments, else 0
+    const double* ce64;     // [G][N] C_n lambda_n on active C segments, else 0
     const float* lam32;     // [N]   FP32 copies for the FP32 build
     const float* dln32;     // [N-1]
     const float* ca32;      // [G][N] C_n lambda_n^2 / h on active C segments, else 0
@@ -65,6 +67,8 @@ struct GrainDev {
                             //   FP32 bits), then one entry of segment -2
     const int* soft_off;    // [G+1] start of each grain's soft list
     const PointEnt* pent;   // point-rule entries, column by column (u descending within a column)
+    const int4* cpieces;    // [n_cpieces] runs of point-rule columns: (grain, first column, last + 1, 0)
+    int n_cpieces;
     const int* pcol;        // [nbt + 1] entries of column j of grain g at pcol[off_g + j] .. pcol[off_g + j + 1]
     const int* kexp;        // [nbt] biased binary exponent of max_lambda K[i][lambda] (-100000: none)
     const RowEnt32* rent;   // [band_total] every band element in band (row) order, for the fused kernel
@@ -119,6 +123,8 @@ struct ChunkDev {
 // group).  Short enough that a solve of one group of cells still fills the device (the
 // 64-grain set has about 1700 pieces), long enough that the piece's start costs little.
 constexpr int kPieceEntries = 384;
+// Entries per run of columns of the point-rule build (a warp's share of a (grain, 32-cell group)).
+constexpr int kPointEntries = 256;
 
 // Solves of at most this many cells use the element-parallel build and recursion (a block
 // per (cell, grain) for the build, a warp per spectrum with lanes over the band for the

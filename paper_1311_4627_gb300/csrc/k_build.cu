@@ -5,6 +5,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "fix60.cuh"
 #include "internal.h"
 
 namespace heat {
@@ -66,6 +67,60 @@ __global__ void k_field(int N, const double* __restrict__ dln, const TU* __restr
 }
 
 // ---------------------------------------------------------------------------
+// FP64 build: a segment's pieces, shared by every kernel of the exact path.  With Omega = u C, slope q - p - 1
+// and Z = q dln, the segment's integral is v dln E1(Z) and up to the fraction tau of it v t E1(Z tau); E1 in 60-bit
+// fixed point where |Z| < 1 (fix60.cuh; about 150 cycles of the integer pipes instead of 8 to 12 FP64
+// multiply-adds of 64 cycles), else the library's expm1.
+__device__ __forceinline__ double e1_of(double Z) {
+    const int cls = e1_class(Z);
+    return cls ? from_q60(e1_q60(cls, to_q60(Z))) : e1d(Z);
+}
+// Phi (Psi) after a segment: + v dln E1(Z)
+__device__ __forceinline__ double add_segment(double sum, double v, double q, double dl) {
+    return v > 0.0 ? fma(v * dl, e1_of(q * dl), sum) : sum;
+}
+struct SegF64 {
+    double a, q1, aq;  // C_n u_n lambda_n^2 / h, slope + 2; a / q1 where the library's expm1 serves
+    int64_t Z;         // q1 dln in Q60
+    int cls;
+    __device__ __forceinline__ SegF64(const GrainDev& gd, int g, int n, double ua, double su) {
+        a = ua * gd.ca64[(size_t)g * gd.N + n];
+        q1 = su + gd.sC[(size_t)g * gd.N + n] + 2.0;
+        const double z = q1 * gd.dln[n];
+        cls = e1_class(z);
+        Z = cls ? to_q60(z) : 0;
+        aq = cls ? 0.0 : a / q1;
+    }
+    // B at offset t (fraction tau) of the segment
+    __device__ __forceinline__ double element(double Phi, double t, int64_t tau) const {
+        if (cls) return fma(a * t, from_q60(e1_q60(cls, mul_q60(Z, tau))), Phi);
+        return fma(aq, expm1(q1 * t), Phi);
+    }
+};
+// The intra-bin term of a bin whose soft photons begin at offset t (fraction tau) of segment n, with Psi the
+// integral of Omega beyond the segment: c (int from t to the segment's end + Psi) / (E_{j+1} - E_j).  The part of
+// the segment is the difference of two fixed-point values, exact to 2^-58 of the whole segment's.
+__device__ __forceinline__ double soft_term(const GrainDev& gd, int g, int n, double ua, double su, double t,
+                                            int64_t tau, double Psi, double invdE) {
+    const double b = ua * gd.ce64[(size_t)g * gd.N + n], q0 = su + gd.sC[(size_t)g * gd.N + n] + 1.0;
+    const double dl = gd.dln[n], z = q0 * dl;
+    double part = 0.0;
+    if (b > 0.0) {
+        const int cls = e1_class(z);
+        if (cls) {
+            const int64_t Z = to_q60(z);
+            const int64_t d = e1_q60(cls, Z) - mul_q60(tau, e1_q60(cls, mul_q60(Z, tau)));
+            part = d > 0 ? (b * dl) * from_q60(d) : 0.0;
+        } else {
+            const double L = dl - t;
+            part = b * exp(q0 * t) * L * e1d(q0 * L);
+        }
+    }
+    return __dmul_rn(__dmul_rn(kC, __dadd_rn(part, Psi)), invdE);
+}
+__device__ __forceinline__ double soft_end(double Psi, double invdE) { return __dmul_rn(__dmul_rn(kC, Psi), invdE); }
+
+// ---------------------------------------------------------------------------
 // k_build: the matrix-build kernel.  One warp per task (grain x 32 cells), one lane
 // per cell.  With Omega = u C on the log-log interpolant (Eq. interpolation), slope
 // s_n and q = s_n + p + 1 on segment n:
@@ -94,69 +149,35 @@ __device__ __forceinline__ void build_task(const GrainDev& gd, const ChunkDev& c
     double Phi = 0.0;
 
     if (BUILD == 0) {
-        const double* Cact = gd.Cact + (size_t)g * N;
         const double* sC = gd.sC + (size_t)g * N;
         for (int n = 0; n < N - 1; ++n) {
-            double ua = ch.ua64[(size_t)n * Cc + cc], su = ch.su64[(size_t)n * Cc + cc];
-            double om = ua * Cact[n];
-            double q1 = su + sC[n] + 2.0;
-            double ln = gd.lam[n];
-            double a = om * ln * ln / kH;
-            const double dl = gd.dln[n];
-            const int cls = series_class64(q1, dl);  // per cell, like the FP32 build's series choice
-            if (cls == 2) {
-                for (int k = sp[n]; k < sp[n + 1]; ++k) {
-                    PatF64 pt = gd.pat64[k];
-                    ch.Bb64[bb + (size_t)pt.e * 32] = Phi + (a * pt.t) * e1d_series_short(q1 * pt.t);
-                }
-                if (om > 0.0) Phi += a * dl * e1d_series_short(q1 * dl);
-            } else if (cls == 1) {
-                for (int k = sp[n]; k < sp[n + 1]; ++k) {
-                    PatF64 pt = gd.pat64[k];
-                    ch.Bb64[bb + (size_t)pt.e * 32] = Phi + (a * pt.t) * e1d_series(q1 * pt.t);
-                }
-                if (om > 0.0) Phi += a * dl * e1d_series(q1 * dl);
-            } else {
-                double aq = (q1 != 0.0) ? a / q1 : a;
-                for (int k = sp[n]; k < sp[n + 1]; ++k) {
-                    PatF64 pt = gd.pat64[k];
-                    double B = Phi + (q1 != 0.0 ? aq * expm1(q1 * pt.t) : aq * pt.t);
-                    ch.Bb64[bb + (size_t)pt.e * 32] = B;
-                }
-                if (om > 0.0) Phi += a * dl * e1d(q1 * dl);
+            const double ua = ch.ua64[(size_t)n * Cc + cc], su = ch.su64[(size_t)n * Cc + cc];
+            const SegF64 sg(gd, g, n, ua, su);
+            for (int k = sp[n]; k < sp[n + 1]; ++k) {
+                const PatF64 pt = gd.pat64[k];
+                ch.Bb64[bb + (size_t)pt.e * 32] = sg.element(Phi, pt.t, pt.tau);
             }
+            Phi = add_segment(Phi, sg.a, sg.q1, gd.dln[n]);
         }
         for (int k = sp[N - 1]; k < sp[N]; ++k) ch.Bb64[bb + (size_t)gd.pat64[k].e * 32] = Phi;
 
         // intra-bin terms go into the diagonal elements (j+1, j) of the band
         auto put64 = [&](const SoftF64& sf, double v) {
             size_t ix = bb + (size_t)sf.e_diag * 32;
-            ch.Bb64[ix] = (sf.diag_in_band ? ch.Bb64[ix] : 0.0) + v;
+            ch.Bb64[ix] = sf.diag_in_band ? __dadd_rn(ch.Bb64[ix], v) : v;
         };
-        while (p < p1 && soft[p].n == N - 1) {
-            put64(soft[p], 0.0);
-            ++p;
-        }
+        while (p < p1 && soft[p].n == N - 1) ++p;  // no photon is too soft: nothing to add
         double Psi = 0.0;  // int Omega from lambda_{n+1} to lambda_{N-1}
         for (int n = N - 2; n >= 0; --n) {
-            double ua = ch.ua64[(size_t)n * Cc + cc], su = ch.su64[(size_t)n * Cc + cc];
-            double om = ua * Cact[n];
-            double q0 = su + sC[n] + 1.0;
-            double b = om * gd.lam[n];
-            double dl = gd.dln[n];
+            const double ua = ch.ua64[(size_t)n * Cc + cc], su = ch.su64[(size_t)n * Cc + cc];
             while (p < p1 && soft[p].n == n) {
-                SoftF64 sf = soft[p];
-                double part = 0.0;
-                if (om > 0.0) {
-                    double L = dl - sf.t;
-                    part = b * exp(q0 * sf.t) * L * e1d(q0 * L);
-                }
-                put64(sf, kC * (part + Psi) * gd.invdE[off + sf.j]);
+                const SoftF64 sf = soft[p];
+                put64(sf, soft_term(gd, g, n, ua, su, sf.t, sf.tau, Psi, gd.invdE[off + sf.j]));
                 ++p;
             }
-            if (om > 0.0) Psi += b * dl * e1d(q0 * dl);
+            Psi = add_segment(Psi, ua * gd.ce64[(size_t)g * N + n], su + sC[n] + 1.0, gd.dln[n]);
         }
-        for (; p < p1; ++p) put64(soft[p], kC * Psi * gd.invdE[off + soft[p].j]);
+        for (; p < p1; ++p) put64(soft[p], soft_end(Psi, gd.invdE[off + soft[p].j]));
         if (ch.pabs) ch.pabs[(size_t)cc * gd.G + g] = kC * Psi;
     } else {
         const float* ca = gd.ca32 + (size_t)g * N;
@@ -268,7 +289,8 @@ __global__ void __launch_bounds__(128) k_build(GrainDev gd, ChunkDev ch) {
 // (elements 2.0 ms, 5.5 TB/s, what the band's 10.2 GB of stores leaves; walks 1.1 ms); 1003 x 37 x 771
 // 2.95 -> 0.75 ms; 4096 x 32 x 2048 with 512 bins 19.9 -> 3.4 ms; 4096 x 80 x 1024 with 512 bins 37.6 -> 11.0 ms.
 // The prefix table costs 4 (8) bytes per grain, wavelength and cell; without room for it the one walk runs.
-// FP64 walks: a warp per (direction, group, grain).
+// FP64 walks: a warp per (direction, group, grain).  Backward, a diagonal element's place takes Psi, from which
+// the element pass makes the intra-bin term.
 __global__ void __launch_bounds__(128) k_prefix64(GrainDev gd, ChunkDev ch) {
     const int N = gd.N, Cc = ch.Cc, lane = threadIdx.x & 31;
     // the grains of one group and direction in turn, so that the warps of a block read the same fields
@@ -279,72 +301,51 @@ __global__ void __launch_bounds__(128) k_prefix64(GrainDev gd, ChunkDev ch) {
     if (back > 1) return;
     const int off = gd.bin_off[g], cc = grp * 32 + lane;
     const size_t bb = (size_t)grp * gd.band_total * 32 + lane;
-    constexpr int U = 4;  // segments whose loads are in flight together
-    const double* __restrict__ Cact = gd.Cact + (size_t)g * N;
+    constexpr int U = 2;  // segments whose series run side by side
+    const double* __restrict__ cf = (back ? gd.ce64 : gd.ca64) + (size_t)g * N;
     const double* __restrict__ sC = gd.sC + (size_t)g * N;
     const double* __restrict__ ua = ch.ua64 + cc;
     const double* __restrict__ su = ch.su64 + cc;
-    if (!back) {
-        double* phi = ch.phi64 + (size_t)g * N * Cc + cc;
-        double Phi = 0.0;
-        for (int n0 = 0; n0 < N - 1; n0 += U) {
-            double m[U], e[U];
-#pragma unroll
-            for (int k = 0; k < U; ++k) {
-                const int n = min(n0 + k, N - 2);
-                const double om = ua[(size_t)n * Cc] * Cact[n], q1 = su[(size_t)n * Cc] + sC[n] + 2.0;
-                const double ln = gd.lam[n], dl = gd.dln[n];
-                const int cls = series_class64(q1, dl);
-                m[k] = om > 0.0 ? om * ln * ln / kH * dl : 0.0;
-                e[k] = om > 0.0 ? (cls ? e1d_by_class(cls, q1 * dl) : e1d(q1 * dl)) : 0.0;
-            }
-#pragma unroll
-            for (int k = 0; k < U; ++k)
-                if (n0 + k < N - 1) {
-                    phi[(size_t)(n0 + k) * Cc] = Phi;
-                    Phi = fma(m[k], e[k], Phi);
-                }
-        }
-        phi[(size_t)(N - 1) * Cc] = Phi;
-        return;
-    }
+    double* phi = back ? nullptr : ch.phi64 + (size_t)g * N * Cc + cc;
     const SoftF64* __restrict__ soft = gd.soft;
-    int p = gd.soft_off[g];
-    const int p1 = gd.soft_off[g + 1];
-    while (p < p1 && soft[p].n == N - 1) ++p;  // no photon is too soft: nothing to add
-    int pn = p < p1 ? soft[p].n : -2;
-    double Psi = 0.0;
-    for (int n0 = N - 2; n0 >= 0; n0 -= U) {
-        double m[U], e[U], om[U], q0[U];
+    int p = 0, p1 = 0, pn = -2;
+    if (back) {
+        p = gd.soft_off[g];
+        p1 = gd.soft_off[g + 1];
+        while (p < p1 && soft[p].n == N - 1) ++p;  // no photon is too soft: nothing to add
+        pn = p < p1 ? soft[p].n : -2;
+    }
+    double sum = 0.0;
+    for (int i0 = 0; i0 < N - 1; i0 += U) {
+        double m[U], e[U];
 #pragma unroll
         for (int k = 0; k < U; ++k) {
-            const int n = max(n0 - k, 0);
-            om[k] = ua[(size_t)n * Cc] * Cact[n];
-            q0[k] = su[(size_t)n * Cc] + sC[n] + 1.0;
+            const int i = min(i0 + k, N - 2), n = back ? N - 2 - i : i;
+            const double v = ua[(size_t)n * Cc] * cf[n], q = su[(size_t)n * Cc] + sC[n] + (back ? 1.0 : 2.0);
             const double dl = gd.dln[n];
-            m[k] = om[k] > 0.0 ? om[k] * gd.lam[n] * dl : 0.0;
-            e[k] = om[k] > 0.0 ? e1d(q0[k] * dl) : 0.0;
+            m[k] = v > 0.0 ? v * dl : 0.0;
+            e[k] = v > 0.0 ? e1_of(q * dl) : 0.0;
         }
 #pragma unroll
         for (int k = 0; k < U; ++k) {
-            const int n = n0 - k;
-            if (n < 0) break;
+            const int i = i0 + k, n = back ? N - 2 - i : i;
+            if (i >= N - 1) break;
+            if (!back) phi[(size_t)n * Cc] = sum;
             while (pn == n) {
-                const SoftF64 sf = soft[p];
-                double part = 0.0;
-                if (om[k] > 0.0) {
-                    const double L = gd.dln[n] - sf.t;
-                    part = om[k] * gd.lam[n] * exp(q0[k] * sf.t) * L * e1d(q0[k] * L);
-                }
-                ch.Bb64[bb + (size_t)sf.e_diag * 32] = kC * (part + Psi) * gd.invdE[off + sf.j];
+                ch.Bb64[bb + (size_t)soft[p].e_diag * 32] = sum;
                 ++p;
                 pn = p < p1 ? soft[p].n : -2;
             }
-            Psi = fma(m[k], e[k], Psi);
+            sum = fma(m[k], e[k], sum);
         }
     }
-    for (; p < p1; ++p) ch.Bb64[bb + (size_t)soft[p].e_diag * 32] = kC * Psi * gd.invdE[off + soft[p].j];
-    if (ch.pabs) ch.pabs[(size_t)cc * gd.G + g] = kC * Psi;
+    if (!back) {
+        phi[(size_t)(N - 1) * Cc] = sum;
+        return;
+    }
+    for (; p < p1; ++p)  // no photon on the grid reaches the next bin: all absorbed power counts
+        ch.Bb64[bb + (size_t)soft[p].e_diag * 32] = soft_end(sum, gd.invdE[off + soft[p].j]);
+    if (ch.pabs) ch.pabs[(size_t)cc * gd.G + g] = kC * sum;
 }
 
 // FP32 walks: a warp takes two grains, one direction, one group of cells.  The two grains share the
@@ -477,14 +478,16 @@ __global__ void __launch_bounds__(128) k_prefix32(GrainDev gd, ChunkDev ch) {
 // One piece of a grain's pattern entries for up to 8 warps' cells.  The piece's entries and segment
 // records are staged in shared memory, where all warps read them as broadcasts; what a warp loads
 // from memory is its cells' prefix and field values, a segment ahead.
-// FP64: a warp per group of 32 cells, lane = cell.
+// FP64: a warp per group of 32 cells, lane = cell.  Bound by the integer pipes and issue (61 % of the slots, 63
+// instructions an element; the FP64 unit does two of them); 512 cells x 64 grains x 1024 wavelengths, walks
+// included: 18.5 ms with the series in FP64 and one walk per task, 3.8 ms (walks 1.3, elements 2.5).
 __global__ void __launch_bounds__(256) k_elem64(GrainDev gd, ChunkDev ch, int gblocks) {
-    __shared__ __align__(16) PatF64 pat[kPieceEntries];
+    __shared__ __align__(8) PatF64 pat[kPieceEntries];
     __shared__ __align__(16) int4 seg[kPieceEntries];
     const int piece = blockIdx.x / gblocks;
     const int4 pc = gd.pieces[2 * piece], ps = gd.pieces[2 * piece + 1];
     const int N = gd.N, Cc = ch.Cc, g = pc.x, ne = pc.z - pc.y, ns = ps.y - ps.x;
-    for (int i = threadIdx.x; i < ne; i += blockDim.x) ((int4*)pat)[i] = __ldg((const int4*)(gd.pat64 + pc.y) + i);
+    for (int i = threadIdx.x; i < 3 * ne; i += blockDim.x) ((int2*)pat)[i] = __ldg((const int2*)(gd.pat64 + pc.y) + i);
     for (int i = threadIdx.x; i < ns; i += blockDim.x) seg[i] = __ldg(gd.pseg + ps.x + i);
     __syncthreads();
     const int grp = (blockIdx.x % gblocks) * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -492,28 +495,24 @@ __global__ void __launch_bounds__(256) k_elem64(GrainDev gd, ChunkDev ch, int gb
     const int cc = grp * 32 + lane;
     int k = 0;
     const double* __restrict__ phi = ch.phi64 + (size_t)g * N * Cc + cc;
+    const double* __restrict__ uap = ch.ua64 + cc;
+    const double* __restrict__ sup = ch.su64 + cc;
     double* Bb = ch.Bb64 + (size_t)grp * gd.band_total * 32 + lane;
     for (int s = 0; s < ns; ++s) {
         const int4 r = seg[s];
         const int n = r.x;
         const double Phi = phi[(size_t)n * Cc];
         if (n == N - 1) {  // at or beyond the last node: the whole grid's prefix
-            for (; k < r.z; ++k) Bb[(size_t)pat[k].e * 32] = Phi;
+            for (; k < r.z; ++k) __stcs(Bb + (size_t)pat[k].e * 32, Phi);
             break;
         }
-        const double om = ch.ua64[(size_t)n * Cc + cc] * gd.Cact[(size_t)g * N + n];
-        const double q1 = ch.su64[(size_t)n * Cc + cc] + gd.sC[(size_t)g * N + n] + 2.0;
-        const double ln = gd.lam[n], a = om * ln * ln / kH;
-        const int cls = series_class64(q1, gd.dln[n]);
-        const double aq = (q1 != 0.0) ? a / q1 : a;
-        auto elem = [&](double t) {
-            if (cls) return Phi + (a * t) * e1d_by_class(cls, q1 * t);
-            return Phi + (q1 != 0.0 ? aq * expm1(q1 * t) : aq * t);
-        };
-        for (; k < r.y; ++k) Bb[(size_t)pat[k].e * 32] = elem(pat[k].t);
-        for (; k < r.z; ++k) {
+        const double ua = uap[(size_t)n * Cc], su = sup[(size_t)n * Cc];
+        const SegF64 sg(gd, g, n, ua, su);
+        for (; k < r.y; ++k) __stcs(Bb + (size_t)pat[k].e * 32, sg.element(Phi, pat[k].t, pat[k].tau));
+        for (; k < r.z; ++k) {  // diagonal elements: plus the intra-bin term, from the Psi in their place
             double* q = Bb + (size_t)pat[k].e * 32;
-            *q = elem(pat[k].t) + *q;
+            const double v = soft_term(gd, g, n, ua, su, pat[k].t, pat[k].tau, *q, gd.invdE[pat[k].j]);
+            __stcs(q, __dadd_rn(sg.element(Phi, pat[k].t, pat[k].tau), v));
         }
     }
 }
@@ -604,22 +603,6 @@ __global__ void __launch_bounds__(256) k_elem32(GrainDev gd, ChunkDev ch, int gb
 // k_build with the same expressions; the cumulative sums run in the same order (one thread),
 // so B is bit-identical.
 
-// Per-segment pieces of the build, shared in form with k_build (same operations, same order).
-struct SegF64 {
-    double om, q1, q0, dl, a;
-};
-__device__ __forceinline__ SegF64 seg64(const GrainDev& gd, int g, int n, double ua, double su) {
-    SegF64 r;
-    r.om = ua * gd.Cact[(size_t)g * gd.N + n];
-    const double sc = gd.sC[(size_t)g * gd.N + n];
-    r.q1 = su + sc + 2.0;
-    r.q0 = su + sc + 1.0;
-    const double ln = gd.lam[n];
-    r.a = r.om * ln * ln / kH;
-    r.dl = gd.dln[n];
-    return r;
-}
-
 // Blocks per (cell, grain): S parts (256 threads each, dynamic shared memory 2 N doubles).
 // Every part forms the segment increments and the cumulative sums; part q writes the
 // elements of the segments n = q (mod S), and the intra-bin terms whose diagonal element it
@@ -647,12 +630,11 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
     for (int n = tid; n < N - 1; n += blockDim.x) {
         double dphi = 0.0, dpsi = 0.0;
         if (BUILD == 0) {
-            const SegF64 s = seg64(gd, g, n, ch.ua64[(size_t)n * Cc + cell], ch.su64[(size_t)n * Cc + cell]);
-            if (s.om > 0.0) {
-                const int cls = series_class64(s.q1, s.dl);
-                dphi = s.a * s.dl * (cls ? e1d_by_class(cls, s.q1 * s.dl) : e1d(s.q1 * s.dl));
-                dpsi = s.om * gd.lam[n] * s.dl * e1d(s.q0 * s.dl);
-            }
+            const double ua = ch.ua64[(size_t)n * Cc + cell], su = ch.su64[(size_t)n * Cc + cell];
+            const size_t gn = (size_t)g * N + n;
+            const double dl = gd.dln[n];
+            dphi = add_segment(0.0, ua * gd.ca64[gn], su + gd.sC[gn] + 2.0, dl);
+            dpsi = add_segment(0.0, ua * gd.ce64[gn], su + gd.sC[gn] + 1.0, dl);
         } else {
             const float2 us = uasu[(size_t)n * Cc + cell];
             const float ua = us.x, su = us.y;
@@ -739,15 +721,11 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
         const int k0 = sp[n], k1 = sp[n + 1];
         if (k0 == k1) continue;
         if (BUILD == 0) {
-            const SegF64 s = seg64(gd, g, n, ch.ua64[(size_t)n * Cc + cell], ch.su64[(size_t)n * Cc + cell]);
-            const double aq = (s.q1 != 0.0) ? s.a / s.q1 : s.a;
+            const SegF64 s(gd, g, n, ch.ua64[(size_t)n * Cc + cell], ch.su64[(size_t)n * Cc + cell]);
             const double Phi = sPhi[n];
-            const int cls = series_class64(s.q1, s.dl);
             for (int k = k0 + lane; k < k1; k += 32) {
                 const PatF64 pt = gd.pat64[k];
-                ch.Bb64[bb + (size_t)pt.e * 32] =
-                    cls ? Phi + (s.a * pt.t) * e1d_by_class(cls, s.q1 * pt.t)
-                        : Phi + (s.q1 != 0.0 ? aq * expm1(s.q1 * pt.t) : aq * pt.t);
+                ch.Bb64[bb + (size_t)pt.e * 32] = s.element(Phi, pt.t, pt.tau);
             }
         } else {
             const float2 us = uasu[(size_t)n * Cc + cell];
@@ -778,16 +756,10 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
             if (sf.n == N - 1) {
                 v = 0.0;
             } else if (sf.n >= 0) {
-                const SegF64 s = seg64(gd, g, sf.n, ch.ua64[(size_t)sf.n * Cc + cell],
-                                       ch.su64[(size_t)sf.n * Cc + cell]);
-                double part = 0.0;
-                if (s.om > 0.0) {
-                    const double L = s.dl - sf.t;
-                    part = s.om * gd.lam[sf.n] * exp(s.q0 * sf.t) * L * e1d(s.q0 * L);
-                }
-                v = kC * (part + sPsi[sf.n]) * gd.invdE[off + sf.j];
+                v = soft_term(gd, g, sf.n, ch.ua64[(size_t)sf.n * Cc + cell], ch.su64[(size_t)sf.n * Cc + cell], sf.t, sf.tau,
+                              sPsi[sf.n], gd.invdE[off + sf.j]);
             } else {
-                v = kC * sPsiTot * gd.invdE[off + sf.j];
+                v = soft_end(sPsiTot, gd.invdE[off + sf.j]);
             }
             const size_t ix = bb + (size_t)sf.e_diag * 32;
             ch.Bb64[ix] = (sf.diag_in_band ? ch.Bb64[ix] : 0.0) + v;
@@ -825,16 +797,16 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
 // suffix recurrence.  Every band element is written (elements the rule leaves at zero
 // carry the column's sum).  Also the absorbed power c int Omega on the grid, summed in
 // k_build's order, for the energy check.
-__device__ __forceinline__ double point_column(const GrainDev& gd, const ChunkDev& ch, int g, int cell, int j,
-                                               double* Bb) {
+__device__ __forceinline__ void point_column(const GrainDev& gd, const ChunkDev& ch, int g, int cell, int j,
+                                             double* Bb) {
     const int N = gd.N, Cc = ch.Cc;
     const double* Cact = gd.Cact + (size_t)g * N;
     const double* sC = gd.sC + (size_t)g * N;
     const int off = gd.bin_off[g];
     const int k1 = gd.pcol[off + j + 1];
     double acc = 0.0, om = 0.0, s = 0.0;
-    bool ser = false;
-    int ncur = -1;
+    int64_t Z = 0;
+    int cls = 1, ncur = -1;
     for (int k = gd.pcol[off + j]; k < k1; ++k) {
         const PointEnt pe = gd.pent[k];
         if (pe.n >= 0) {
@@ -842,43 +814,54 @@ __device__ __forceinline__ double point_column(const GrainDev& gd, const ChunkDe
                 ncur = pe.n;
                 om = ch.ua64[(size_t)pe.n * Cc + cell] * Cact[pe.n];
                 s = ch.su64[(size_t)pe.n * Cc + cell] + sC[pe.n];
-                ser = short_series64(s, gd.dln[pe.n]);
+                const double z = s * gd.dln[pe.n];
+                cls = e1_class(z);
+                Z = cls ? to_q60(z) : 0;
             }
-            const double z = s * pe.t;  // e^z = 1 + z E1(z)
-            acc += om * (ser ? fma(z, e1d_series(z), 1.0) : exp(z)) * pe.fac;
+            double e;  // e^{s t} = 1 + z E1(z), in fixed point where |s| dln < 1
+            if (cls) {
+                const int64_t z = mul_q60(Z, pe.tau);
+                e = from_q60(kQ60 + mul_q60(z, e1_q60(cls, z)));
+            } else {
+                e = exp(s * pe.t);
+            }
+            acc = fma(om * pe.fac, e, acc);
         }
-        Bb[(size_t)pe.e * 32] = acc;
+        __stcs(Bb + (size_t)pe.e * 32, acc);
     }
-    return acc;
 }
 
+// c int Omega over the grid, in the order and arithmetic of the integral form's walk
 __device__ __forceinline__ double absorbed_power(const GrainDev& gd, const ChunkDev& ch, int g, int cell) {
     const int N = gd.N, Cc = ch.Cc;
-    const double* Cact = gd.Cact + (size_t)g * N;
+    const double* ce = gd.ce64 + (size_t)g * N;
     const double* sC = gd.sC + (size_t)g * N;
     double Psi = 0.0;
-    for (int n = N - 2; n >= 0; --n) {
-        const double om = ch.ua64[(size_t)n * Cc + cell] * Cact[n];
-        const double q0 = ch.su64[(size_t)n * Cc + cell] + sC[n] + 1.0;
-        const double b = om * gd.lam[n];
-        const double dl = gd.dln[n];
-        if (om > 0.0) Psi += b * dl * e1d(q0 * dl);
-    }
+    for (int n = N - 2; n >= 0; --n)
+        Psi = add_segment(Psi, ch.ua64[(size_t)n * Cc + cell] * ce[n], ch.su64[(size_t)n * Cc + cell] + sC[n] + 1.0,
+                          gd.dln[n]);
     return kC * Psi;
 }
 
-// Lane per cell, warp per task (grain x 32 cells), columns in turn.
+// Lane per cell, a warp per run of columns of about kPointEntries entries (any number of warps, all alike: with a
+// warp per (grain, 32 cells) 203 cells of 19 grains were 133 warps on 608 sub-partitions), then a warp per
+// (grain, 32 cells) for the absorbed power.  203 cells x 19 grains x 500
+// wavelengths: 17.6 ms with a warp per task and FP64 exponentials, 0.64 ms.
 __global__ void __launch_bounds__(128) k_build_point(GrainDev gd, ChunkDev ch) {
-    const int task = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    long long w = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    if (task >= ch.n_tasks) return;
-    const int2 tk = (ch.btasks ? ch.btasks : ch.tasks)[task];
-    const int g = tk.x, grp = tk.y;
-    const int cell = grp * 32 + lane;
-    const int M = gd.bin_off[g + 1] - gd.bin_off[g] - 1;
+    const long long power = ch.pabs ? (long long)gd.G * ch.NG : 0;
+    if (w < power) {  // the longest chains first
+        const int g = (int)(w / ch.NG), cell = (int)(w % ch.NG) * 32 + lane;
+        ch.pabs[(size_t)cell * gd.G + g] = absorbed_power(gd, ch, g, cell);
+        return;
+    }
+    w -= power;
+    if (w >= (long long)gd.n_cpieces * ch.NG) return;
+    const int4 pc = gd.cpieces[w / ch.NG];
+    const int grp = (int)(w % ch.NG), cell = grp * 32 + lane;
     double* Bb = ch.Bb64 + (size_t)grp * gd.band_total * 32 + lane;
-    for (int j = 0; j < M; ++j) point_column(gd, ch, g, cell, j, Bb);
-    if (ch.pabs) ch.pabs[(size_t)cell * gd.G + g] = absorbed_power(gd, ch, g, cell);
+    for (int j = pc.y; j < pc.z; ++j) point_column(gd, ch, pc.x, cell, j, Bb);
 }
 
 // Few cells: block per (cell, grain), threads over the columns (each column's sum is the
@@ -920,7 +903,8 @@ cudaError_t launch_build(const GrainDev& g, const ChunkDev& ch, int build, cudaS
             const unsigned blocks = (unsigned)(ch.cells * g.G);
             if (blocks) k_build_point_small<<<blocks, 128, 0, st>>>(g, ch);
         } else {
-            k_build_point<<<(ch.n_tasks + 3) / 4, 128, 0, st>>>(g, ch);
+            const long long warps = (long long)ch.NG * (g.n_cpieces + (ch.pabs ? g.G : 0));
+            k_build_point<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(g, ch);
         }
         return cudaGetLastError();
     }

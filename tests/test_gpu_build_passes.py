@@ -13,7 +13,7 @@ from tests.gpu_helpers import Lib
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("build", [heat.HEAT_BUILD_F32])
+@pytest.mark.parametrize("build", [heat.HEAT_BUILD_F32, heat.HEAT_BUILD_F64])
 @pytest.mark.parametrize("cells,grains,n_lambda", [(17, 1, 2), (33, 3, 3), (64, 2, 40), (97, 5, 257), (545, 1, 1100)])
 def test_two_passes_equal_one_walk(build, cells, grains, n_lambda):
     import torch
