@@ -27,10 +27,13 @@ cudaError_t launch_gemm_bf16(const GemmTcParams& p, int sms, cudaStream_t st);
 cudaError_t launch_to_bf16(long long n, int rows, int cols, const float* w, __nv_bfloat16* Wb, __nv_bfloat16* WTb,
                            cudaStream_t st);
 cudaError_t launch_count_valid(long long n, const float* T, unsigned long long* count, cudaStream_t st);
-cudaError_t launch_gelu_fwd(long long n, const float* Z, __nv_bfloat16* X, cudaStream_t st);
-cudaError_t launch_gelu_bwd(long long n, const float* dX, const float* Z, __nv_bfloat16* dZ, cudaStream_t st);
-cudaError_t launch_transpose_bf16(int rows, int cols, const __nv_bfloat16* in, __nv_bfloat16* out, cudaStream_t st);
-cudaError_t launch_colsum_bf16(int rows, int cols, const __nv_bfloat16* A, float* out, cudaStream_t st);
+// out [cols][rows] = G^T and (part given) part[rows/64][cols] = column sums of its 64-row tiles; with dX and Z,
+// G = dX GELU'(Z) is made and stored first.  rows, cols multiples of 64.
+cudaError_t launch_grad_tile(int rows, int cols, const float* dX, const float* Z, __nv_bfloat16* G, __nv_bfloat16* out,
+                             float* part, cudaStream_t st);
+// out[i] = sum_p in[p * n + i], p < parts
+cudaError_t launch_sum_parts(long long n, int parts, const float* in, float* out, cudaStream_t st);
+cudaError_t launch_round_bf16(long long n, const float* in, __nv_bfloat16* out, cudaStream_t st);
 // Rows of N standardised outputs Y against targets T: d = Y - T where T is finite; where T is
 // NaN and tb (per-row mask level in raw units, or null) is given, d = 0.3 max(0, raw Y - tb)
 // in standardised units (ym, ys de-standardise).  dY = 2 d / count, loss_acc (or null) += sum

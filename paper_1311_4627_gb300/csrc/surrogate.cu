@@ -50,7 +50,7 @@ struct Surrogate {
     unsigned long long seed = 0;
     // work buffers for one member and a batch of B rows
     int B = 0;
-    DevBuf Xn, Tn, Z[kLayers], Act[kLayers], dYb, dXf, dZb, T1, T2, loss, ens_mean, ens_m2, tb, cnt;
+    DevBuf Xn, Tn, Z[kLayers], Act[kLayers], dYb, dXf, dZb, T1, T2, loss, ens_mean, ens_m2, tb, cnt, csum, dWp;
     // inference of all members at once: hidden activations (ping-pong) and outputs per member
     int IB = 0;
     DevBuf H[8][2], Zo[8];
@@ -60,7 +60,7 @@ void surrogate_free(Surrogate* s) {
     if (!s) return;
     DevBuf* bufs[] = {&s->params, &s->grads, &s->adam_m, &s->adam_v, &s->wb, &s->wtb, &s->xmean, &s->xstd,
                       &s->ymean, &s->ystd, &s->d_gfeat, &s->Xn, &s->Tn, &s->dYb, &s->dXf, &s->dZb, &s->T1,
-                      &s->T2, &s->loss, &s->ens_mean, &s->ens_m2, &s->tb, &s->cnt};
+                      &s->T2, &s->loss, &s->ens_mean, &s->ens_m2, &s->tb, &s->cnt, &s->csum, &s->dWp};
     for (DevBuf* b : bufs) b->release();
     for (int l = 0; l < kLayers; ++l) {
         s->Z[l].release();
@@ -405,7 +405,8 @@ using namespace heat;
 namespace {
 
 // K-major BF16 operand map: rows x k elements (k a multiple of 64), box (64, 128).
-bool encode_bf16(CUtensorMap* m, const void* base, long long rows, long long k) {
+// ld: elements from row to row (0: k); with ld > k, columns past k read as zeros.
+bool encode_bf16(CUtensorMap* m, const void* base, long long rows, long long k, long long ld = 0) {
     static PFN_cuTensorMapEncodeTiled_v12000 enc = nullptr;
     if (!enc) {
         cudaDriverEntryPointQueryResult q;
@@ -417,7 +418,7 @@ bool encode_bf16(CUtensorMap* m, const void* base, long long rows, long long k) 
         enc = (PFN_cuTensorMapEncodeTiled_v12000)f;
     }
     cuuint64_t dims[2] = {(cuuint64_t)k, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)(k * 2)};
+    cuuint64_t strides[1] = {(cuuint64_t)((ld ? ld : k) * 2)};
     cuuint32_t box[2] = {64, 128};
     cuuint32_t es[2] = {1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
@@ -457,6 +458,41 @@ heat_status gemm(heat_ctx* ctx, int M, int N, int K, const __nv_bfloat16* A, con
     return HEAT_OK;
 }
 
+// Slices of a weight gradient's sum over the batch: as many as fill the device with 128 x 128 tiles, whole k
+// blocks of 64 rows each.
+int dw_slices(const heat_ctx* ctx, int M, int N, int B) {
+    const int tiles = ((M + 127) / 128) * ((N + 127) / 128);
+    return std::max(1, std::min({kMaxGemmZ, ctx->sms / tiles, B / 64}));
+}
+
+// dW [M x N] = T1 [M x B] . T2 [N x B]^T over the batch in slices (problem z = slice) summed afterwards: 16 to 32
+// tiles of one long sum had left most of the device idle (8192 rows of 512 x 512: 44 -> 12 us, summing included 15).
+heat_status gemm_dw(heat_ctx* ctx, Surrogate* s, int M, int N, int B, const __nv_bfloat16* A, const __nv_bfloat16* Bm,
+                    float* C, cudaStream_t st) {
+    const int slices = dw_slices(ctx, M, N, B), kb = (B / 64 + slices - 1) / slices * 64;
+    GemmTcParams p;
+    std::memset(&p, 0, sizeof(p));
+    int nz = 0;
+    for (int k0 = 0; k0 < B; k0 += kb, ++nz) {
+        const int k = std::min(kb, B - k0);
+        if (!encode_bf16(&p.ta[nz], A + k0, M, k, B) || !encode_bf16(&p.tb[nz], Bm + k0, N, k, B))
+            return ctx->fail(HEAT_ECUDA, "surrogate: cuTensorMapEncodeTiled failed");
+        p.c[nz] = slices == 1 ? C : s->dWp.as<float>() + (size_t)nz * M * N;
+    }
+    p.ldc = p.ldcb = N;
+    p.M = M;
+    p.N = N;
+    p.K = kb;
+    p.nz = nz;
+    p.mtiles = (M + 127) / 128;
+    p.ntiles = (N + 127) / 128;
+    p.status = ctx->d_status.as<int>();
+    p.wait_polls = ctx->wait_polls;
+    SCK(launch_gemm_bf16(p, ctx->sms, st));
+    if (slices > 1) SCK(launch_sum_parts((long long)M * N, nz, s->dWp.as<float>(), C, st));
+    return HEAT_OK;
+}
+
 // One layer of every member in one launch (problem z = member): C[z] = A[z] W[z]^T + b[z].
 heat_status gemm_members(heat_ctx* ctx, Surrogate* s, int l, int M, const __nv_bfloat16* const* A, float* const* C,
                          __nv_bfloat16* const* Cb, int act, cudaStream_t st);
@@ -470,7 +506,9 @@ heat_status ensure_batch(heat_ctx* ctx, Surrogate* s, int B) {
               !s->dZb.ensure(bf * (size_t)B * kHidden) && !s->T1.ensure(bf * (size_t)B * wmax) &&
               !s->T2.ensure(bf * (size_t)B * std::max(kFeat, kHidden)) && !s->loss.ensure(16) &&
               !s->ens_mean.ensure(f4 * (size_t)B * s->N) && !s->ens_m2.ensure(f4 * (size_t)B * s->N) &&
-              !s->tb.ensure(sizeof(float) * (size_t)B) && !s->cnt.ensure(16);
+              !s->tb.ensure(sizeof(float) * (size_t)B) && !s->cnt.ensure(16) &&
+              !s->csum.ensure(f4 * (size_t)(B / 64 + 1) * wmax) &&
+              !s->dWp.ensure(f4 * (size_t)kMaxGemmZ * wmax * kHidden);
     for (int l = 0; l < kLayers; ++l) {
         ok = ok && !s->Z[l].ensure(f4 * (size_t)B * s->Nout[l]);
         ok = ok && !s->Act[l].ensure(bf * (size_t)B * s->Kin[l]);
@@ -531,22 +569,22 @@ heat_status forward(heat_ctx* ctx, Surrogate* s, int m, int B, cudaStream_t st) 
 // weight and bias into Gm(m).
 heat_status backward(heat_ctx* ctx, Surrogate* s, int m, int B, cudaStream_t st) {
     __nv_bfloat16* Gb = s->dYb.as<__nv_bfloat16>();  // gradient w.r.t. the layer output, [B][Nout]
+    __nv_bfloat16 *T1 = s->T1.as<__nv_bfloat16>(), *T2 = s->T2.as<__nv_bfloat16>();
+    float* cs = s->csum.as<float>();
+    SCK(launch_grad_tile(B, s->Nout[kLayers - 1], nullptr, nullptr, Gb, T1, cs, st));
     for (int l = kLayers - 1; l >= 0; --l) {
         const int K = s->Kin[l], Nn = s->Nout[l];
         // dW = G^T Act[l]: operands transposed so both are K-major over the batch
-        SCK(launch_transpose_bf16(B, Nn, Gb, s->T1.as<__nv_bfloat16>(), st));
-        SCK(launch_transpose_bf16(B, K, s->Act[l].as<__nv_bfloat16>(), s->T2.as<__nv_bfloat16>(), st));
-        heat_status h = gemm(ctx, Nn, K, B, s->T1.as<__nv_bfloat16>(), s->T2.as<__nv_bfloat16>(),
-                             Gm(s, m) + s->woff[l], nullptr, nullptr, 0, st);
+        SCK(launch_sum_parts(Nn, B / 64, cs, Gm(s, m) + s->boff[l], st));
+        SCK(launch_grad_tile(B, K, nullptr, nullptr, s->Act[l].as<__nv_bfloat16>(), T2, nullptr, st));
+        heat_status h = gemm_dw(ctx, s, Nn, K, B, T1, T2, Gm(s, m) + s->woff[l], st);
         if (h != HEAT_OK) return h;
-        SCK(launch_colsum_bf16(B, Nn, Gb, Gm(s, m) + s->boff[l], st));
         if (l == 0) break;
         // dAct = G W  (B-operand W^T, K-major over Nout); then through the GELU of layer l-1
         h = gemm(ctx, B, K, Nn, Gb, WTb(s, m, l), s->dXf.as<float>(), nullptr, nullptr, 0, st);
         if (h != HEAT_OK) return h;
-        SCK(launch_gelu_bwd((long long)B * K, s->dXf.as<float>(), s->Z[l - 1].as<float>(), s->dZb.as<__nv_bfloat16>(),
-                            st));
         Gb = s->dZb.as<__nv_bfloat16>();
+        SCK(launch_grad_tile(B, K, s->dXf.as<float>(), s->Z[l - 1].as<float>(), Gb, T1, cs, st));
     }
     return HEAT_OK;
 }
@@ -802,13 +840,11 @@ heat_status heat_surrogate_grads(heat_ctx* ctx, int member, const float* Xn, con
     cudaStream_t st = (cudaStream_t)stream;
     heat_status h = ensure_batch(ctx, s, n);
     if (h != HEAT_OK) return h;
-    // inputs given already standardised: round to BF16 into the activation buffer
-    std::vector<float> xh((size_t)n * kFeat);
-    std::vector<__nv_bfloat16> xb(xh.size());
-    SCK(cudaMemcpy(xh.data(), Xn, 4 * xh.size(), cudaMemcpyDeviceToHost));
-    for (size_t i = 0; i < xh.size(); ++i) xb[i] = __float2bfloat16_rn(xh[i]);
-    SCK(cudaMemcpy(s->Act[0].p, xb.data(), 2 * xb.size(), cudaMemcpyHostToDevice));
-    SCK(cudaMemcpy(s->Tn.p, Tn, 4 * (size_t)n * s->N, cudaMemcpyDeviceToDevice));
+    // inputs given already standardised: round to BF16 into the activation buffer (after the legacy stream's
+    // work, on which the caller may have made them)
+    if (st) SCK(cudaStreamSynchronize(nullptr));
+    SCK(launch_round_bf16((long long)n * kFeat, Xn, s->Act[0].as<__nv_bfloat16>(), st));
+    SCK(cudaMemcpyAsync(s->Tn.p, Tn, 4 * (size_t)n * s->N, cudaMemcpyDeviceToDevice, st));
     if ((h = forward(ctx, s, member, n, st)) != HEAT_OK) return h;
     SCK(cudaMemsetAsync(s->loss.p, 0, sizeof(double), st));
     if ((h = loss_grad(ctx, s, n, true, false, s->loss.as<double>(), st)) != HEAT_OK) return h;
