@@ -67,6 +67,24 @@ struct BandRaw<1> {
     static __device__ __forceinline__ double wide(T v) { return widen_pos(v); }
 };
 
+// The same with a predicate instead of a branch: 0 where `on` is false.
+__device__ __forceinline__ double band_load_if(const double* p, bool on) {
+    double v;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\tmov.f64 %0, 0d0000000000000000;\n\t"
+                 "@p ld.global.cs.f64 %0, [%1];\n\t}"
+                 : "=d"(v)
+                 : "l"(p), "r"((int)on));
+    return v;
+}
+__device__ __forceinline__ float band_load_if(const float* p, bool on) {
+    float v;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\tmov.f32 %0, 0f00000000;\n\t"
+                 "@p ld.global.cs.f32 %0, [%1];\n\t}"
+                 : "=f"(v)
+                 : "l"(p), "r"((int)on));
+    return v;
+}
+
 // x * 2^(-800 d) for x >= 0 and d >= 0 on the integer pipe (the exponent field lowered), zero
 // where the result would fall below the normal range (values under 2^-1022 of the current
 // scale, far below anything an output resolves).  The recursion's rescales and the
@@ -620,6 +638,179 @@ __global__ void __launch_bounds__(WARP ? 32 : 1024, 1) k_recur_small(GrainDev gd
     if (numeric_bad && tid == 0) atomicOr(ch.status, kStatNumeric);
 }
 
+// ---------------------------------------------------------------------------
+// The same for unpruned solves whose rows are at most 32 x 31 wide, in row blocks: warp w holds rows 32 b ..
+// 32 b + 31 (lane = row), b = w (mod W).  Columns go in runs of eight.  The warp whose rows are due (the chain)
+// finishes its eight rows one by one with shuffles only: X_f = S_f / T, spread to the warp, one FMA into the rows
+// below; meanwhile every other warp adds the eight columns before to its rows.  So the path from one X to the
+// next is a multiply, a shuffle and an FMA, about 170 cycles, and a block barrier comes once per eight columns,
+// where k_recur_small pays a barrier, a trip through shared memory and the FP64 unit's other rows per column
+// (about 800 cycles).  W = row blocks a band can span, so a warp's next rows never need a column that went by
+// before it took them up.  Elements are loaded a run ahead; nothing is staged.
+// Each row is summed in ascending column order with one accumulator, as in k_recur: the same bits.
+// Rescales: the chain scales its own rows and the run's X, the rest follows at the run's end.
+template <int BUILD, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS > 256 ? 1 : 2) k_recur_chain(GrainDev gd, ChunkDev ch) {
+    using Raw = BandRaw<BUILD>;
+    extern __shared__ double xs[];  // X history [max_bins]
+    __shared__ double total_s;
+    __shared__ int event_s;  // rescales in the current run
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x, W = T >> 5;
+    const int cell = blockIdx.x / gd.G, g = blockIdx.x % gd.G;
+    const int grp = cell >> 5, lc = cell & 31;
+    const int off = gd.bin_off[g];
+    const int M = gd.bin_off[g + 1] - off - 1;
+    const int* rp = gd.rowptr + off + g;
+    const double* ic_row = gd.invC + off;
+    const size_t bb = (size_t)grp * gd.band_total * 32 + lc;
+    const float* B32 = ch.Bb32 + (BUILD ? bb : 0);
+    const double* B64 = ch.Bb64 + (BUILD ? 0 : bb);
+    // a row: number, band start, element of column j at rs + j, 1 / T; row 0 gives X = 1 of itself, rows past M
+    // hold nothing and give 0
+    struct Row {
+        int f, jl, rs;
+        double ic;
+    };
+    auto open_row = [&](int rb) {
+        Row r;
+        r.f = 32 * rb + lane;
+        const bool on = r.f >= 1 && r.f <= M;
+        const int p0 = on ? rp[r.f] : 0, p1 = on ? rp[r.f + 1] : 0;
+        r.jl = on ? r.f - (p1 - p0) : 1 << 30;
+        r.rs = p0 - r.jl;
+        r.ic = on ? ic_row[r.f] : (r.f == 0 ? 1.0 : 0.0);
+        return r;
+    };
+    int rb = warp;
+    Row row = open_row(rb), nxt = open_row(rb + W);
+    double acc = row.f == 0 ? 1.0 : 0.0;
+    typename Raw::T a[8], c[8];  // elements of the run before (to add), of the run itself (the chain)
+    const typename Raw::T* B = BUILD ? (const typename Raw::T*)B32 : (const typename Raw::T*)B64;
+    auto load = [&](const Row& r, int j) { return band_load_if(B + (ptrdiff_t)(r.rs + j) * 32, j >= r.jl && j < r.f); };
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        a[k] = 0;
+        c[k] = warp == 0 ? load(row, k) : 0;
+    }
+    if (tid == 0) total_s = 0.0, event_s = 0;
+    __syncthreads();
+    bool numeric_bad = false;
+    const int runs = M / 8 + 1;
+    for (int s = 0; s < runs; ++s) {
+        const bool chain = (s >> 2) == rb, last_run = chain && (s & 3) == 3;
+        if (s > 0 && !(((s - 1) >> 2) == rb)) {  // add the run before (its X are final)
+            const int j0 = 8 * (s - 1);
+            double ad[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) ad[k] = Raw::wide(a[k]);
+            if (!chain) {  // the next run's elements, a run ahead of their use
+                const bool next_chain = ((s + 1) >> 2) == rb;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    a[k] = load(row, 8 * s + k);
+                    if (next_chain) c[k] = load(row, 8 * (s + 1) + k);
+                }
+            }
+            // (the columns between the run's first and last of any row of the warp: no FMA for the others)
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (j0 + k >= row.jl && j0 + k < row.f) acc = fma(ad[k], xs[j0 + k], acc);
+        } else if (!chain) {
+            const bool next_chain = ((s + 1) >> 2) == rb;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                a[k] = load(row, 8 * s + k);
+                if (next_chain) c[k] = load(row, 8 * (s + 1) + k);
+            }
+        }
+        // the running sum, in ascending order, by a warp beside the chain's
+        if (s > 0 && lane == 0 && warp == ((s >> 2) + 1) % W) {
+            double t = total_s;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) t += xs[8 * (s - 1) + k];
+            total_s = t;
+        }
+        if (chain) {
+            double cd[8], x[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) cd[k] = Raw::wide(c[k]);
+            const Row& rn = last_run ? nxt : row;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {  // the next run's elements: the chain's own, or to add to the next rows
+                const typename Raw::T e = load(rn, last_run ? 8 * s + k : 8 * (s + 1) + k);
+                a[k] = e;
+                c[k] = e;
+            }
+            int ev = 0;
+            const bool icz = __double2hiint(row.ic) == 0 && __double2loint(row.ic) == 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int f = 8 * s + k;
+                // (an FP64 instruction takes its 64 cycles whatever lanes are active, so none is predicated)
+                const double X = __shfl_sync(0xffffffffu, acc * row.ic, f & 31);  // 0 for a zero cooling rate
+                if (icz && row.f == f && f <= M && __double_as_longlong(acc) != 0)
+                    numeric_bad = true;  // zero cooling rate with inflow (acc >= 0)
+                acc = fma(cd[k], X, acc);  // (elements outside a row's band are 0)
+                x[k] = X;
+                if (above_rescale(X)) {
+                    ++ev;
+                    acc = scale_down_800(acc, 1);
+#pragma unroll
+                    for (int i = 0; i <= k; ++i) x[i] = scale_down_800(x[i], 1);
+                }
+            }
+            double mine = 0.0;  // lane k stores the run's k-th X
+#pragma unroll
+            for (int k = 0; k < 8; ++k) mine = lane == k ? x[k] : mine;
+            if (lane < 8 && 8 * s + lane <= M) xs[8 * s + lane] = mine;
+            if (lane == 0) event_s = ev;
+        }
+        __syncthreads();
+        const int ev = event_s;
+        if (ev) {  // the rest of the block follows the chain's rescales
+            if (!chain) acc = scale_down_800(acc, ev);
+            for (int i = tid; i < 8 * s; i += T) xs[i] = scale_down_800(xs[i], ev);
+            if (tid == 0) total_s = scale_down_800(total_s, ev);
+            __syncthreads();
+        }
+        if (last_run) {
+            rb += W;
+            row = nxt;
+            nxt = open_row(rb + W);
+            acc = 0.0;
+            if (W == 1 || ((s + 1) >> 2) == rb)
+#pragma unroll
+                for (int k = 0; k < 8; ++k) c[k] = load(row, 8 * (s + 1) + k);
+        }
+    }
+    if (tid == 0)
+        for (int i = 8 * (runs - 1); i <= M; ++i) total_s += xs[i];
+    __syncthreads();
+    const double inv = 1.0 / total_s;
+    double* prow = ch.P + (size_t)cell * ch.ldP + off;
+    double emit = 0.0;
+    for (int i = tid; i <= M; i += T) {
+        const double p = xs[i] * inv;
+        prow[i] = p;
+        emit = fma(p, gd.cde[off + i], emit);
+    }
+    if (ch.ledger) {
+        for (int o = 16; o > 0; o >>= 1) emit += __shfl_xor_sync(0xffffffffu, emit, o);
+        __shared__ double wsum[32];
+        if (lane == 0) wsum[warp] = emit;
+        __syncthreads();
+        if (tid == 0) {
+            double t = 0.0;
+            for (int w = 0; w < W; ++w) t += wsum[w];
+            double* lg = ch.ledger + ((size_t)cell * gd.G + g) * 2;
+            lg[0] = ch.pabs[(size_t)cell * gd.G + g];
+            lg[1] = t;
+        }
+    }
+    numeric_bad = __syncthreads_or(numeric_bad);
+    if (numeric_bad && tid == 0) atomicOr(ch.status, kStatNumeric);
+}
+
 // Blocks of 128 threads (a warp per task) for the task-list kernels: one per 4 tasks, or, for
 // the persistent launches (ch.work set), no more than stay resident on the device at once.
 template <typename K>
@@ -640,6 +831,14 @@ cudaError_t launch_recur(const GrainDev& g, const ChunkDev& ch, int build, cudaS
     if (ch.small) {
         const long long spectra = (long long)ch.cells * g.G;
         if (spectra == 0) return cudaSuccess;
+        const int W = (g.wmax_all + 31) / 32 + 1;  // row blocks of 32 that a band can span
+        if (!ch.prune && W <= 32) {
+            const size_t smem = sizeof(double) * (size_t)g.max_bins;  // at most 32 KB (4096 bins)
+            auto kern = build == 0 ? (W <= 8 ? k_recur_chain<0, 256> : k_recur_chain<0, 1024>)
+                                   : (W <= 8 ? k_recur_chain<1, 256> : k_recur_chain<1, 1024>);
+            kern<<<(unsigned)spectra, 32 * W, smem, st>>>(g, ch);
+            return cudaGetLastError();
+        }
         // a multiple of 32 threads above the widest band row (one row in progress per thread;
         // one warp needs no block barrier per column), at most 1024 (then up to four rows per
         // thread).  Measured on the single cell (rows up to 127 wide): one warp with four rows
