@@ -414,6 +414,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
     rowptr.reserve(nbt + G);
     std::vector<PatF64> pat64;
     std::vector<PatF32> pat32;
+    std::vector<int> pat_seg;
     std::vector<int> seg_ptr((size_t)G * (N + 1), 0);
     std::vector<int4> pieces, pseg, cpieces;
     std::vector<SoftF64> soft;
@@ -563,6 +564,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
             b.cat = (float)(ca * en.t);
             b.zt = (float)(s2 * en.t);
             pat64.push_back(a);
+            pat_seg.push_back(en.n);
             pat32.push_back(b);
             RowEnt32& re = rent[(size_t)en.e];  // the same element in row order
             re.n = en.n;
@@ -651,6 +653,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
         upload(ctx->d_sC, sC) || upload(ctx->d_ca32, ca32) || upload(ctx->d_ce32, ce32) ||
         upload(ctx->d_sC32, sC32) || upload(ctx->d_rowptr, rowptr) || upload(ctx->d_wmax, wmax) || upload(ctx->d_pat64, pat64) ||
         upload(ctx->d_pat32, pat32) || upload(ctx->d_seg_ptr, seg_ptr) || upload(ctx->d_seg32, seg32) ||
+        upload(ctx->d_pat_seg, pat_seg) ||
         upload(ctx->d_ca64, ca64) || upload(ctx->d_ce64, ce64) || upload(ctx->d_cpieces, cpieces) ||
         upload(ctx->d_soft32, soft32) ||
         upload(ctx->d_pieces, pieces) || upload(ctx->d_pseg, pseg) || upload(ctx->d_soft, soft) || upload(ctx->d_soft_off, soft_off) ||
@@ -994,6 +997,7 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
     gd.pieces = ctx->d_pieces.as<int4>();
     gd.pseg = ctx->d_pseg.as<int4>();
     gd.n_pieces = ctx->n_pieces;
+    gd.pat_seg = ctx->d_pat_seg.as<int>();
     gd.pat64 = ctx->d_pat64.as<PatF64>();
     gd.pat32 = ctx->d_pat32.as<PatF32>();
     gd.soft = ctx->d_soft.as<SoftF64>();
@@ -1460,7 +1464,7 @@ void heat_destroy(heat_ctx* ctx) {
     DevBuf* bufs[] = {&ctx->d_lam, &ctx->d_dln, &ctx->d_lam32, &ctx->d_dln32, &ctx->d_bin_off, &ctx->d_cabs,
                       &ctx->d_T, &ctx->d_E, &ctx->d_Cf, &ctx->d_invC, &ctx->d_invdE, &ctx->d_invdE32, &ctx->d_Cact,
                       &ctx->d_sC, &ctx->d_ca32, &ctx->d_ce32, &ctx->d_sC32, &ctx->d_rowptr, &ctx->d_wmax, &ctx->d_seg_ptr,
-                      &ctx->d_seg32, &ctx->d_soft32, &ctx->d_ca64, &ctx->d_ce64, &ctx->d_cpieces, &ctx->d_pieces, &ctx->d_pseg, &ctx->d_pat64, &ctx->d_pat32, &ctx->d_soft, &ctx->d_soft_off, &ctx->d_K, &ctx->d_Kw, &ctx->d_w,
+                      &ctx->d_seg32, &ctx->d_soft32, &ctx->d_pat_seg, &ctx->d_ca64, &ctx->d_ce64, &ctx->d_cpieces, &ctx->d_pieces, &ctx->d_pseg, &ctx->d_pat64, &ctx->d_pat32, &ctx->d_soft, &ctx->d_soft_off, &ctx->d_K, &ctx->d_Kw, &ctx->d_w,
                       &ctx->d_koff_all, &ctx->d_cde, &ctx->d_pent, &ctx->d_pcol, &ctx->d_kexp, &ctx->d_rent, &ctx->d_gl, &ctx->d_Dtd, &ctx->d_Dtd_off, &ctx->d_Dtd_woff, &ctx->d_Dtd_order, &ctx->d_u_own, &ctx->s_tasks, &ctx->s_tasks_tail, &ctx->d_status};
     for (DevBuf* b : bufs) b->release();
     for (auto& sl : ctx->slots) {
@@ -1530,6 +1534,7 @@ __attribute__((visibility("hidden"))) heat_status heat_internal_grain_view(heat_
     gd->band_max = ctx->band_max;
     gd->wmax_all = ctx->wmax_all;
     gd->seg_ptr = ctx->d_seg_ptr.as<int>();
+    gd->pat_seg = ctx->d_pat_seg.as<int>();
     gd->pat64 = ctx->d_pat64.as<PatF64>();
     gd->pat32 = ctx->d_pat32.as<PatF32>();
     gd->soft = ctx->d_soft.as<SoftF64>();

@@ -60,6 +60,7 @@ struct GrainDev {
     const int4* pseg;       // segment records: (segment, first diagonal entry, end), entries counted from the
                             //   piece's begin; a segment's diagonal elements come last in it
     int n_pieces;
+    const int* pat_seg;     // segment of each pattern entry
     const PatF64* pat64;    // pattern entries (FP64 build)
     const PatF32* pat32;    // pattern entries (FP32 build), then 64 zero entries (prefetch margin)
     const SoftF64* soft;    // [nbt - G] per grain, sorted by segment (descending)

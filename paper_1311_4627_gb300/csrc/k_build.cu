@@ -3,10 +3,11 @@
 // with the suffix sums of Eq. brecurrence), as lane-per-cell kernels (warp = grain x 32 cells)
 // and element-parallel kernels for solves of few cells.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
-#include "fix60.cuh"
 #include "internal.h"
+#include "seg64.cuh"
 
 namespace heat {
 
@@ -65,60 +66,6 @@ __global__ void k_field(int N, const double* __restrict__ dln, const TU* __restr
     }
     if (bad) atomicOr(status, kStatBadInput);
 }
-
-// ---------------------------------------------------------------------------
-// FP64 build: a segment's pieces, shared by every kernel of the exact path.  With Omega = u C, slope q - p - 1
-// and Z = q dln, the segment's integral is v dln E1(Z) and up to the fraction tau of it v t E1(Z tau); E1 in 60-bit
-// fixed point where |Z| < 1 (fix60.cuh; about 150 cycles of the integer pipes instead of 8 to 12 FP64
-// multiply-adds of 64 cycles), else the library's expm1.
-__device__ __forceinline__ double e1_of(double Z) {
-    const int cls = e1_class(Z);
-    return cls ? from_q60(e1_q60(cls, to_q60(Z))) : e1d(Z);
-}
-// Phi (Psi) after a segment: + v dln E1(Z)
-__device__ __forceinline__ double add_segment(double sum, double v, double q, double dl) {
-    return v > 0.0 ? fma(v * dl, e1_of(q * dl), sum) : sum;
-}
-struct SegF64 {
-    double a, q1, aq;  // C_n u_n lambda_n^2 / h, slope + 2; a / q1 where the library's expm1 serves
-    int64_t Z;         // q1 dln in Q60
-    int cls;
-    __device__ __forceinline__ SegF64(const GrainDev& gd, int g, int n, double ua, double su) {
-        a = ua * gd.ca64[(size_t)g * gd.N + n];
-        q1 = su + gd.sC[(size_t)g * gd.N + n] + 2.0;
-        const double z = q1 * gd.dln[n];
-        cls = e1_class(z);
-        Z = cls ? to_q60(z) : 0;
-        aq = cls ? 0.0 : a / q1;
-    }
-    // B at offset t (fraction tau) of the segment
-    __device__ __forceinline__ double element(double Phi, double t, int64_t tau) const {
-        if (cls) return fma(a * t, from_q60(e1_q60(cls, mul_q60(Z, tau))), Phi);
-        return fma(aq, expm1(q1 * t), Phi);
-    }
-};
-// The intra-bin term of a bin whose soft photons begin at offset t (fraction tau) of segment n, with Psi the
-// integral of Omega beyond the segment: c (int from t to the segment's end + Psi) / (E_{j+1} - E_j).  The part of
-// the segment is the difference of two fixed-point values, exact to 2^-58 of the whole segment's.
-__device__ __forceinline__ double soft_term(const GrainDev& gd, int g, int n, double ua, double su, double t,
-                                            int64_t tau, double Psi, double invdE) {
-    const double b = ua * gd.ce64[(size_t)g * gd.N + n], q0 = su + gd.sC[(size_t)g * gd.N + n] + 1.0;
-    const double dl = gd.dln[n], z = q0 * dl;
-    double part = 0.0;
-    if (b > 0.0) {
-        const int cls = e1_class(z);
-        if (cls) {
-            const int64_t Z = to_q60(z);
-            const int64_t d = e1_q60(cls, Z) - mul_q60(tau, e1_q60(cls, mul_q60(Z, tau)));
-            part = d > 0 ? (b * dl) * from_q60(d) : 0.0;
-        } else {
-            const double L = dl - t;
-            part = b * exp(q0 * t) * L * e1d(q0 * L);
-        }
-    }
-    return __dmul_rn(__dmul_rn(kC, __dadd_rn(part, Psi)), invdE);
-}
-__device__ __forceinline__ double soft_end(double Psi, double invdE) { return __dmul_rn(__dmul_rn(kC, Psi), invdE); }
 
 // ---------------------------------------------------------------------------
 // k_build: the matrix-build kernel.  One warp per task (grain x 32 cells), one lane
@@ -609,12 +556,18 @@ __global__ void __launch_bounds__(256) k_elem32(GrainDev gd, ChunkDev ch, int gb
 // wrote: the diagonal (j+1, j) and bin j's soft-photon edge are the same wavelength,
 // hc/(Elo_{j+1} - E_j), so both fall in segment sf.n (sf.n < 0: the diagonal is not in the
 // band, part 0).  Few spectra (a single cell) then spread over many SMs.
+// The sums are the serial part: FP32, one thread in the lane-per-cell kernel's order (its bits), on FP32 values
+// throughout (a conversion to or from FP64 takes the FP64 unit 64 cycles); FP64, a warp, a run of segments a lane
+// and a scan over the lanes.  The elements take a thread each.  Against a warp per segment and FP64 sums on one thread:
+// 5 cells x 64 grains x 1024 wavelengths (FP32) 216 -> 130 us, single cell (FP64) 28 -> 23 us.
 template <int BUILD>
 __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, int S) {
+    using Real = typename std::conditional<BUILD == 0, double, float>::type;
     extern __shared__ double sm[];
-    double* sPhi = sm;          // [N]: Phi before segment n (exclusive prefix), then Phi at the end
-    double* sPsi = sm + gd.N;   // [N]: Psi after the segments above n (exclusive suffix)
-    __shared__ double sPhiEnd, sPsiTot;
+    Real* sPhi = (Real*)sm;     // [N]: Phi before segment n (exclusive prefix)
+    Real* sPsi = sPhi + gd.N;   // [N]: Psi after the segments above n (exclusive suffix)
+    __shared__ Real sPhiEnd;
+    __shared__ double sPsiTot;
     __shared__ float sPsiEnd32;  // FP32 build: the FP32 value of the compensated total
     const int N = gd.N, Cc = ch.Cc;
     const int spec = blockIdx.x / S, part = blockIdx.x % S;
@@ -624,119 +577,99 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
     const int off = gd.bin_off[g];
     const size_t bb = (size_t)grp * gd.band_total * 32 + lc;
     const int* sp = gd.seg_ptr + (size_t)g * (N + 1);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
     const float2* uasu = (const float2*)ch.ua32;
     // 1. segment increments, in parallel
     for (int n = tid; n < N - 1; n += blockDim.x) {
-        double dphi = 0.0, dpsi = 0.0;
+        const size_t gn = (size_t)g * N + n;
+        Real dphi = 0, dpsi = 0;
         if (BUILD == 0) {
             const double ua = ch.ua64[(size_t)n * Cc + cell], su = ch.su64[(size_t)n * Cc + cell];
-            const size_t gn = (size_t)g * N + n;
             const double dl = gd.dln[n];
             dphi = add_segment(0.0, ua * gd.ca64[gn], su + gd.sC[gn] + 2.0, dl);
             dpsi = add_segment(0.0, ua * gd.ce64[gn], su + gd.sC[gn] + 1.0, dl);
         } else {
             const float2 us = uasu[(size_t)n * Cc + cell];
             const float ua = us.x, su = us.y;
-            const float sc = gd.sC32[(size_t)g * N + n], dl = gd.dln32[n];
-            const float a = ua * gd.ca32[(size_t)g * N + n];
-            if (a > 0.0f) dphi = widen_pos(a * dl * e1f((su + sc + 2.0f) * dl));
-            const float b = ua * gd.ce32[(size_t)g * N + n];
-            if (b > 0.0f) dpsi = widen_pos(b * dl * e1f((su + sc + 1.0f) * dl));
+            const float sc = gd.sC32[gn], dl = gd.dln32[n];
+            const float a = ua * gd.ca32[gn];
+            if (a > 0.0f) dphi = a * dl * e1f((su + sc + 2.0f) * dl);
+            const float b = ua * gd.ce32[gn];
+            if (b > 0.0f) dpsi = b * dl * e1f((su + sc + 1.0f) * dl);
         }
         sPhi[n] = dphi;
         sPsi[n] = dpsi;
     }
     __syncthreads();
-    // 2. the cumulative sums, in the lane-per-cell kernel's order and arithmetic (FP64 build:
-    // FP64 sums; FP32 build: compensated FP32 sums, whose FP32 values are kept)
-    // (the increments are read eight at a time ahead of the sums, so no shared-memory load
-    // latency sits on the sums' dependent chain)
-    constexpr int R = 8;
-    if (tid == 0) {
-        if (BUILD == 0) {
-            double Phi = 0.0;
-            for (int n0 = 0; n0 < N - 1; n0 += R) {
-                double d[R];
-#pragma unroll
-                for (int k = 0; k < R; ++k) d[k] = n0 + k < N - 1 ? sPhi[n0 + k] : 0.0;
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-                    if (n0 + k < N - 1) {
-                        sPhi[n0 + k] = Phi;
-                        Phi += d[k];
-                    }
+    // 2. the cumulative sums
+    if constexpr (BUILD == 0) {
+        if (tid < 64) {  // warp 0 upward over sPhi, warp 1 downward over sPsi
+            const bool down = tid >= 32;
+            Real* v = down ? sPsi : sPhi;
+            const int per = (N - 1 + 31) / 32, i0 = min(lane * per, N - 1), i1 = min(i0 + per, N - 1);
+            double run = 0.0;
+            for (int i = i0; i < i1; ++i) run += v[down ? N - 2 - i : i];
+            double incl = run;
+            for (int o = 1; o < 32; o <<= 1) {
+                const double t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
             }
-            sPhiEnd = Phi;
-        } else {
-            Sum32 Phi;
-            for (int n0 = 0; n0 < N - 1; n0 += R) {
-                float d[R];
-#pragma unroll
-                for (int k = 0; k < R; ++k) d[k] = n0 + k < N - 1 ? (float)sPhi[n0 + k] : 0.0f;
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-                    if (n0 + k < N - 1) {
-                        sPhi[n0 + k] = Phi.val();
-                        Phi.add(d[k]);
-                    }
+            double before = __shfl_up_sync(0xffffffffu, incl, 1);
+            if (lane == 0) before = 0.0;
+            for (int i = i0; i < i1; ++i) {
+                const int n = down ? N - 2 - i : i;
+                const double d = v[n];
+                v[n] = before;
+                before += d;
             }
-            sPhiEnd = Phi.val();
+            const double tot = __shfl_sync(0xffffffffu, incl, 31);
+            if (lane == 0) {
+                if (down)
+                    sPsiTot = tot;
+                else
+                    sPhiEnd = tot;
+            }
         }
-    } else if (tid == 32) {
-        if (BUILD == 0) {
-            double Psi = 0.0;
-            for (int n0 = N - 2; n0 >= 0; n0 -= R) {
-                double d[R];
+    } else if (tid == 0 || tid == 32) {
+        // the increments are read eight at a time ahead of the sums, so that no shared-memory load latency sits on
+        // the sums' dependent chain
+        constexpr int R = 8;
+        const bool down = tid == 32;
+        Real* v = down ? sPsi : sPhi;
+        Sum32 sum;
+        for (int i0 = 0; i0 < N - 1; i0 += R) {
+            float d[R];
 #pragma unroll
-                for (int k = 0; k < R; ++k) d[k] = n0 - k >= 0 ? sPsi[n0 - k] : 0.0;
+            for (int k = 0; k < R; ++k) d[k] = i0 + k < N - 1 ? (float)v[down ? N - 2 - i0 - k : i0 + k] : 0.0f;
 #pragma unroll
-                for (int k = 0; k < R; ++k)
-                    if (n0 - k >= 0) {
-                        sPsi[n0 - k] = Psi;
-                        Psi += d[k];
-                    }
-            }
-            sPsiTot = Psi;
+            for (int k = 0; k < R; ++k)
+                if (i0 + k < N - 1) {
+                    v[down ? N - 2 - i0 - k : i0 + k] = sum.val();
+                    sum.add(d[k]);
+                }
+        }
+        if (down) {
+            sPsiTot = sum.wide();
+            sPsiEnd32 = sum.val();
         } else {
-            Sum32 Psi;
-            for (int n0 = N - 2; n0 >= 0; n0 -= R) {
-                float d[R];
-#pragma unroll
-                for (int k = 0; k < R; ++k) d[k] = n0 - k >= 0 ? (float)sPsi[n0 - k] : 0.0f;
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-                    if (n0 - k >= 0) {
-                        sPsi[n0 - k] = Psi.val();
-                        Psi.add(d[k]);
-                    }
-            }
-            sPsiTot = Psi.wide();
-            sPsiEnd32 = Psi.val();
+            sPhiEnd = sum.val();
         }
     }
     __syncthreads();
-    // 3. band elements: warp per segment (this part's), lanes over its pattern entries
-    for (int n = part + S * warp; n < N - 1; n += S * (blockDim.x >> 5)) {
-        const int k0 = sp[n], k1 = sp[n + 1];
-        if (k0 == k1) continue;
+    // 3. band elements of this part's segments, a thread each
+    for (int k = sp[0] + tid; k < sp[N - 1]; k += blockDim.x) {
+        const int n = gd.pat_seg[k];
+        if (n % S != part) continue;
         if (BUILD == 0) {
             const SegF64 s(gd, g, n, ch.ua64[(size_t)n * Cc + cell], ch.su64[(size_t)n * Cc + cell]);
-            const double Phi = sPhi[n];
-            for (int k = k0 + lane; k < k1; k += 32) {
-                const PatF64 pt = gd.pat64[k];
-                ch.Bb64[bb + (size_t)pt.e * 32] = s.element(Phi, pt.t, pt.tau);
-            }
+            const PatF64 pt = gd.pat64[k];
+            ch.Bb64[bb + (size_t)pt.e * 32] = s.element(sPhi[n], pt.t, pt.tau);
         } else {
             const float2 us = uasu[(size_t)n * Cc + cell];
-            const float ua = us.x, su = us.y;
-            const float phi = __double2float_rn(sPhi[n]);
-            const bool sh = short_series(su, gd.sC32[(size_t)g * N + n], gd.dln32[n]);
-            for (int k = k0 + lane; k < k1; k += 32) {
-                const PatF32 a0 = gd.pat32[k];
-                const float z = fmaf(su, a0.t, a0.zt);
-                ch.Bb32[bb + (size_t)a0.e * 32] = fmaf(ua * a0.cat, sh ? e1f_small(z) : e1f(z), phi);
-            }
+            const bool sh = short_series(us.y, gd.sC32[(size_t)g * N + n], gd.dln32[n]);
+            const PatF32 a0 = gd.pat32[k];
+            const float z = fmaf(us.y, a0.t, a0.zt);
+            ch.Bb32[bb + (size_t)a0.e * 32] = fmaf(us.x * a0.cat, sh ? e1f_small(z) : e1f(z), (float)sPhi[n]);
         }
     }
     if ((N - 1) % S == part)
@@ -744,7 +677,7 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
             if (BUILD == 0)
                 ch.Bb64[bb + (size_t)gd.pat64[k].e * 32] = sPhiEnd;
             else
-                ch.Bb32[bb + (size_t)gd.pat32[k].e * 32] = __double2float_rn(sPhiEnd);
+                ch.Bb32[bb + (size_t)gd.pat32[k].e * 32] = (float)sPhiEnd;
         }
     __syncthreads();  // the intra-bin terms add to diagonal elements written above (by this part)
     // 4. intra-bin terms, one per soft entry (each has its own diagonal element)
@@ -778,7 +711,7 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
                     const float L = dl - ts;
                     part = b * __expf(q0 * ts) * L * e1f(q0 * L);
                 }
-                v = (part + __double2float_rn(sPsi[sf.n])) * gd.invdE32[off + sf.j];
+                v = (part + (float)sPsi[sf.n]) * gd.invdE32[off + sf.j];
             } else {
                 v = sPsiEnd32 * gd.invdE32[off + sf.j];
             }
@@ -909,7 +842,7 @@ cudaError_t launch_build(const GrainDev& g, const ChunkDev& ch, int build, cudaS
         return cudaGetLastError();
     }
     if (ch.small) {
-        const size_t smem = sizeof(double) * 2 * (size_t)g.N;
+        const size_t smem = (build == 0 ? sizeof(double) : sizeof(float)) * 2 * (size_t)g.N;
         const long long spectra = (long long)ch.cells * g.G;
         if (spectra == 0) return cudaSuccess;
         // parts per spectrum: about two blocks per SM in all (one part when spectra suffice)
