@@ -81,6 +81,14 @@ struct SoftF64 {
     int64_t tau;  // t / ln(lambda_{n+1}/lambda_n) in Q60
 };
 
+// Place of a band element's transition wavelength on the grid, in band (row) order, for the thermal-discrete
+// rates: segment n (-1 below the grid, N - 1 at or beyond the last node), offset t, fraction tau in Q60.
+struct __align__(8) TdEdge {
+    int n;
+    double t;
+    int64_t tau;
+};
+
 // X > 2^800 for a positive finite double, tested on the exponent bits (integer pipe).
 __device__ __forceinline__ bool above_rescale(double x) {
     return __double2hiint(x) > (int)((1023 + 800) << 20) - 1;

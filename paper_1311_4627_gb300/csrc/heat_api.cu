@@ -741,6 +741,18 @@ static heat_status ensure_discrete(heat_ctx* ctx, cudaStream_t st) {
     CKR(launch_cooling_window(ctx->N, ctx->d_lam.as<double>(), ctx->d_cabs.as<double>(), ctx->d_bin_off.as<int>(), G,
                               ctx->d_T.as<double>(), ctx->d_E.as<double>(), ctx->d_Dtd_woff.as<long long>(), woff[G],
                               ctx->d_Dtd_off.as<long long>(), ctx->d_Dtd.as<double>(), gl, gl + kGLPoints, st));
+    if (ctx->d_Dtd_edge.ensure(sizeof(TdEdge) * (size_t)std::max(1LL, ctx->band_per_cell)))
+        return ctx->fail(HEAT_ENOMEM, "heat_solve: allocation of thermal-discrete rates failed");
+    GrainDev gd{};
+    gd.N = ctx->N;
+    gd.G = G;
+    gd.nbt = ctx->nbt;
+    gd.lam = ctx->d_lam.as<double>();
+    gd.dln = ctx->d_dln.as<double>();
+    gd.bin_off = ctx->d_bin_off.as<int>();
+    gd.rowptr = ctx->d_rowptr.as<int>();
+    gd.E = ctx->d_E.as<double>();
+    CKR(launch_td_edges(gd, ctx->d_Dtd_edge.as<TdEdge>(), st));
     CKR(cudaStreamSynchronize(st));
     ctx->td_built = true;
     return HEAT_OK;
@@ -815,7 +827,7 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
     const bool discrete = o.cooling == HEAT_COOLING_DISCRETE;
     if (discrete && (o.build != HEAT_BUILD_F64 || o.heating != HEAT_HEATING_INTEGRAL))
         return ctx->fail(HEAT_EINVAL, "heat_solve: thermal-discrete cooling needs the exact build and integral heating");
-    if (discrete && (ctx->max_bins > kDiscreteMaxBins || td_fill_smem_bytes(ctx->N) > kMaxSmemPerBlock))
+    if (discrete && (ctx->max_bins > kDiscreteMaxBins || ctx->N > kDiscreteMaxLambda))
         return ctx->fail(HEAT_EINVAL, "heat_solve: thermal-discrete cooling takes at most 2048 bins per grain and "
                                       "6456 wavelengths");
     const int emis_nt = o.emis_n_tile ? o.emis_n_tile : (ctx->tuned_emis_nt ? ctx->tuned_emis_nt : 256);
@@ -1072,8 +1084,8 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
             for (long long s0 = 0, nsp = (long long)ch.cells * G; s0 < nsp; s0 += td_batch) {
                 const long long n = discrete_batch_spectra(gd, ch, s0, td_batch);
                 TIMED(HEAT_T_BUILD, launch_discrete_fill(gd, ch, ctx->d_Dtd.as<double>(), ctx->d_Dtd_off.as<long long>(),
-                                                         ctx->d_Dtd_order.as<int>(), sl.tdq.as<double>(), qst, s0, n,
-                                                         cs));
+                                                         ctx->d_Dtd_order.as<int>(), ctx->d_Dtd_edge.as<TdEdge>(),
+                                                         sl.tdq.as<double>(), qst, s0, n, cs));
                 TIMED(HEAT_T_RECUR, launch_discrete_gth(gd, ch, ctx->d_Dtd_order.as<int>(), sl.tdq.as<double>(), qst, s0,
                                                         n, cs));
             }
@@ -1465,7 +1477,7 @@ void heat_destroy(heat_ctx* ctx) {
                       &ctx->d_T, &ctx->d_E, &ctx->d_Cf, &ctx->d_invC, &ctx->d_invdE, &ctx->d_invdE32, &ctx->d_Cact,
                       &ctx->d_sC, &ctx->d_ca32, &ctx->d_ce32, &ctx->d_sC32, &ctx->d_rowptr, &ctx->d_wmax, &ctx->d_seg_ptr,
                       &ctx->d_seg32, &ctx->d_soft32, &ctx->d_pat_seg, &ctx->d_ca64, &ctx->d_ce64, &ctx->d_cpieces, &ctx->d_pieces, &ctx->d_pseg, &ctx->d_pat64, &ctx->d_pat32, &ctx->d_soft, &ctx->d_soft_off, &ctx->d_K, &ctx->d_Kw, &ctx->d_w,
-                      &ctx->d_koff_all, &ctx->d_cde, &ctx->d_pent, &ctx->d_pcol, &ctx->d_kexp, &ctx->d_rent, &ctx->d_gl, &ctx->d_Dtd, &ctx->d_Dtd_off, &ctx->d_Dtd_woff, &ctx->d_Dtd_order, &ctx->d_u_own, &ctx->s_tasks, &ctx->s_tasks_tail, &ctx->d_status};
+                      &ctx->d_koff_all, &ctx->d_cde, &ctx->d_pent, &ctx->d_pcol, &ctx->d_kexp, &ctx->d_rent, &ctx->d_gl, &ctx->d_Dtd, &ctx->d_Dtd_off, &ctx->d_Dtd_woff, &ctx->d_Dtd_order, &ctx->d_Dtd_edge, &ctx->d_u_own, &ctx->s_tasks, &ctx->s_tasks_tail, &ctx->d_status};
     for (DevBuf* b : bufs) b->release();
     for (auto& sl : ctx->slots) {
         DevBuf* sb[] = {&sl.ua64, &sl.su64, &sl.ua32, &sl.Bb64, &sl.Bb32, &sl.xs, &sl.ep,   &sl.pabs,

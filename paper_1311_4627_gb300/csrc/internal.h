@@ -10,6 +10,7 @@ struct PatF64;
 struct PatF32;
 struct SoftF64;
 struct RowEnt32;
+struct TdEdge;
 
 // ---- grain set-up (k_setup.cu)
 cudaError_t set_gauss_legendre(const double* x, const double* w);
@@ -161,14 +162,16 @@ size_t gth_smem_bytes(int max_bins);
 size_t td_fill_smem_bytes(int N);
 // Shared memory per block of the few-cell recursion up to which the band is staged there.
 constexpr size_t kSmallRecurStage = 100 * 1024;
+constexpr int kDiscreteMaxLambda = 6456;              // the fill's tables in shared memory
 constexpr int kDiscreteMaxBins = 2048;                // the state reduction's vectors in shared memory
 constexpr size_t kMaxSmemPerBlock = 227 * 1024;       // opt-in dynamic shared memory per block
 // Spectra are solved in launches of `batch` (rate matrices at q + k * qstride): the k-th
 // spectrum from s0 is grain gorder[(s0 + k) / cells], cell (s0 + k) % cells.
 long long discrete_batch_spectra(const GrainDev& g, const ChunkDev& ch, long long s0, long long batch);
 cudaError_t launch_discrete_fill(const GrainDev& g, const ChunkDev& ch, const double* D, const long long* doff,
-                                 const int* gorder, double* q, long long qstride, long long s0, long long n,
-                                 cudaStream_t st);
+                                 const int* gorder, const TdEdge* edge, double* q, long long qstride, long long s0,
+                                 long long n, cudaStream_t st);
+cudaError_t launch_td_edges(const GrainDev& g, TdEdge* edge, cudaStream_t st);
 cudaError_t launch_discrete_gth(const GrainDev& g, const ChunkDev& ch, const int* gorder, double* q, long long qstride,
                                 long long s0, long long n, cudaStream_t st);
 

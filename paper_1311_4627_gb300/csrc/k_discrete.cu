@@ -23,6 +23,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "seg64.cuh"
 
 namespace heat {
 
@@ -203,37 +204,50 @@ __global__ void k_cooling_window(int N, const double* __restrict__ lam, const do
     if (lane == 0) D[doff[g] + (size_t)u * nb + l] = 4.0 * kPi * acc / (Eg[u] - Eg[l]);
 }
 
-namespace {
-
-// Integral over [x, y] of Omega lambda^p in segment n of the cell's interpolant:
-// Omega_n lambda_n^(p+1) e^(q tx) (ty - tx) E1(q (ty - tx)), q = s_n + p + 1.
-__device__ __forceinline__ double seg_part(double om, double s, double lamn, int p, double x, double y) {
-    const double tx = log(x / lamn), dt = log(y / x);
-    const double q = s + p + 1.0;
-    const double lp = p == 1 ? lamn * lamn : lamn;
-    return om * lp * exp(q * tx) * dt * e1d(q * dt);
-}
-
-// Segment n (0 .. N-2) holding x in [lam_0, lam_{N-1}]: lam_n <= x < lam_{n+1} (x = lam_{N-1} in
-// the last).  Searched in FP32, then moved by at most one node with the FP64 grid.
-__device__ __forceinline__ int seg_of(const float* l32, const double* lam, int N, double x) {
-    const float xf = (float)x;
-    int lo = 0, hi = N - 2;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (l32[mid] <= xf) lo = mid; else hi = mid - 1;
+// Where the transition wavelength hc / (Elo_f - E_j) of every band element (f, j) falls on the grid: its segment n
+// and offset (n = -1 below the grid, N - 1 at or beyond the last node).  Once per grain set; a warp per row f.
+__global__ void __launch_bounds__(128) k_td_edges(GrainDev gd, TdEdge* __restrict__ edge) {
+    const int w = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (w >= gd.nbt) return;
+    int g = 0;
+    while (gd.bin_off[g + 1] <= w) ++g;
+    const int off = gd.bin_off[g], f = w - off, N = gd.N;
+    if (f == 0) return;
+    const int e0 = gd.rowptr[off + g + f], wd = gd.rowptr[off + g + f + 1] - e0;
+    const double* E = gd.E + off;
+    const double elo = 0.5 * (E[f - 1] + E[f]);
+    for (int k = lane; k < wd; k += 32) {
+        const double x = kHC / (elo - E[f - wd + k]);
+        TdEdge r;
+        r.n = -1;
+        r.t = 0.0;
+        r.tau = 0;
+        if (x >= gd.lam[N - 1]) {
+            r.n = N - 1;
+        } else if (x >= gd.lam[0]) {
+            int lo = 0, hi = N - 2;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (gd.lam[mid] <= x) lo = mid; else hi = mid - 1;
+            }
+            r.n = lo;
+            r.t = log(x / gd.lam[lo]);
+            r.tau = to_q60(fmin(r.t / gd.dln[lo], 1.0));
+        }
+        edge[e0 + k] = r;
     }
-    if (lo < N - 2 && lam[lo + 1] <= x) ++lo;
-    else if (lo > 0 && lam[lo] > x) --lo;
-    return lo;
 }
 
-}  // namespace
+cudaError_t launch_td_edges(const GrainDev& g, TdEdge* edge, cudaStream_t st) {
+    k_td_edges<<<(unsigned)((g.nbt + 3) / 4), 128, 0, st>>>(g, edge);
+    return cudaGetLastError();
+}
 
-// Shared memory of k_td_fill for a grid of N wavelengths: per segment the cell's Omega_n and
-// log-log slope, the segment's integral of Omega lambda, the suffix sums of the integrals of
-// Omega, and the grid in FP32.
-size_t td_fill_smem_bytes(int N) { return sizeof(double) * 4 * (size_t)N + sizeof(float) * (size_t)N; }
+// Shared memory of k_td_fill for a grid of N wavelengths, per segment: the cell's A = Omega_n lambda_n^2 dln / h,
+// Z = (slope + 2) dln in Q60 (kNoQ60: |Z| >= 1), R = E1(Z) in Q60 (kNoQ60: the bits of the whole segment's integral), and
+// the suffix sums of the integrals of Omega.
+size_t td_fill_smem_bytes(int N) { return 32 * (size_t)N; }
+constexpr int64_t kNoQ60 = INT64_MIN;
 
 // Spectrum of block b of a launch that starts at spectrum s0: grains in the order `gorder`
 // (most bins first), every cell of the chunk for each grain in turn, so that the spectra of one
@@ -252,42 +266,52 @@ __device__ __forceinline__ void td_spectrum(const ChunkDev& ch, const int* gorde
 // rate from i into bin j > i is (1/h) int Omega lambda over the photon wavelengths that end in
 // bin j, [hc/(Ehi_j - E_i), hc/(Elo_j - E_i)] (Ehi_M = infinity), plus on j = i + 1 the
 // power of the photons too soft to leave bin i, c int_{lambda > hc/(Elo_j - E_i)} Omega,
-// over E_j - E_i.  A row's windows tile the grid: each is the closed-form integral of its
-// partial end segments plus the segment integrals between them (summed, not differenced);
-// the soft term is its partial segment plus a suffix sum.  A warp per row, a lane per j;
-// neighbouring lanes share their window edge, and the row ends where the window leaves the
-// short-wavelength end of the grid.
+// over E_j - E_i.  The window's edges are the band's transition wavelengths (j + 1, i) and (j, i), whose places on
+// the grid do not depend on the cell (edge table).  A row's windows tile the grid: each is its
+// partial end segments plus the segment integrals between them (summed, not differenced; inside one segment
+// a difference of two Q60 values, exact to 2^-58 of the segment); the soft term is its partial segment plus
+// a suffix sum.  A warp per row, a lane per j; neighbouring lanes share their window edge, so a window costs one
+// fixed-point E1 (seg64.cuh).  With the edges and each partial segment's logarithms and exponentials in FP64
+// the fill was bound by the FP64 unit (83 % busy): 8 cells x 64 grains x 1024 wavelengths 8.7 ms, now 2.0 ms.
 __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const double* __restrict__ Dt,
                                                  const long long* __restrict__ doff, const int* __restrict__ gorder,
-                                                 long long s0, double* q, long long qstride, int S) {
+                                                 const TdEdge* __restrict__ edge, long long s0, double* q,
+                                                 long long qstride, int S) {
     extern __shared__ double fsm[];
     const int bsp = blockIdx.x / S, part = blockIdx.x % S;  // spectrum of the launch, part of its rows
     int cell, g;
     td_spectrum(ch, gorder, s0, cell, g, bsp);
     const int N = gd.N;
-    const double* lam = gd.lam;
-    double* om = fsm;
-    double* sl = om + N;
-    double* I1 = sl + N;
-    double* S0 = I1 + N;
-    float* l32 = (float*)(S0 + N);
+    double* A = fsm;
+    int64_t* Z = (int64_t*)(A + N);
+    int64_t* R = Z + N;
+    double* S0 = (double*)(R + N);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     for (int n = tid; n < N; n += blockDim.x) {
-        l32[n] = gd.lam32[n];
-        double o = 0.0, sv = 0.0, i0 = 0.0, i1 = 0.0;
+        double a = 0.0, i0 = 0.0;
+        int64_t z = 0, r = kQ60;
         if (n < N - 1) {
-            o = ch.ua64[(size_t)n * ch.Cc + cell] * gd.Cact[(size_t)g * N + n];
-            sv = ch.su64[(size_t)n * ch.Cc + cell] + gd.sC[(size_t)g * N + n];
-            if (o > 0.0) {
-                i0 = seg_part(o, sv, lam[n], 0, lam[n], lam[n + 1]);
-                i1 = seg_part(o, sv, lam[n], 1, lam[n], lam[n + 1]);
+            const size_t gn = (size_t)g * N + n;
+            const double ua = ch.ua64[(size_t)n * ch.Cc + cell], su = ch.su64[(size_t)n * ch.Cc + cell];
+            const double dl = gd.dln[n], q1 = su + gd.sC[gn] + 2.0, zd = q1 * dl;
+            a = ua * gd.ca64[gn] * dl;
+            if (a > 0.0) {
+                i0 = add_segment(0.0, ua * gd.ce64[gn], q1 - 1.0, dl);
+                const int cls = e1_class(zd);
+                if (cls) {
+                    z = to_q60(zd);
+                    r = e1_q60(cls, z);
+                } else {
+                    z = kNoQ60;
+                    r = __double_as_longlong(a * e1d(zd));
+                }
             } else {
-                o = 0.0;
+                a = 0.0;
             }
         }
-        om[n] = o;
-        sl[n] = sv;
-        I1[n] = i1;
+        A[n] = a;
+        Z[n] = z;
+        R[n] = r;
         S0[n] = i0;
     }
     __syncthreads();
@@ -309,45 +333,83 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
     const int off = gd.bin_off[g], nb = gd.bin_off[g + 1] - off;
     const double* E = gd.E + off;
     const double* Dg = Dt + doff[g];
+    const int* rp = gd.rowptr + off + g;
     double* qs = q + (size_t)bsp * qstride;
-    const double lam0 = lam[0], lamN = lam[N - 1];
-    const int M = nb - 1;
+    // the cell's slope + 2 of segment n (only where |Z| >= 1)
+    auto slope = [&](int n) { return ch.su64[(size_t)n * ch.Cc + cell] + gd.sC[(size_t)g * N + n] + 2.0; };
+    // tau E1(Z tau) in Q60: the fraction of A up to an edge in segment n
+    auto upto = [&](int n, int64_t tau) -> int64_t {
+        const int64_t z = Z[n];
+        if (z == kNoQ60) return 0;
+        const int64_t az = z < 0 ? -z : z;
+        return mul_q60(tau, e1_q60(az < (kQ60 >> 4) ? 3 : az < (kQ60 >> 2) ? 2 : 1, mul_q60(z, tau)));
+    };
+    auto whole = [&](int n) {
+        return Z[n] == kNoQ60 ? __longlong_as_double(R[n]) : A[n] * from_q60(R[n]);
+    };
+    // integral between offsets ta and tb of segment n (r: upto() of both)
+    auto between = [&](int n, double ta, double tb, int64_t ra, int64_t rb) {
+        if (A[n] == 0.0) return 0.0;
+        if (Z[n] != kNoQ60) return rb > ra ? A[n] * from_q60(rb - ra) : 0.0;
+        const double q1 = slope(n);
+        return A[n] / (q1 * gd.dln[n]) * exp(q1 * ta) * expm1(q1 * (tb - ta));
+    };
     for (int i = part + S * warp; i < nb; i += S * nw) {
         double* qi = qs + (size_t)i * nb;
         const double* di = Dg + (size_t)i * nb;
         for (int j = lane; j <= i; j += 32) qi[j] = j < i ? di[j] : 0.0;
-        const double Ei = E[i];
         int jb = i + 1;
         for (; jb < nb; jb += 32) {
             const int j = jb + lane;
-            double lb = 0.0, la = 0.0;
-            if (j < nb) lb = kHC / (0.5 * (E[j - 1] + E[j]) - Ei);
-            const double nxt = __shfl_down_sync(0xffffffffu, lb, 1);
-            if (j < nb) la = j == M ? 0.0 : (lane < 31 ? nxt : kHC / (0.5 * (E[j] + E[j + 1]) - Ei));
-            double v = 0.0;
-            if (j < nb) {
-                const double a = la > lam0 ? la : lam0, b = lb < lamN ? lb : lamN;
-                if (b > a) {
-                    const int na = seg_of(l32, lam, N, a), nz = seg_of(l32, lam, N, b);
-                    if (na == nz) {
-                        if (om[na] > 0.0) v = seg_part(om[na], sl[na], lam[na], 1, a, b);
-                    } else {
-                        if (om[na] > 0.0) v = seg_part(om[na], sl[na], lam[na], 1, a, lam[na + 1]);
-                        for (int n = na + 1; n < nz; ++n) v += I1[n];
-                        if (om[nz] > 0.0 && b > lam[nz]) v += seg_part(om[nz], sl[nz], lam[nz], 1, lam[nz], b);
-                    }
-                    v /= kH;
+            // the window's long-wavelength edge, element (j, i); n = -1: below the grid (or no such bin)
+            auto edge_of = [&](int jj) {
+                TdEdge r;
+                r.n = -1;
+                r.t = 0.0;
+                r.tau = 0;
+                if (jj < nb) {
+                    const int p0 = rp[jj], p1 = rp[jj + 1];
+                    const int k = i - (jj - (p1 - p0));
+                    if (k >= 0) r = edge[p0 + k];
                 }
-                if (j == i + 1 && lb < lamN) {  // photons too soft to leave bin i
-                    const double x = lb > lam0 ? lb : lam0;
-                    const int n = seg_of(l32, lam, N, x);
-                    double w = S0[n + 1];
-                    if (om[n] > 0.0) w += seg_part(om[n], sl[n], lam[n], 0, x, lam[n + 1]);
-                    v += kC * w / (E[j] - Ei);
+                return r;
+            };
+            const TdEdge b = edge_of(j);
+            const int64_t rb = b.n >= 0 && b.n < N - 1 ? upto(b.n, b.tau) : 0;
+            // the other edge is the next lane's
+            TdEdge a;
+            a.n = __shfl_down_sync(0xffffffffu, b.n, 1);
+            a.t = __shfl_down_sync(0xffffffffu, b.t, 1);
+            int64_t ra = __shfl_down_sync(0xffffffffu, (long long)rb, 1);
+            if (lane == 31) {
+                a = edge_of(j + 1);
+                ra = a.n >= 0 && a.n < N - 1 ? upto(a.n, a.tau) : 0;
+            }
+            if (a.n < 0) {  // from the grid's short end
+                a.n = 0;
+                a.t = 0.0;
+                ra = 0;
+            }
+            if (j < nb) {
+                double v = 0.0;
+                if (b.n >= 0) {
+                    if (a.n == b.n) {
+                        if (b.n < N - 1) v = between(b.n, a.t, b.t, ra, rb);
+                    } else {
+                        v = between(a.n, a.t, gd.dln[a.n], ra, R[a.n]);
+                        for (int n = a.n + 1; n < b.n; ++n) v += whole(n);
+                        if (b.n < N - 1) v += between(b.n, 0.0, b.t, 0, rb);
+                    }
+                }
+                if (j == i + 1 && b.n < N - 1) {  // photons too soft to leave bin i
+                    const double ide = gd.invdE[off + i];
+                    v += b.n < 0 ? soft_end(S0[0], ide)
+                                 : soft_term(gd, g, b.n, ch.ua64[(size_t)b.n * ch.Cc + cell],
+                                             ch.su64[(size_t)b.n * ch.Cc + cell], b.t, b.tau, S0[b.n + 1], ide);
                 }
                 qi[j] = v;
             }
-            if (__all_sync(0xffffffffu, j >= nb || lb <= lam0)) {  // every later window is shortward of the grid
+            if (__all_sync(0xffffffffu, b.n < 0)) {  // every later window is shortward of the grid
                 jb += 32;
                 break;
             }
@@ -617,8 +679,8 @@ long long discrete_batch_spectra(const GrainDev& g, const ChunkDev& ch, long lon
 }
 
 cudaError_t launch_discrete_fill(const GrainDev& g, const ChunkDev& ch, const double* D, const long long* doff,
-                                 const int* gorder, double* q, long long qstride, long long s0, long long n,
-                                 cudaStream_t st) {
+                                 const int* gorder, const TdEdge* edge, double* q, long long qstride, long long s0,
+                                 long long n, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const size_t smem = td_fill_smem_bytes(g.N);
     if (smem > 48 * 1024) {
@@ -629,7 +691,7 @@ cudaError_t launch_discrete_fill(const GrainDev& g, const ChunkDev& ch, const do
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int S = (int)(n >= 2LL * sms ? 1 : std::min(16LL, std::max(1LL, 2LL * sms / n)));
-    k_td_fill<<<(unsigned)(n * S), 256, smem, st>>>(g, ch, D, doff, gorder, s0, q, qstride, S);
+    k_td_fill<<<(unsigned)(n * S), 256, smem, st>>>(g, ch, D, doff, gorder, edge, s0, q, qstride, S);
     return cudaGetLastError();
 }
 
