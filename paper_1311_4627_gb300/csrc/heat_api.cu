@@ -728,20 +728,17 @@ static heat_status ensure_discrete(heat_ctx* ctx, cudaStream_t st) {
         doff[g + 1] = doff[g] + nb * nb;
         woff[g + 1] = woff[g] + nb * (nb - 1) / 2;
     }
-    std::vector<int> order(G);  // grains with the most bins first (the solve's launch order)
-    for (int g = 0; g < G; ++g) order[g] = g;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        return ctx->bin_off[a + 1] - ctx->bin_off[a] > ctx->bin_off[b + 1] - ctx->bin_off[b];
-    });
     if (ctx->d_Dtd.ensure(sizeof(double) * (size_t)std::max(1LL, doff[G])) || upload(ctx->d_Dtd_off, doff) ||
-        upload(ctx->d_Dtd_woff, woff) || upload(ctx->d_Dtd_order, order))
+        upload(ctx->d_Dtd_woff, woff))
         return ctx->fail(HEAT_ENOMEM, "heat_solve: allocation of thermal-discrete rates failed");
     CKR(cudaMemsetAsync(ctx->d_Dtd.p, 0, sizeof(double) * (size_t)doff[G], st));
     const double* gl = ctx->d_gl.as<double>();
     CKR(launch_cooling_window(ctx->N, ctx->d_lam.as<double>(), ctx->d_cabs.as<double>(), ctx->d_bin_off.as<int>(), G,
                               ctx->d_T.as<double>(), ctx->d_E.as<double>(), ctx->d_Dtd_woff.as<long long>(), woff[G],
                               ctx->d_Dtd_off.as<long long>(), ctx->d_Dtd.as<double>(), gl, gl + kGLPoints, st));
-    if (ctx->d_Dtd_edge.ensure(sizeof(TdEdge) * (size_t)std::max(1LL, ctx->band_per_cell)))
+    const size_t n_env = (size_t)ctx->nbt / kGthB + G;
+    if (ctx->d_Dtd_edge.ensure(sizeof(TdEdge) * (size_t)std::max(1LL, ctx->band_per_cell)) ||
+        ctx->d_Dtd_env.ensure(sizeof(int4) * n_env + sizeof(int) * (2 + (size_t)G)))
         return ctx->fail(HEAT_ENOMEM, "heat_solve: allocation of thermal-discrete rates failed");
     GrainDev gd{};
     gd.N = ctx->N;
@@ -753,7 +750,20 @@ static heat_status ensure_discrete(heat_ctx* ctx, cudaStream_t st) {
     gd.rowptr = ctx->d_rowptr.as<int>();
     gd.E = ctx->d_E.as<double>();
     CKR(launch_td_edges(gd, ctx->d_Dtd_edge.as<TdEdge>(), st));
+    int4* env = ctx->d_Dtd_env.as<int4>();
+    int* wmax = (int*)(env + n_env);
+    std::vector<int> info(2 + (size_t)G, 0);
+    CKR(cudaMemsetAsync(wmax, 0, sizeof(int) * info.size(), st));
+    CKR(launch_td_env(gd, ctx->d_Dtd.as<double>(), ctx->d_Dtd_off.as<long long>(), env, wmax, st));
+    CKR(cudaMemcpyAsync(info.data(), wmax, sizeof(int) * info.size(), cudaMemcpyDeviceToHost, st));
     CKR(cudaStreamSynchronize(st));
+    ctx->td_rw = info[0];
+    ctx->td_cw = info[1];
+    std::vector<int> order(G);  // grains whose reduction takes longest first (the solve's launch order)
+    for (int g = 0; g < G; ++g) order[g] = g;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return info[2 + a] > info[2 + b]; });
+    if (upload(ctx->d_Dtd_order, order))
+        return ctx->fail(HEAT_ENOMEM, "heat_solve: allocation of thermal-discrete rates failed");
     ctx->td_built = true;
     return HEAT_OK;
 }
@@ -1085,9 +1095,9 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
                 const long long n = discrete_batch_spectra(gd, ch, s0, td_batch);
                 TIMED(HEAT_T_BUILD, launch_discrete_fill(gd, ch, ctx->d_Dtd.as<double>(), ctx->d_Dtd_off.as<long long>(),
                                                          ctx->d_Dtd_order.as<int>(), ctx->d_Dtd_edge.as<TdEdge>(),
-                                                         sl.tdq.as<double>(), qst, s0, n, cs));
-                TIMED(HEAT_T_RECUR, launch_discrete_gth(gd, ch, ctx->d_Dtd_order.as<int>(), sl.tdq.as<double>(), qst, s0,
-                                                        n, cs));
+                                                         ctx->d_Dtd_env.as<int4>(), sl.tdq.as<double>(), qst, s0, n, cs));
+                TIMED(HEAT_T_RECUR, launch_discrete_gth(gd, ch, ctx->d_Dtd_order.as<int>(), ctx->d_Dtd_env.as<int4>(),
+                                                        ctx->td_rw, ctx->td_cw, sl.tdq.as<double>(), qst, s0, n, cs));
             }
         } else if (fused) {
             ch.phs = sl.phs.as<float>();
@@ -1477,7 +1487,7 @@ void heat_destroy(heat_ctx* ctx) {
                       &ctx->d_T, &ctx->d_E, &ctx->d_Cf, &ctx->d_invC, &ctx->d_invdE, &ctx->d_invdE32, &ctx->d_Cact,
                       &ctx->d_sC, &ctx->d_ca32, &ctx->d_ce32, &ctx->d_sC32, &ctx->d_rowptr, &ctx->d_wmax, &ctx->d_seg_ptr,
                       &ctx->d_seg32, &ctx->d_soft32, &ctx->d_pat_seg, &ctx->d_ca64, &ctx->d_ce64, &ctx->d_cpieces, &ctx->d_pieces, &ctx->d_pseg, &ctx->d_pat64, &ctx->d_pat32, &ctx->d_soft, &ctx->d_soft_off, &ctx->d_K, &ctx->d_Kw, &ctx->d_w,
-                      &ctx->d_koff_all, &ctx->d_cde, &ctx->d_pent, &ctx->d_pcol, &ctx->d_kexp, &ctx->d_rent, &ctx->d_gl, &ctx->d_Dtd, &ctx->d_Dtd_off, &ctx->d_Dtd_woff, &ctx->d_Dtd_order, &ctx->d_Dtd_edge, &ctx->d_u_own, &ctx->s_tasks, &ctx->s_tasks_tail, &ctx->d_status};
+                      &ctx->d_koff_all, &ctx->d_cde, &ctx->d_pent, &ctx->d_pcol, &ctx->d_kexp, &ctx->d_rent, &ctx->d_gl, &ctx->d_Dtd, &ctx->d_Dtd_off, &ctx->d_Dtd_woff, &ctx->d_Dtd_order, &ctx->d_Dtd_edge, &ctx->d_Dtd_env, &ctx->d_u_own, &ctx->s_tasks, &ctx->s_tasks_tail, &ctx->d_status};
     for (DevBuf* b : bufs) b->release();
     for (auto& sl : ctx->slots) {
         DevBuf* sb[] = {&sl.ua64, &sl.su64, &sl.ua32, &sl.Bb64, &sl.Bb32, &sl.xs, &sl.ep,   &sl.pabs,

@@ -153,12 +153,11 @@ cudaError_t launch_cooling_window(int N, const double* lam, const double* cabs, 
                                   cudaStream_t st);
 // P (and the ledger) of the chunk's cells x grains by the full stationary solve, `batch`
 // spectra at a time, each with an nb x nb rate matrix at q + k * qstride.
-// State reduction: states removed per panel, threads per spectrum, and the largest grain whose
-// rate matrix is kept in shared memory (row stride nb + 1; 218,880 B at 160 bins).
+// State reduction: states removed per panel, threads per block, and the rows below a panel whose panel columns are held
+// in shared memory at a time.
 constexpr int kGthB = 8;
 constexpr int kGthThreads = 256;
-constexpr int kGthSmemBins = 160;
-size_t gth_smem_bytes(int max_bins);
+constexpr int kGthRows = 512;
 size_t td_fill_smem_bytes(int N);
 // Shared memory per block of the few-cell recursion up to which the band is staged there.
 constexpr size_t kSmallRecurStage = 100 * 1024;
@@ -169,11 +168,13 @@ constexpr size_t kMaxSmemPerBlock = 227 * 1024;       // opt-in dynamic shared m
 // spectrum from s0 is grain gorder[(s0 + k) / cells], cell (s0 + k) % cells.
 long long discrete_batch_spectra(const GrainDev& g, const ChunkDev& ch, long long s0, long long batch);
 cudaError_t launch_discrete_fill(const GrainDev& g, const ChunkDev& ch, const double* D, const long long* doff,
-                                 const int* gorder, const TdEdge* edge, double* q, long long qstride, long long s0,
-                                 long long n, cudaStream_t st);
+                                 const int* gorder, const TdEdge* edge, const int4* env, double* q, long long qstride,
+                                 long long s0, long long n, cudaStream_t st);
+cudaError_t launch_td_env(const GrainDev& g, const double* D, const long long* doff, int4* env, int* wmax,
+                          cudaStream_t st);
 cudaError_t launch_td_edges(const GrainDev& g, TdEdge* edge, cudaStream_t st);
-cudaError_t launch_discrete_gth(const GrainDev& g, const ChunkDev& ch, const int* gorder, double* q, long long qstride,
-                                long long s0, long long n, cudaStream_t st);
+cudaError_t launch_discrete_gth(const GrainDev& g, const ChunkDev& ch, const int* gorder, const int4* env, int rw,
+                                int cw, double* q, long long qstride, long long s0, long long n, cudaStream_t st);
 
 // ---- emissivity (k_emis.cu)
 // C[z][m][n] = sum_{k in [koff[z], koff[z+1])} A[m][k] B[k][n] for z < nz, m < M, n < N;

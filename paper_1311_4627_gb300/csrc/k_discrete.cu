@@ -243,6 +243,70 @@ cudaError_t launch_td_edges(const GrainDev& g, TdEdge* edge, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// Structure of every grain's rate matrix under the state reduction (once per grain set): states are removed from the
+// top in panels of kGthB (panel p: states p0 .. hi = nb - 1 - kGthB p), and env[p] holds the lowest row with a
+// rate into panel p or a higher one (x), the lowest column its rows reach (y), and the number of panels from
+// p on whose rows have only the next lower column (z; 0 for a panel with any other).  Removing a
+// panel fills rows [x, p0) with its columns [y, p0), which counts for the panels below.  wmax: the most rows (0) and
+// columns (1) below a panel with z = 0; wmax[2 + g]: about how many cycles grain g's reduction takes.  A block per grain.
+__global__ void __launch_bounds__(256) k_td_env(GrainDev gd, const double* __restrict__ Dt,
+                                                const long long* __restrict__ doff, int4* __restrict__ env,
+                                                int* __restrict__ wmax) {
+    __shared__ int jl[kDiscreteMaxBins], lo[kDiscreteMaxBins];
+    const int g = blockIdx.x, off = gd.bin_off[g], nb = gd.bin_off[g + 1] - off;
+    if (nb > kDiscreteMaxBins) return;  // such sets are refused before the solve
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const double* Dg = Dt + doff[g];
+    for (int k = 1 + warp; k < nb; k += nw) {
+        int j0 = k - 1;
+        for (int j = lane; j < k; j += 32)
+            if (Dg[(size_t)k * nb + j] != 0.0) {
+                j0 = min(j0, j);
+                break;
+            }
+        j0 = __reduce_min_sync(0xffffffffu, j0);
+        if (lane == 0) {
+            jl[k] = j0;
+            lo[k] = min(k - 1, k - (gd.rowptr[off + g + k + 1] - gd.rowptr[off + g + k]));
+        }
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    int4* ev = env + (off / kGthB + g);
+    const int np = (nb - 1 + kGthB - 1) / kGthB;
+    int low = nb, rw = 0, cw = 0;
+    long long cost = 300LL * nb;
+    for (int p = 0; p < np; ++p) {
+        const int hi = nb - 1 - kGthB * p, p0 = max(1, hi - kGthB + 1), k = p0 + lane;
+        const bool in = k <= hi;
+        low = min(low, __reduce_min_sync(0xffffffffu, in ? lo[k] : nb));
+        const int jp = __reduce_min_sync(0xffffffffu, in ? jl[k] : nb);
+        const bool adj = __all_sync(0xffffffffu, !in || jl[k] == k - 1);
+        if (lane == 0) ev[p] = make_int4(low, jp, adj ? 1 : 0, 0);
+        if (!adj) {
+            rw = max(rw, p0 - low);
+            cw = max(cw, p0 - jp);
+            cost += 12000 + 4LL * (p0 - low) * (p0 - jp);  // the serial part, kGthB multiply-adds per element
+            for (int i = low + lane; i < p0; i += 32)
+                if (i > 0) jl[i] = min(jl[i], jp);
+        }
+        __syncwarp();
+    }
+    if (lane == 0) {
+        for (int p = np - 2; p >= 0; --p)
+            if (ev[p].z) ev[p].z = ev[p + 1].z + 1;
+        atomicMax(&wmax[0], rw);
+        atomicMax(&wmax[1], cw);
+        wmax[2 + g] = (int)min(cost, 1LL << 30);
+    }
+}
+
+cudaError_t launch_td_env(const GrainDev& g, const double* D, const long long* doff, int4* env, int* wmax,
+                          cudaStream_t st) {
+    k_td_env<<<(unsigned)g.G, 256, 0, st>>>(g, D, doff, env, wmax);
+    return cudaGetLastError();
+}
+
 // Shared memory of k_td_fill for a grid of N wavelengths, per segment: the cell's A = Omega_n lambda_n^2 dln / h,
 // Z = (slope + 2) dln in Q60 (kNoQ60: |Z| >= 1), R = E1(Z) in Q60 (kNoQ60: the bits of the whole segment's integral), and
 // the suffix sums of the integrals of Omega.
@@ -250,7 +314,7 @@ size_t td_fill_smem_bytes(int N) { return 32 * (size_t)N; }
 constexpr int64_t kNoQ60 = INT64_MIN;
 
 // Spectrum of block b of a launch that starts at spectrum s0: grains in the order `gorder`
-// (most bins first), every cell of the chunk for each grain in turn, so that the spectra of one
+// (longest state reduction first), every cell of the chunk for each grain in turn, so that the spectra of one
 // launch have similar cost and the largest start first.
 __device__ __forceinline__ void td_spectrum(const ChunkDev& ch, const int* gorder, long long s0, int& cell, int& g,
                                             int b = -1) {
@@ -260,8 +324,8 @@ __device__ __forceinline__ void td_spectrum(const ChunkDev& ch, const int* gorde
 }
 
 // S blocks per spectrum (cell, grain) of the chunk's cells, each the rows i = part (mod S): q
-// [nb][nb] (row-major, rate from row to column) at q + spectrum * qstride, and the absorbed
-// power c int Omega on the grid (part 0).
+// [nb][nb] (row-major, rate from row to column) at q + spectrum * qstride, the elements that the state reduction
+// touches (env), and the absorbed power c int Omega on the grid (part 0).
 // Downward rates are copied from the grain's table (Dt[u][l], from u to l).  The heating
 // rate from i into bin j > i is (1/h) int Omega lambda over the photon wavelengths that end in
 // bin j, [hc/(Ehi_j - E_i), hc/(Elo_j - E_i)] (Ehi_M = infinity), plus on j = i + 1 the
@@ -275,8 +339,8 @@ __device__ __forceinline__ void td_spectrum(const ChunkDev& ch, const int* gorde
 // the fill was bound by the FP64 unit (83 % busy): 8 cells x 64 grains x 1024 wavelengths 8.7 ms, now 2.0 ms.
 __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const double* __restrict__ Dt,
                                                  const long long* __restrict__ doff, const int* __restrict__ gorder,
-                                                 const TdEdge* __restrict__ edge, long long s0, double* q,
-                                                 long long qstride, int S) {
+                                                 const TdEdge* __restrict__ edge, const int4* __restrict__ env,
+                                                 long long s0, double* q, long long qstride, int S) {
     extern __shared__ double fsm[];
     const int bsp = blockIdx.x / S, part = blockIdx.x % S;  // spectrum of the launch, part of its rows
     int cell, g;
@@ -334,6 +398,8 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
     const double* E = gd.E + off;
     const double* Dg = Dt + doff[g];
     const int* rp = gd.rowptr + off + g;
+    const int4* ev = env + (off / kGthB + g);
+    const int np = (nb - 1 + kGthB - 1) / kGthB;
     double* qs = q + (size_t)bsp * qstride;
     // the cell's slope + 2 of segment n (only where |Z| >= 1)
     auto slope = [&](int n) { return ch.su64[(size_t)n * ch.Cc + cell] + gd.sC[(size_t)g * N + n] + 2.0; };
@@ -357,9 +423,17 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
     for (int i = part + S * warp; i < nb; i += S * nw) {
         double* qi = qs + (size_t)i * nb;
         const double* di = Dg + (size_t)i * nb;
-        for (int j = lane; j <= i; j += 32) qi[j] = j < i ? di[j] : 0.0;
-        int jb = i + 1;
-        for (; jb < nb; jb += 32) {
+        const int p = min((nb - 1 - i) / kGthB, np - 1);  // row 0 is in no panel: its first column is its own
+        for (int j = (i == 0 ? 0 : ev[p].z ? i - 1 : ev[p].y) + lane; j <= i; j += 32) qi[j] = j < i ? di[j] : 0.0;
+        int reach = i;  // the row's last column
+        for (int pb = 0; pb < np; pb += 32) {
+            const unsigned m = __ballot_sync(0xffffffffu, pb + lane < np && ev[min(pb + lane, np - 1)].x <= i);
+            if (m) {
+                reach = nb - 1 - kGthB * (pb + __ffs(m) - 1);
+                break;
+            }
+        }
+        for (int jb = i + 1; jb <= reach; jb += 32) {
             const int j = jb + lane;
             // the window's long-wavelength edge, element (j, i); n = -1: below the grid (or no such bin)
             auto edge_of = [&](int jj) {
@@ -390,7 +464,7 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
                 a.t = 0.0;
                 ra = 0;
             }
-            if (j < nb) {
+            if (j <= reach) {
                 double v = 0.0;
                 if (b.n >= 0) {
                     if (a.n == b.n) {
@@ -409,12 +483,7 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
                 }
                 qi[j] = v;
             }
-            if (__all_sync(0xffffffffu, b.n < 0)) {  // every later window is shortward of the grid
-                jb += 32;
-                break;
-            }
         }
-        for (int j = jb + lane; j < nb; j += 32) qi[j] = 0.0;
     }
     if (tid == 0 && part == 0 && ch.pabs) ch.pabs[(size_t)cell * gd.G + g] = kC * S0[0];
 }
@@ -439,201 +508,337 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 
 }  // namespace
 
-// Exit rate of state k, s_k = sum_{j < k} q_kj, its reciprocal, and the lowest column with a
-// rate out of k (k if none), by one warp; lane 0 stores them.  The lanes read the row as
-// j = lane + 32 t, so a warp that has just written the row calls __syncwarp first.
-__device__ __forceinline__ void row_exit(const double* qk, int k, double* s, double* rs, int* jlo, int lane) {
-    double part = 0.0;
-    int jl = k;
-    for (int j = lane; j < k; j += 32) {
-        const double v = qk[j];
-        part += v;
-        if (v != 0.0 && j < jl) jl = j;
-    }
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    jl = __reduce_min_sync(0xffffffffu, jl);
-    if (lane == 0) {
-        s[k] = part;
-        rs[k] = part > 0.0 ? 1.0 / part : 0.0;  // s_k = 0: nothing leaves k downward
-        jlo[k] = jl;
-    }
+namespace {
+
+// Reciprocal of x >= 0 (0 for 0): for a mantissa m in [1, 2) the hardware's FP32 reciprocal y of its leading
+// bits (relative error e = 1 - m y < 2^-21), then y + y (e + e^2), whose error e^3 is below 2^-63, so that the result
+// is off by half an ulp and 2^-10 of one.  Three dependent FP64 operations of 64 cycles where a division has eight.
+__device__ __forceinline__ double rcp_or_0(double x) {
+    const int h = __double2hiint(x), l = __double2loint(x), ex = h >> 20;
+    if ((unsigned)(ex - 64) > 1900u) return x > 0.0 ? 1.0 / x : 0.0;  // zero, subnormal, very large, infinite
+    const double m = __hiloint2double((h & 0xfffff) | 0x3ff00000, l);
+    float yf;
+    asm("rcp.approx.ftz.f32 %0, %1;"
+        : "=f"(yf)
+        : "f"(__uint_as_float(0x3f800000u | ((unsigned)(h & 0xfffff) << 3) | ((unsigned)l >> 29))));
+    const unsigned fb = __float_as_uint(yf);
+    double y = __hiloint2double((int)((fb >> 3) + 0x38000000u), (int)(fb << 29));
+    const double e = fma(-m, y, 1.0);
+    y = fma(y, fma(e, e, e), y);
+    return __hiloint2double(__double2hiint(y) + ((1023 - ex) << 20), __double2loint(y));
 }
 
-// One block per spectrum: state reduction of q, back substitution, P and the energy check.
-//
-// States are removed kGthB at a time (a panel [p0, hi]).  Removing state k adds
-// q_ik q_kj / s_k to q_ij for i, j < k.  Inside the panel, step by step, for the rows of the
-// panel's remaining states; after the panel, for the rows below it, first their panel columns
-// (a sweep over the panel's states in removal order, in registers) and then the block below
-// the panel in one pass: sum over the panel's k of q_ik (q_kj / s_k), a rank-kGthB product
-// in which q_ik is column k as it stood when k was removed (final from then on: it is the
-// column the back substitution reads) and q_kj / s_k is row k at that time, kept in U.  Every
-// term stays a sum of products of non-negative numbers; only the order of the additions
-// differs from removing the states one by one.  The diagonal of q is never read (s_k sums
-// the off-diagonal row), so the updates do not skip it.  The warp that updates the row of the
-// next state to be removed also sums it (row_exit), so a step waits on no block-wide sum.
-// The fill-in of removing k stays inside the rows that reach k and the columns k reaches:
-// rows with no rate into the panel are skipped and columns start at the panel's lowest.
-//
-// Back substitution, right-looking: X_0 = 1, and once X_i is final every column n > i
-// (owned by a fixed thread) takes X_i q_in; X_{i+1} is then complete and its owner divides by
-// s_{i+1}.  Past 2^800 every X is scaled by 2^-800 (exact).  P = X / sum X.
-//
-// SMQ: q is copied into shared memory (row stride nb + 1), for grains of up to kGthSmemBins
-// bins; otherwise it is updated in place in device memory, where each panel reads and writes
-// the block below it once for kGthB fused multiply-adds per element.
-// Shared memory: s, 1/s, X [nb] each, U [kGthB][nb], the lowest columns [nb] (ints, padded
-// to doubles), then q (SMQ).
-static_assert(kGthB - 1 < kGthThreads / 32, "k_gth: the last warp must be free of panel rows");
-template <bool SMQ>
-__global__ void __launch_bounds__(kGthThreads, 1) k_gth(GrainDev gd, ChunkDev ch, const int* __restrict__ gorder,
-                                                        long long s0, double* q, long long qstride) {
-    extern __shared__ double smd[];
-    __shared__ double red[kGthThreads / 32];
-    __shared__ int rescale;
-    int cell, g;
-    td_spectrum(ch, gorder, s0, cell, g);
-    const int off = gd.bin_off[g], nb = gd.bin_off[g + 1] - off;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kGthThreads / 32;
-    double* s = smd;
-    double* rs = s + nb;
-    double* X = rs + nb;
-    double* U = X + nb;
-    int* jlo = (int*)(U + kGthB * nb);
-    double* qg = q + (size_t)blockIdx.x * qstride;
-    double* qs = qg;
-    int ld = nb;
-    if (SMQ) {
-        qs = U + kGthB * nb + (nb + 1) / 2;
-        ld = nb + 1;
-        for (int i = warp; i < nb; i += nw)
-            for (int j = lane; j < nb; j += 32) qs[(size_t)i * ld + j] = qg[(size_t)i * nb + j];
+// 1/s as kept for the back substitution: -1 where nothing leaves a state downward.  Comparisons are on the bits:
+// the FP64 unit takes 64 cycles for one too.
+__device__ __forceinline__ double exit_of(double s, double r) { return __double_as_longlong(s) == 0 ? -1.0 : r; }
+
+template <bool CLUSTER>
+__device__ __forceinline__ void gth_sync() {
+    if (CLUSTER)
+        asm volatile(
+            "barrier.cluster.arrive.release;\n\t"
+            "barrier.cluster.wait.acquire;" ::
+                : "memory");
+    else
         __syncthreads();
-    }
-    if (warp == 0) row_exit(qs + (size_t)(nb - 1) * ld, nb - 1, s, rs, jlo, lane);
-    if (tid == 0) rescale = 0;
+}
+
+}  // namespace
+
+// Shared memory of k_gth: 1/s and X [nb], the panel's rows below it [kGthB][cw], the rows' panel columns
+// [rcap][kGthB], the panel table.
+size_t gth_smem_bytes(int max_bins, int rcap, int cw) {
+    const int np = (max_bins + kGthB - 1) / kGthB;
+    return sizeof(double) * (2 * (size_t)max_bins + (size_t)kGthB * cw + (size_t)kGthB * rcap + 2) +
+           sizeof(int4) * (size_t)np;
+}
+
+// One block (CLUSTER: a cluster of C blocks) per spectrum: state reduction of q, back substitution, P and the
+// energy check.
+//
+// States are removed from the top; removing state k, with s_k = sum_{j < k} q_kj, adds q_ik q_kj / s_k to q_ij
+// for i, j < k.  Every term is a product of non-negative numbers.  kGthB states [p0, hi] are removed at a time:
+//  - The panel by itself: its kGthB x kGthB block and, per row, the sums R(m) of the elements below column m
+//    (the row's sum below the panel and the block's lower part).  They are updated like
+//    elements, R_i(m) += (q_ik / s_k) R_k(m) for m <= i, so s_k = R_k(k) is at hand when k's turn comes without a sum
+//    over the row and without the rest of the row.  One warp, four numbers a lane, no barrier: per state the
+//    chain is a shuffle, a reciprocal, a multiply and a multiply-add (about 500 cycles).
+//  - Then, with the panel's multipliers known, its rows below the panel, a thread per column, and the
+//    panel's columns of the rows below, a thread per row.
+//  - Then the block below: q_ij += sum_k (q_ik / s_k) q_kj, a warp per two rows and 32 columns.
+// Rows that do not reach the panel and columns it does not reach are left out (env).  A run of panels whose rows
+// have only the next lower column (grains whose levels are wider than the photons they emit) fills nothing below the
+// diagonal: all its s_k = q_k,k-1 are known at once, and removing k moves q_ik to q_i,k-1, a thread per row.
+//
+// Back substitution: X_0 = 1, X_n = sum_{i < n} X_i q_in / s_n, in ascending i, 32 states at a time: one warp
+// through the 32 x 32 block in shared memory (a lane per column; multiply, shuffle, multiply-add per state), then all
+// threads add the 32 rows to the columns beyond.  Past 2^800 every X is scaled by 2^-800 (exact).  P = X / sum X.
+//
+// Removing state by state with a barrier, a sum over the row and a division each took 5,000 cycles a state at
+// 128 bins, two thirds of them waiting: 8 spectra x 128 bins 431 us, now 186 us; 512 spectra of 128 ..
+// 1024 bins 7.7 ms, now 1.2 ms.  At 128 bins, where every rate is non-zero, one block is bound by its
+// SM's FP64 unit (183 us for the nb^3 / 3 multiply-adds), hence the cluster when a launch has few spectra:
+// rows below a panel go round the blocks in pairs, and each block repeats the panel's own part.
+template <bool CLUSTER>
+__global__ void __launch_bounds__(kGthThreads, 2) k_gth(GrainDev gd, ChunkDev ch, const int* __restrict__ gorder,
+                                                        const int4* __restrict__ env, int rcap, int cw, int C,
+                                                        long long s0, double* q, long long qstride) {
+    extern __shared__ __align__(16) double smd[];
+    __shared__ double red[kGthThreads / 32];
+    __shared__ double tile[32][32];
+    __shared__ double As[kGthB][kGthB], CL[kGthB][kGthB], UA[kGthB][kGthB], Rs[kGthB], rk[kGthB];
+    constexpr int nw = kGthThreads / 32;
+    static_assert(kGthB == 8 && nw >= kGthB, "k_gth: a warp per panel row, four numbers of the panel per lane");
+    const int rank = CLUSTER ? (int)(blockIdx.x % C) : 0, sp = CLUSTER ? (int)(blockIdx.x / C) : (int)blockIdx.x;
+    const int nC = CLUSTER ? C : 1;
+    int cell, g;
+    td_spectrum(ch, gorder, s0, cell, g, sp);
+    const int off = gd.bin_off[g], nb = gd.bin_off[g + 1] - off;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double* Ls = smd;                      // [rcap][kGthB], rcap even
+    double* U = Ls + (size_t)rcap * kGthB;  // [kGthB][cw]
+    double* rs = U + (size_t)kGthB * cw;
+    double* X = rs + nb;
+    int4* ev = (int4*)(X + nb);  // an even number of doubles before it
+    double* qs = q + (size_t)sp * qstride;
+    const int np = (nb - 1 + kGthB - 1) / kGthB;
+    for (int p = tid; p < np; p += kGthThreads) ev[p] = env[off / kGthB + g + p];
     __syncthreads();
-    for (int hi = nb - 1; hi >= 1; hi -= kGthB) {
-        const int p0 = hi - kGthB + 1 > 1 ? hi - kGthB + 1 : 1;
-        const int nk = hi - p0 + 1;
-        for (int k = hi; k >= p0; --k) {
-            double* Uk = U + (size_t)(hi - k) * nb;
-            const double* qk = qs + (size_t)k * ld;
-            const double r = rs[k];
-            const int jk = jlo[k];
-            // the last warp (never one of the panel's rows below k: at most kGthB - 1 < nw of them)
-            // keeps the normalised row for the rows below the panel, while the panel's rows take
-            // their multiple of row k directly: no barrier between the two
-            if (warp == nw - 1)
-                for (int j = lane; j < k; j += 32) Uk[j] = j < jk ? 0.0 : qk[j] * r;
-            for (int i = p0 + warp; i < k; i += nw) {  // the panel's rows below k, columns from jk
-                double* qi = qs + (size_t)i * ld;
-                const double qik = qi[k];
-                if (qik != 0.0) {
-                    const double c = qik * r;
-                    for (int j = jk + lane; j < k; j += 32) qi[j] = fma(c, qk[j], qi[j]);
+    const int pi = lane & 7, pc = lane >> 3;  // the panel in warp 0: row, first column (and + 4)
+    double b0 = 0.0, b1 = 0.0;                // the last panel's block above the diagonal, stored one panel late:
+    int bp = -1, bn = 0;                              // other blocks of the cluster may still be reading it
+    auto store_block = [&]() {
+        if (warp == 0 && rank == 0 && bp > 0) {
+            double* qr = qs + (size_t)(bp + pi) * nb + bp;
+            if (pc > pi && pc < bn) qr[pc] = b0;
+            if (pc + 4 > pi && pc + 4 < bn) qr[pc + 4] = b1;
+        }
+    };
+    for (int p = 0; p < np;) {
+        const int4 e = ev[p];
+        const int hi = nb - 1 - kGthB * p;
+        if (e.z > 0) {  // a run of panels with adjacent downward rates only
+            const int pe = p + e.z, a = max(1, nb - kGthB * pe), lo = ev[pe - 1].x;
+            for (int k = a + tid; k <= hi; k += kGthThreads) {
+                const double s = qs[(size_t)k * nb + k - 1];
+                rs[k] = exit_of(s, rcp_or_0(s));
+            }
+            __syncthreads();
+            for (int i = lo + rank * kGthThreads + tid; i < hi - 1; i += nC * kGthThreads) {
+                int t0 = p, t1 = pe;  // first panel of the run that row i reaches (x falls with the panel)
+                while (t0 < t1) {
+                    const int m = (t0 + t1) >> 1;
+                    if (ev[m].x > i) t0 = m + 1; else t1 = m;
                 }
-                if (i == k - 1) {  // the next state to be removed
-                    __syncwarp();
-                    row_exit(qi, k - 1, s, rs, jlo, lane);
+                const int top = nb - 1 - kGthB * t0;
+                double* qi = qs + (size_t)i * nb;
+                const int bot = max(a, i + 2);
+                if (top < bot) continue;
+                double x = qi[top];
+                for (int k = top; k >= bot; k -= 8) {
+                    double v[8];
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) v[t] = k - t >= bot ? qi[k - t - 1] : 0.0;
+#pragma unroll
+                    for (int t = 0; t < 8; ++t)
+                        if (k - t >= bot) {
+                            x = __double2hiint(rs[k - t]) > 0 ? v[t] + x : v[t];
+                            qi[k - t - 1] = x;
+                        }
+                }
+            }
+            gth_sync<CLUSTER>();
+            store_block();
+            bp = -1;
+            p = pe;
+            continue;
+        }
+        const int p0 = max(1, hi - kGthB + 1), nk = hi - p0 + 1, ilo = e.x, jp = e.y, nc = p0 - jp, nr = p0 - ilo;
+        // the panel's block and its rows' sums below it
+        if (tid < kGthB * kGthB) {
+            const int i = tid >> 3, c = tid & 7;
+            As[i][c] = i < nk && c < nk && i != c ? qs[(size_t)(p0 + i) * nb + p0 + c] : 0.0;
+        }
+        if (warp < kGthB) {
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            if (warp < nk) {
+                const double* qk = qs + (size_t)(p0 + warp) * nb;
+                for (int j = jp + lane; j < p0; j += 128)
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) s[t] += j + 32 * t < p0 ? qk[j + 32 * t] : 0.0;
+            }
+            double t = (s[0] + s[1]) + (s[2] + s[3]);
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) Rs[warp] = t;
+        }
+        __syncthreads();
+        store_block();
+        bp = -1;
+        if (warp == 0) {
+            double e0 = As[pi][pc], e1 = As[pi][pc + 4], R0 = Rs[pi], R1;
+#pragma unroll
+            for (int m = 0; m < 3; ++m) R0 = m < pc ? R0 + As[pi][m] : R0;
+            R1 = R0;
+#pragma unroll
+            for (int m = 0; m < 7; ++m) R1 = m >= pc && m < pc + 4 ? R1 + As[pi][m] : R1;
+            double rown = 0.0;  // 1/s of this lane's row
+#pragma unroll
+            for (int k = kGthB - 1; k >= 0; --k) {
+                const double s = __shfl_sync(0xffffffffu, k < 4 ? R0 : R1, k | ((k & 3) << 3));
+                const double r = rcp_or_0(s);
+                if (pi == k) rown = r;
+                if (lane == 0 && k < nk) rs[p0 + k] = exit_of(s, r);
+                if (k == 0) break;
+                const double qik = __shfl_sync(0xffffffffu, k < 4 ? e0 : e1, pi | ((k & 3) << 3));
+                const int src = k | (pc << 3);
+                const double v0 = __shfl_sync(0xffffffffu, e0, src), u0 = __shfl_sync(0xffffffffu, R0, src);
+                const double c = qik * r;
+                if (pi < k) {
+                    if (pc == 0) CL[pi][k] = c;
+                    R0 = fma(c, u0, R0);
+                    if (pc < k) e0 = fma(c, v0, e0);
+                }
+                if (k > 4) {
+                    const double v1 = __shfl_sync(0xffffffffu, e1, src), u1 = __shfl_sync(0xffffffffu, R1, src);
+                    if (pi < k) {
+                        R1 = fma(c, u1, R1);
+                        if (pc + 4 < k) e1 = fma(c, v1, e1);
+                    }
+                }
+            }
+            UA[pi][pc] = e0 * rown;
+            UA[pi][pc + 4] = e1 * rown;
+            if (pc == 0) rk[pi] = rown;
+            b0 = e0;
+            b1 = e1;
+            bp = p0;
+            bn = nk;
+        }
+        __syncthreads();
+        // rows below the panel: this block's, in pairs
+        const int lp_all = (nr + 1) / 2, lp_own = (lp_all - rank + nC - 1) / nC;
+        const int ncp = (nc + 31) & ~31;
+        for (int l0 = 0; l0 == 0 || l0 < 2 * lp_own; l0 += rcap) {
+            const int ln = min(rcap, 2 * lp_own - l0);  // rows of this turn
+            auto row_of = [&](int l) { return ilo + 2 * (((l0 + l) >> 1) * nC + rank) + (l & 1); };
+            for (int t = (l0 == 0 ? 0 : ncp) + tid; t < ncp + ln; t += kGthThreads) {
+                asm volatile("" ::: "memory");  // read the multipliers per turn: they'd fill the registers
+                if (t < ncp) {  // a column of the panel's rows
+                    if (t >= nc) continue;
+                    double v[kGthB];
+#pragma unroll
+                    for (int k = 0; k < kGthB; ++k) v[k] = k < nk ? qs[(size_t)(p0 + k) * nb + jp + t] : 0.0;
+#pragma unroll
+                    for (int k = kGthB - 1; k > 0; --k)
+#pragma unroll
+                        for (int i = 0; i < k; ++i) v[i] = fma(CL[i][k], v[k], v[i]);
+#pragma unroll
+                    for (int k = 0; k < kGthB; ++k) U[k * cw + t] = v[k];
+                } else {  // a row's panel columns
+                    const int l = t - ncp, i = row_of(l);
+                    double x[kGthB];
+                    double* qi = qs + (size_t)i * nb + p0;
+#pragma unroll
+                    for (int k = 0; k < kGthB; ++k) x[k] = i < p0 && k < nk ? qi[k] : 0.0;
+#pragma unroll
+                    for (int k = kGthB - 1; k > 0; --k)
+#pragma unroll
+                        for (int j = 0; j < k; ++j) x[j] = fma(x[k], UA[k][j], x[j]);
+#pragma unroll
+                    for (int k = 0; k < kGthB; ++k) {
+                        if (i < p0 && k < nk) qi[k] = x[k];
+                        Ls[l * kGthB + k] = x[k] * rk[k];
+                    }
                 }
             }
             __syncthreads();
+            // the block below: two rows and 32 columns per warp
+            const int ncc = ncp >> 5, nt = ln > 0 ? (ln / 2) * ncc : 0;
+            double v0 = 0.0, v1 = 0.0, n0 = 0.0, n1 = 0.0;
+            auto load = [&](int t, double& x0, double& x1) {
+                const int l = 2 * (t / ncc), j = jp + 32 * (t % ncc) + lane, i = row_of(l);
+                if (t < nt && j < p0) {
+                    x0 = qs[(size_t)i * nb + j];
+                    if (i + 1 < p0) x1 = qs[(size_t)(i + 1) * nb + j];
+                }
+            };
+            if (nt > 0) load(warp, n0, n1);
+            for (int t = warp; t < nt; t += nw) {
+                v0 = n0;
+                v1 = n1;
+                load(t + nw, n0, n1);
+                const int l = 2 * (t / ncc), cj = 32 * (t % ncc) + lane, i = row_of(l);
+                const double2* L0 = (const double2*)(Ls + l * kGthB);
+                const double* Uj = U + min(cj, nc - 1);
+#pragma unroll
+                for (int k = kGthB - 2; k >= 0; k -= 2) {
+                    const double2 a = L0[k >> 1], b = L0[(k >> 1) + kGthB / 2];
+                    const double uh = Uj[(k + 1) * cw], ul = Uj[k * cw];
+                    v0 = fma(a.y, uh, v0);
+                    v1 = fma(b.y, uh, v1);
+                    v0 = fma(a.x, ul, v0);
+                    v1 = fma(b.x, ul, v1);
+                }
+                if (cj < nc) {
+                    qs[(size_t)i * nb + jp + cj] = v0;
+                    if (i + 1 < p0) qs[(size_t)(i + 1) * nb + jp + cj] = v1;
+                }
+            }
+            if (l0 + rcap < 2 * lp_own) __syncthreads();
         }
-        if (nk > 1)  // rows below the panel: the panel's columns, state by state in removal order
-            for (int i = tid; i < p0; i += kGthThreads) {
-                double* qi = qs + (size_t)i * ld;
-                double x[kGthB];
-                bool any = false;
-#pragma unroll
-                for (int kk = 0; kk < kGthB; ++kk) {
-                    const double v = qi[hi - kk > 0 ? hi - kk : 0];
-                    x[kk] = kk < nk ? v : 0.0;
-                    any |= x[kk] != 0.0;
-                }
-                if (!any) continue;
-#pragma unroll
-                for (int kk = 0; kk < kGthB - 1; ++kk) {
-                    if (kk < nk - 1 && x[kk] != 0.0) {
-                        const double* Uk = U + (size_t)kk * nb;
-#pragma unroll
-                        for (int k2 = kk + 1; k2 < kGthB; ++k2)
-                            if (k2 < nk) x[k2] = fma(x[kk], Uk[hi - k2], x[k2]);
-                    }
-                }
-#pragma unroll
-                for (int kk = 1; kk < kGthB; ++kk)
-                    if (kk < nk) qi[hi - kk] = x[kk];
-            }
-        int jp = nb;
-        for (int k = p0; k <= hi; ++k) jp = jlo[k] < jp ? jlo[k] : jp;
-        __syncthreads();
-        // the block below the panel, two rows per warp so that each U value loaded serves both
-        // (each element's FMAs in the same order as one row at a time); rows with no rate into
-        // the panel are left as they are
-        for (int i0 = 2 * warp; i0 < p0; i0 += 2 * nw) {
-            const bool has1 = i0 + 1 < p0;
-            double* q0 = qs + (size_t)i0 * ld;
-            double* q1 = qs + (size_t)(has1 ? i0 + 1 : i0) * ld;
-            const double lv0 = lane < nk ? q0[hi - lane] : 0.0;
-            const double lv1 = (has1 && lane < nk) ? q1[hi - lane] : 0.0;
-            const bool a0 = __ballot_sync(0xffffffffu, lv0 != 0.0) != 0u;
-            const bool a1 = __ballot_sync(0xffffffffu, lv1 != 0.0) != 0u;
-            if (a0 || a1) {
-                double l0[kGthB], l1[kGthB];
-#pragma unroll
-                for (int kk = 0; kk < kGthB; ++kk) {
-                    l0[kk] = __shfl_sync(0xffffffffu, lv0, kk);
-                    l1[kk] = __shfl_sync(0xffffffffu, lv1, kk);
-                }
-                for (int j = jp + lane; j < p0; j += 32) {
-                    double v0 = q0[j], v1 = q1[j];
-#pragma unroll
-                    for (int kk = 0; kk < kGthB; ++kk) {
-                        const double u = U[kk * nb + j];
-                        v0 = fma(l0[kk], u, v0);
-                        v1 = fma(l1[kk], u, v1);
-                    }
-                    if (a0) q0[j] = v0;
-                    if (a1) q1[j] = v1;
-                }
-            }
-            const int inext = p0 - 1;  // the first state of the next panel
-            if (inext > 0 && (i0 == inext || (has1 && i0 + 1 == inext))) {
-                __syncwarp();
-                row_exit(qs + (size_t)inext * ld, inext, s, rs, jlo, lane);
-            }
-        }
-        __syncthreads();
+        gth_sync<CLUSTER>();
+        ++p;
     }
-    // back substitution
+    store_block();
+    if (rank != 0) return;
+    // back substitution (X holds the sums so far beyond the current block)
     for (int n = tid; n < nb; n += kGthThreads) X[n] = n == 0 ? 1.0 : 0.0;
+    if (tid == 0) rs[0] = 1.0;
     __syncthreads();
     bool bad = false;
-    for (int i = 0; i + 1 < nb; ++i) {
-        const double xi = X[i];
-        const double* qi = qs + (size_t)i * ld;
-        for (int n = tid; n < nb; n += kGthThreads) {
-            if (n <= i) continue;
-            double a = fma(xi, qi[n], X[n]);
-            if (n == i + 1) {  // every state below n has contributed
-                if (s[n] == 0.0) {
-                    bad |= a != 0.0;
-                    a = 0.0;
-                } else {
-                    a *= rs[n];
+    auto low_of = [&](int n) { return n == 0 ? 0 : ev[(nb - 1 - n) / kGthB].x; };
+    for (int n0 = 0; n0 < nb; n0 += 32) {
+        const int n = n0 + lane;
+        const bool in = n < nb;
+        const int low = in ? low_of(n) : nb;
+#pragma unroll
+        for (int i = warp; i < 32; i += nw)
+            tile[i][lane] = i < lane && n0 + i >= low ? qs[(size_t)(n0 + i) * nb + n] : 0.0;
+        __syncthreads();
+        if (warp == 0) {
+            double x = in ? X[n] : 0.0;
+            const double r = in ? rs[n] : 0.0;
+#pragma unroll 8
+            for (int i = 0; i < 32; ++i) {
+                double xi = x * r;  // lane i: every state below it has contributed
+                if (lane == i) {
+                    if (__double2hiint(r) < 0) {
+                        bad |= x != 0.0;
+                        xi = 0.0;
+                    }
+                    x = xi;
                 }
-                if (a > 0x1p800) rescale = 1;
+                xi = __shfl_sync(0xffffffffu, xi, i);
+                if (__double2hiint(xi) >= (1023 + 800) << 20) {
+                    xi *= 0x1p-800;
+                    x *= 0x1p-800;
+                    for (int m = lane; m < nb; m += 32)
+                        if (m < n0 || m >= n0 + 32) X[m] *= 0x1p-800;
+                }
+                if (lane > i) x = fma(xi, tile[i][lane], x);
             }
-            X[n] = a;
+            if (in) X[n] = x;
         }
         __syncthreads();
-        if (rescale) {
-            for (int n = tid; n < nb; n += kGthThreads) X[n] *= 0x1p-800;
-            __syncthreads();
-            if (tid == 0) rescale = 0;
-            __syncthreads();
+        for (int n = n0 + 32 + tid; n < nb; n += kGthThreads) {
+            const int low = max(low_of(n), n0);
+            if (low >= n0 + 32) break;  // nor do the columns beyond reach down here
+            double x = X[n];
+#pragma unroll 8
+            for (int i = low; i < n0 + 32; ++i) x = fma(X[i], qs[(size_t)i * nb + n], x);
+            X[n] = x;
         }
+        __syncthreads();
     }
     bad = __syncthreads_or(bad);
     double part = 0.0;
@@ -642,9 +847,9 @@ __global__ void __launch_bounds__(kGthThreads, 1) k_gth(GrainDev gd, ChunkDev ch
     double emit = 0.0;
     double* prow = ch.P + (size_t)cell * ch.ldP + off;
     for (int i = tid; i < nb; i += kGthThreads) {
-        const double p = X[i] * inv;
-        prow[i] = p;
-        emit = fma(p, gd.cde[off + i], emit);
+        const double pr = X[i] * inv;
+        prow[i] = pr;
+        emit = fma(pr, gd.cde[off + i], emit);
     }
     emit = block_sum(emit, red);
     if (tid == 0) {
@@ -668,19 +873,14 @@ cudaError_t launch_cooling_window(int N, const double* lam, const double* cabs, 
     return cudaGetLastError();
 }
 
-size_t gth_smem_bytes(int max_bins) {
-    const size_t vec = sizeof(double) * ((size_t)(3 + kGthB) * max_bins + (max_bins + 1) / 2);
-    return max_bins <= kGthSmemBins ? vec + sizeof(double) * (size_t)max_bins * (max_bins + 1) : vec;
-}
-
 long long discrete_batch_spectra(const GrainDev& g, const ChunkDev& ch, long long s0, long long batch) {
     const long long spectra = (long long)ch.cells * g.G;
     return spectra - s0 < batch ? spectra - s0 : batch;
 }
 
 cudaError_t launch_discrete_fill(const GrainDev& g, const ChunkDev& ch, const double* D, const long long* doff,
-                                 const int* gorder, const TdEdge* edge, double* q, long long qstride, long long s0,
-                                 long long n, cudaStream_t st) {
+                                 const int* gorder, const TdEdge* edge, const int4* env, double* q, long long qstride,
+                                 long long s0, long long n, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const size_t smem = td_fill_smem_bytes(g.N);
     if (smem > 48 * 1024) {
@@ -691,25 +891,39 @@ cudaError_t launch_discrete_fill(const GrainDev& g, const ChunkDev& ch, const do
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int S = (int)(n >= 2LL * sms ? 1 : std::min(16LL, std::max(1LL, 2LL * sms / n)));
-    k_td_fill<<<(unsigned)(n * S), 256, smem, st>>>(g, ch, D, doff, gorder, edge, s0, q, qstride, S);
+    k_td_fill<<<(unsigned)(n * S), 256, smem, st>>>(g, ch, D, doff, gorder, edge, env, s0, q, qstride, S);
     return cudaGetLastError();
 }
 
-cudaError_t launch_discrete_gth(const GrainDev& g, const ChunkDev& ch, const int* gorder, double* q, long long qstride,
-                                long long s0, long long n, cudaStream_t st) {
+cudaError_t launch_discrete_gth(const GrainDev& g, const ChunkDev& ch, const int* gorder, const int4* env, int rw,
+                                int cw, double* q, long long qstride, long long s0, long long n, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    const bool smq = g.max_bins <= kGthSmemBins;
-    const size_t smem = gth_smem_bytes(g.max_bins);
-    if (smem > 48 * 1024) {
-        cudaError_t e = smq ? cudaFuncSetAttribute(k_gth<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                            : cudaFuncSetAttribute(k_gth<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    if (smq)
-        k_gth<true><<<(unsigned)n, kGthThreads, smem, st>>>(g, ch, gorder, s0, q, qstride);
-    else
-        k_gth<false><<<(unsigned)n, kGthThreads, smem, st>>>(g, ch, gorder, s0, q, qstride);
-    return cudaGetLastError();
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // Blocks per spectrum: the most that still run at once, where panels have enough rows to share (each block
+    // repeats a panel's serial part, so narrow ones gain nothing).
+    int C = 1;
+    if (rw >= 32)
+        while (C < 8 && n * C * 2 <= sms) C *= 2;
+    const int rcap = std::min(kGthRows, (rw + 2 * C - 1) / (2 * C) * 2);
+    const size_t smem = gth_smem_bytes(g.max_bins, rcap, cw);
+    const void* fn = C > 1 ? (const void*)k_gth<true> : (const void*)k_gth<false>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3((unsigned)(n * C));
+    lc.blockDim = dim3(kGthThreads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)C;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    lc.attrs = &at;
+    lc.numAttrs = C > 1 ? 1 : 0;
+    return C > 1 ? cudaLaunchKernelEx(&lc, k_gth<true>, g, ch, gorder, env, rcap, cw, C, s0, q, qstride)
+                 : cudaLaunchKernelEx(&lc, k_gth<false>, g, ch, gorder, env, rcap, cw, C, s0, q, qstride);
 }
 
 }  // namespace heat
