@@ -308,9 +308,9 @@ cudaError_t launch_td_env(const GrainDev& g, const double* D, const long long* d
 }
 
 // Shared memory of k_td_fill for a grid of N wavelengths, per segment: the cell's A = Omega_n lambda_n^2 dln / h,
-// Z = (slope + 2) dln in Q60 (kNoQ60: |Z| >= 1), R = E1(Z) in Q60 (kNoQ60: the bits of the whole segment's integral), and
-// the suffix sums of the integrals of Omega.
-size_t td_fill_smem_bytes(int N) { return 32 * (size_t)N; }
+// Z = (slope + 2) dln in Q60 (kNoQ60: |Z| >= 1), the segment's integral W = A E1(Z) and the suffix sums of the integrals of
+// Omega; and the sums of W over aligned blocks of 8 segments.
+size_t td_fill_smem_bytes(int N) { return 32 * (size_t)N + 8 * (((size_t)N + 7) / 8); }
 constexpr int64_t kNoQ60 = INT64_MIN;
 
 // Spectrum of block b of a launch that starts at spectrum s0: grains in the order `gorder`
@@ -332,11 +332,12 @@ __device__ __forceinline__ void td_spectrum(const ChunkDev& ch, const int* gorde
 // power of the photons too soft to leave bin i, c int_{lambda > hc/(Elo_j - E_i)} Omega,
 // over E_j - E_i.  The window's edges are the band's transition wavelengths (j + 1, i) and (j, i), whose places on
 // the grid do not depend on the cell (edge table).  A row's windows tile the grid: each is its
-// partial end segments plus the segment integrals between them (summed, not differenced; inside one segment
+// partial end segments plus the segment integrals between them (summed, by eights, not differenced; inside one segment
 // a difference of two Q60 values, exact to 2^-58 of the segment); the soft term is its partial segment plus
 // a suffix sum.  A warp per row, a lane per j; neighbouring lanes share their window edge, so a window costs one
 // fixed-point E1 (seg64.cuh).  With the edges and each partial segment's logarithms and exponentials in FP64
-// the fill was bound by the FP64 unit (83 % busy): 8 cells x 64 grains x 1024 wavelengths 8.7 ms, now 2.0 ms.
+// the fill was bound by the FP64 unit (83 % busy): 8 cells x 64 grains x 1024 wavelengths 8.7 ms, then
+// 2.0 ms, bound by the lanes whose window spans a hundred segments; with the sums by eights 0.64 ms.
 __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const double* __restrict__ Dt,
                                                  const long long* __restrict__ doff, const int* __restrict__ gorder,
                                                  const TdEdge* __restrict__ edge, const int4* __restrict__ env,
@@ -348,12 +349,13 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
     const int N = gd.N;
     double* A = fsm;
     int64_t* Z = (int64_t*)(A + N);
-    int64_t* R = Z + N;
-    double* S0 = (double*)(R + N);
+    double* W = (double*)(Z + N);
+    double* S0 = W + N;
+    double* W8 = S0 + N;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     for (int n = tid; n < N; n += blockDim.x) {
-        double a = 0.0, i0 = 0.0;
-        int64_t z = 0, r = kQ60;
+        double a = 0.0, i0 = 0.0, w = 0.0;
+        int64_t z = 0;
         if (n < N - 1) {
             const size_t gn = (size_t)g * N + n;
             const double ua = ch.ua64[(size_t)n * ch.Cc + cell], su = ch.su64[(size_t)n * ch.Cc + cell];
@@ -364,10 +366,10 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
                 const int cls = e1_class(zd);
                 if (cls) {
                     z = to_q60(zd);
-                    r = e1_q60(cls, z);
+                    w = a * from_q60(e1_q60(cls, z));
                 } else {
                     z = kNoQ60;
-                    r = __double_as_longlong(a * e1d(zd));
+                    w = a * e1d(zd);
                 }
             } else {
                 a = 0.0;
@@ -375,10 +377,15 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
         }
         A[n] = a;
         Z[n] = z;
-        R[n] = r;
+        W[n] = w;
         S0[n] = i0;
     }
     __syncthreads();
+    for (int b = tid; b < (N + 7) / 8; b += blockDim.x) {
+        double w = 0.0;
+        for (int n = 8 * b; n < min(N, 8 * b + 8); ++n) w += W[n];
+        W8[b] = w;
+    }
     if (warp == 0) {  // suffix sums of the segment integrals of Omega, S0[n] = sum_{m >= n}
         const int per = (N + 31) / 32, b0 = lane * per, b1 = min(N, b0 + per);
         double part = 0.0;
@@ -410,8 +417,15 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
         const int64_t az = z < 0 ? -z : z;
         return mul_q60(tau, e1_q60(az < (kQ60 >> 4) ? 3 : az < (kQ60 >> 2) ? 2 : 1, mul_q60(z, tau)));
     };
-    auto whole = [&](int n) {
-        return Z[n] == kNoQ60 ? __longlong_as_double(R[n]) : A[n] * from_q60(R[n]);
+    // sum of the whole segments n0 .. n1 - 1
+    auto wholes = [&](int n0, int n1) {
+        double v = 0.0;
+        int n = n0;
+        for (; n < n1 && (n & 7); ++n) v += W[n];
+#pragma unroll 4
+        for (; n + 8 <= n1; n += 8) v += W8[n >> 3];
+        for (; n < n1; ++n) v += W[n];
+        return v;
     };
     // integral between offsets ta and tb of segment n (r: upto() of both)
     auto between = [&](int n, double ta, double tb, int64_t ra, int64_t rb) {
@@ -470,8 +484,7 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
                     if (a.n == b.n) {
                         if (b.n < N - 1) v = between(b.n, a.t, b.t, ra, rb);
                     } else {
-                        v = between(a.n, a.t, gd.dln[a.n], ra, R[a.n]);
-                        for (int n = a.n + 1; n < b.n; ++n) v += whole(n);
+                        v = between(a.n, a.t, gd.dln[a.n], ra, upto(a.n, kQ60)) + wholes(a.n + 1, b.n);
                         if (b.n < N - 1) v += between(b.n, 0.0, b.t, 0, rb);
                     }
                 }
