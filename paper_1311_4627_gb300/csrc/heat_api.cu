@@ -246,10 +246,29 @@ static void order_grains(heat_ctx* ctx) {
     ctx->tail_NG = -1;
 }
 
-// (grain, group) task lists of a chunk of NG groups: the recursion's order, then the build's.
+// Grains whose recursion takes the four warps of a block per task instead of one (chunks of NG groups): those that a
+// warp alone would be busy with for more than a third of what bounds the launch, the FP64 units' 64 cycles per element
+// and four per row or the warps' time (20 a SM; alone, 150 cycles per element and 1300 per row).  Four warps
+// spend more per element on barriers and narrow rows, so a launch with enough tasks leaves grains to single
+// warps: 4096 cells x 64 grains, none 6.12 ms, a half 6.14, a third 6.10, a quarter 6.8, all 7.6; 4096 cells x 32 grains of
+// 512 bins, none 12.8, the whole 8.6, a half 7.0, a third 6.9, a quarter 6.6, all 6.9.
+static std::vector<char> quad_grains(const heat_ctx* ctx, int NG) {
+    std::vector<char> quad(ctx->G, 0);
+    double fp64 = 0.0, warps = 0.0;
+    auto alone = [&](int g) { return 150.0 * (double)ctx->grain_band[g] + 1300.0 * (double)ctx->grain_rows[g]; };
+    for (int g = 0; g < ctx->G; ++g) {
+        fp64 += 64.0 * (double)(ctx->grain_band[g] + 4LL * ctx->grain_rows[g]);
+        warps += alone(g);
+    }
+    const double bound = std::max(fp64 / 4.0, warps / 20.0) * NG / ctx->sms;
+    for (int g = 0; g < ctx->G; ++g) quad[g] = 3.0 * alone(g) > bound;
+    return quad;
+}
+
+// (grain, group) task lists of a chunk of NG groups: the fused kernel's order, the build's, the recursion's.
 static std::vector<int2> make_tasks(const heat_ctx* ctx, int NG) {
     std::vector<int2> tasks;
-    tasks.reserve(2 * (size_t)ctx->G * NG);
+    tasks.reserve(3 * (size_t)ctx->G * NG);
     // recursion: near-chain grains (fewer than 8 band elements per row: their time is the
     // per-row latency, they hardly use the FP64 unit) interleaved with the wide-band grains
     // in proportion to each list's cost, so that every SM holds both kinds throughout
@@ -260,14 +279,21 @@ static std::vector<int2> make_tasks(const heat_ctx* ctx, int NG) {
     for (int g : chain) tc += cost(g);
     for (int g : wide) tw += cost(g);
     size_t ic = 0, iw = 0;
+    std::vector<int> mixed;
     while (ic < chain.size() || iw < wide.size()) {
         const bool take_chain = iw == wide.size() || (ic < chain.size() && dc / tc <= dw / tw);
         const int g = take_chain ? chain[ic++] : wide[iw++];
         (take_chain ? dc : dw) += cost(g);
+        mixed.push_back(g);
         for (int grp = 0; grp < NG; ++grp) tasks.push_back(make_int2(g, grp));
     }
     for (int gi = 0; gi < ctx->G; ++gi)
         for (int grp = 0; grp < NG; ++grp) tasks.push_back(make_int2(ctx->grain_order_build[gi], grp));
+    const std::vector<char> quad = quad_grains(ctx, NG);
+    for (const char q : {1, 0})
+        for (int g : q ? ctx->grain_order : mixed)
+            if (quad[g] == q)
+                for (int grp = 0; grp < NG; ++grp) tasks.push_back(make_int2(g, grp));
     return tasks;
 }
 
@@ -1050,6 +1076,10 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
         ch.tasks = (ch.NG == NG ? ctx->s_tasks : ctx->s_tasks_tail).as<int2>();
         ch.btasks = ch.tasks + (size_t)G * ch.NG;
         ch.n_tasks = G * ch.NG;
+        ch.rtasks = ch.btasks + (size_t)G * ch.NG;
+        ch.n_quad = 0;
+        for (const char q : quad_grains(ctx, ch.NG)) ch.n_quad += q ? ch.NG : 0;
+        ch.sms = ctx->sms;
         ch.ua64 = sl.ua64.as<double>();
         ch.su64 = sl.su64.as<double>();
         ch.ua32 = sl.ua32.as<float>();

@@ -84,6 +84,10 @@ struct ChunkDev {
     const int2* tasks;  // [G * NG] (grain, group), largest work first (recursion order)
     const int2* btasks; // the same pairs in the build's order, or null (then `tasks`)
     int n_tasks;
+    // the recursion's tasks: grains with wide rows, a block each (the first n_quad), then the rest, a warp each
+    const int2* rtasks;
+    int n_quad;
+    int sms;            // SMs of the device (with `work`)
     // field tables, transposed [N][Cc]
     double* ua64; double* su64;
     float* ua32; float* su32;  // FP32 build: su32 unused; ua32 holds float2 (u_n, su_n) pairs

@@ -1,6 +1,6 @@
 // The Guhathakurta-Draine recursion (Eq. xf) and renormalisation (Eq. renormalization) over
-// the B band that the build wrote: a persistent lane-per-cell kernel (warp = grain x 32 cells,
-// one FP64 FMA per band element and cell, no divergence, no cross-lane reductions) and a
+// the B band that the build wrote: a persistent lane-per-cell kernel (a warp, or the four warps of a block, per grain x
+// 32 cells, one FP64 FMA per band element and cell, no divergence, no cross-lane reductions) and a
 // warp-per-spectrum column sweep for solves of few cells.
 #include <algorithm>
 
@@ -121,24 +121,25 @@ __device__ __forceinline__ void window_tail(int nreg, const typename BandRaw<BUI
 // the energy check (returned), and packed for the tensor cores exactly as k_pack_p packs a P
 // row: row scale 2^e from the row's largest P (its running maximum, normalised), then each P
 // divided by 2^e, rounded to FP32 and split into hi + lo, eight bins per 16-byte store (each
-// lane writes its own cell's row).
+// lane writes its own cell's row).  Part `part` of `parts` takes every parts-th store; the energy check's sum, in
+// ascending order, is then left to energy_sum.
 __device__ __noinline__ double pack_epilogue(const GrainDev& gd, const ChunkDev& ch, int g, int cc, int M, int i_end,
                                              double inv, int epoch, long long xmaxb, const double* xl,
-                                             const unsigned short* epl) {
+                                             const unsigned short* epl, int part, int parts) {
     const int off = gd.bin_off[g];
     double* prow = ch.P ? ch.P + (size_t)cc * ch.ldP + off : nullptr;
     const double* cde = gd.cde + off;
     double emit = 0.0;
     const int e = row_scale_exp((unsigned)__double2hiint(__longlong_as_double(xmaxb) * inv));
-    ch.pack_rowscale[(size_t)cc * gd.G + g] = ldexpf(1.0f, e);
+    if (part == 0) ch.pack_rowscale[(size_t)cc * gd.G + g] = ldexpf(1.0f, e);
     const int K = ch.pack_kp[g], half = ch.pack_split ? K / 2 : K;
-    const bool ledger = ch.ledger != nullptr;
+    const bool ledger = ch.ledger != nullptr && parts == 1;
     auto p_of = [&](int i) {
         return i <= i_end ? scale_down_800(xl[i * 32], epoch - (int)epl[i * 32]) * inv : 0.0;
     };
     if (ch.pack_tf32) {
         float* row = (float*)ch.packA + ch.pack_aoff[g] + (size_t)cc * K;
-        for (int i0 = 0; i0 < half; i0 += 4) {
+        for (int i0 = 4 * part; i0 < half; i0 += 4 * parts) {
             float4 h, l;
             float* hv = &h.x;
             float* lv = &l.x;
@@ -157,7 +158,7 @@ __device__ __noinline__ double pack_epilogue(const GrainDev& gd, const ChunkDev&
         }
     } else {
         uint16_t* row = (uint16_t*)ch.packA + ch.pack_aoff[g] + (size_t)cc * K;
-        for (int i0 = 0; i0 < half; i0 += 8) {
+        for (int i0 = 8 * part; i0 < half; i0 += 8 * parts) {
             uint4 h, l;
             unsigned* hv = &h.x;
             unsigned* lv = &l.x;
@@ -184,6 +185,52 @@ __device__ __noinline__ double pack_epilogue(const GrainDev& gd, const ChunkDev&
         }
     }
     return emit;
+}
+
+// The power emitted by the probabilities P_i = X_i / sum X of rows 0 .. i_end, summed in ascending order.
+__device__ __forceinline__ double energy_sum(const double* cde, int i_end, double inv, int epoch, const double* xl,
+                                             const unsigned short* epl) {
+    double emit = 0.0;
+    for (int i = 0; i <= i_end; ++i) emit = fma(scale_down_800(xl[i * 32], epoch - (int)epl[i * 32]) * inv, cde[i], emit);
+    return emit;
+}
+
+// The end of a task: normalisation, P (or the packed emissivity operand) and the energy check of rows 0 .. i_end (P = 0
+// above, with tail pruning); part `part` of `parts` warps that share the rows.
+__device__ __forceinline__ void finish_task(const GrainDev& gd, const ChunkDev& ch, int g, int cc, int M, int i_end,
+                                            bool pruned, double total, int epoch, long long xmaxb, const double* xl,
+                                            const unsigned short* epl, int part, int parts) {
+    if (cc >= ch.cells) return;
+    const int off = gd.bin_off[g];
+    const double inv = 1.0 / total;
+    const double* cde = gd.cde + off;
+    double emit = 0.0;
+    if (ch.packA) {
+        emit = pack_epilogue(gd, ch, g, cc, M, i_end, inv, epoch, xmaxb, xl, epl, part, parts);
+    } else {
+        double* prow = ch.P + (size_t)cc * ch.ldP + off;
+        // scale X first (as the plain rescale would have), then normalise: the factor alone
+        // could underflow where the product is still a normal number.  Two loops, so that
+        // no predicated-off FMA of the energy check occupies the FP64 unit without a ledger
+        if (ch.ledger && parts == 1) {
+            for (int i = 0; i <= i_end; ++i) {
+                const double p = scale_down_800(xl[i * 32], epoch - (int)epl[i * 32]) * inv;
+                prow[i] = p;
+                emit = fma(p, cde[i], emit);
+            }
+        } else {
+            for (int i = part; i <= i_end; i += parts)
+                prow[i] = scale_down_800(xl[i * 32], epoch - (int)epl[i * 32]) * inv;
+        }
+        if (pruned)
+            for (int i = i_end + 1 + part; i <= M; i += parts) prow[i] = 0.0;  // rows past a pruned tail
+    }
+    if (ch.ledger && part == 0) {
+        if (parts > 1) emit = energy_sum(cde, i_end, inv, epoch, xl, epl);
+        double* lg = ch.ledger + ((size_t)cc * gd.G + g) * 2;
+        lg[0] = ch.pabs[(size_t)cc * gd.G + g];
+        lg[1] = emit;
+    }
 }
 
 // One task: the recursion of grain g for the 32 cells of group grp (lane = cell).  W is
@@ -378,47 +425,211 @@ __device__ __forceinline__ void recur_task(const GrainDev& gd, const ChunkDev& c
 #pragma unroll
         for (int k = 0; k < W; ++k) br[k] = br_n[k];
     }
-    if (cc < ch.cells && ch.packA) {
-        const double inv = 1.0 / total;
-        const double emit = pack_epilogue(gd, ch, g, cc, M, PRUNE ? f_last : M, inv, epoch, xmaxb, xl, epl);
-        if (ch.ledger) {
-            double* lg = ch.ledger + ((size_t)cc * gd.G + g) * 2;
-            lg[0] = ch.pabs[(size_t)cc * gd.G + g];
-            lg[1] = emit;
-        }
-    } else if (cc < ch.cells) {
-        const double inv = 1.0 / total;
-        double* prow = ch.P + (size_t)cc * ch.ldP + off;
-        double emit = 0.0;
-        const double* cde = gd.cde + off;
-        const int i_end = PRUNE ? f_last : M;
-        // scale X first (as the plain rescale would have), then normalise: the factor alone
-        // could underflow where the product is still a normal number.  Two loops, so that
-        // no predicated-off FMA of the energy check occupies the FP64 unit without a ledger
-        if (ch.ledger) {
-            for (int i = 0; i <= i_end; ++i) {
-                const double p = scale_down_800(xl[i * 32], epoch - (int)epl[i * 32]) * inv;
-                prow[i] = p;
-                emit = fma(p, cde[i], emit);
-            }
-        } else {
-            for (int i = 0; i <= i_end; ++i) prow[i] = scale_down_800(xl[i * 32], epoch - (int)epl[i * 32]) * inv;
-        }
-        if constexpr (PRUNE)
-            for (int i = f_last + 1; i <= M; ++i) prow[i] = 0.0;  // rows past a pruned tail
-        if (ch.ledger) {
-            double* lg = ch.ledger + ((size_t)cc * gd.G + g) * 2;
-            lg[0] = ch.pabs[(size_t)cc * gd.G + g];
-            lg[1] = emit;
-        }
-    }
+    finish_task(gd, ch, g, cc, M, PRUNE ? f_last : M, PRUNE, total, epoch, xmaxb, xl, epl, 0, 1);
     if (numeric_bad) atomicOr(ch.status, kStatNumeric);
 }
 
+// One task of a grain with wide rows, by the block's four warps: rows in blocks of four, a warp per row, so that a row's
+// chain of multiply-adds runs on its own FP64 unit beside the other three rows'.  Columns before the block's first
+// row are summed at once; the block's own columns follow row by row, each X through shared memory (at most three
+// multiply-adds a row, a barrier per row).  Each row's sum has recur_task's order, so P has the same bits.
+//
+// A warp alone takes 130 to 180 cycles per element (two batches of loads in flight against 64 cycles of the FP64
+// unit), so the widest grain of a launch was the launch: a grain of 512 bins all of which reach each other 9.1 ms at any
+// number of cells.  Four units shorten that chain four times and leave the FP64 units' total (64 cycles per element)
+// as the bound.  Recursion before and now: 32 grains of 512 bins, 4096 cells 12.8 -> 6.9 ms; 37 grains, 1003 cells 2.0 ->
+// 1.4; FP64, 512 cells x 64 grains 3.1 -> 1.4, 203 cells x 19 grains (point rule's field) 2.8 -> 0.6.  Which grains: quad_grains
+// (heat_api.cu).
+template <int BUILD, bool PRUNE>
+__device__ __noinline__ void recur_quad(const GrainDev& gd, const ChunkDev& ch, int g, int grp, int lane, int w,
+                                           double (&xs)[4][32]) {
+    using Raw = BandRaw<BUILD>;
+    const int nbt = gd.nbt;
+    const int off = gd.bin_off[g];
+    const int M = gd.bin_off[g + 1] - off - 1;
+    const int cc = grp * 32 + lane;
+    const size_t xb = ((size_t)grp * nbt + off) * 32 + lane;
+    const int* rp = gd.rowptr + off + g;
+    const double* ic_row = gd.invC + off;
+    double* xl = ch.xs + xb;
+    unsigned short* epl = ch.ep + xb;
+    const size_t bb = (size_t)grp * gd.band_total * 32 + lane;
+    const float* __restrict__ B32 = ch.Bb32 + (BUILD ? bb : 0);
+    const double* __restrict__ B64 = ch.Bb64 + (BUILD ? 0 : bb);
+    const size_t lane_base = bb - lane;
+    bool numeric_bad = false;
+    int epoch = 0;
+    if (w == 0) {
+        xl[0] = 1.0;
+        epl[0] = 0;
+    }
+    double total = 1.0;                                // warp 0's, as xmaxb
+    long long xmaxb = __double_as_longlong(1.0);
+    const int* kx = gd.kexp + off;
+    int xmax = 1023, cmax = 0, last_big = 0, f_last = M;
+    bool stopped = false;
+    if constexpr (PRUNE) cmax = 1023 + kx[0];
+    __syncthreads();
+    int f = 1 + w;
+    int e = f <= M ? rp[f] : 0, e1 = f <= M ? rp[f + 1] : 0;
+    double ic = f <= M ? ic_row[f] : 0.0;
+    for (int f0 = 1; f0 <= M; f0 += 4, f += 4) {
+        // the next block's bounds
+        const int en = f + 4 <= M ? rp[f + 4] : 0, en1 = f + 4 <= M ? rp[f + 5] : 0;
+        const double ic_n = f + 4 <= M ? ic_row[f + 4] : 0.0;
+        const int jb = f - (e1 - e), nbulk = f0 - jb;  // columns jb .. f0 - 1 (none if negative)
+        typename Raw::T bt[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) bt[i] = (f <= M && i < w && f0 + i >= jb) ? Raw::load(B32, B64, e + f0 + i - jb) : 0;
+        double S = 0.0;
+        if (f <= M && nbulk > 0) {
+            int j = jb, q = e;
+            const int rem = nbulk & 3, nb = nbulk >> 2;
+            typename Raw::T bR[3], bA[4], bB[4];
+            double xR[3], xA[4], xB[4];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                bR[k] = k < rem ? Raw::load(B32, B64, q + k) : 0;
+                xR[k] = k < rem ? xl[(j + k) * 32] : 0.0;
+            }
+            q += rem;
+            j += rem;
+            if (nb > 0) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) bA[k] = Raw::load(B32, B64, q + k);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) xA[k] = xl[(j + k) * 32];
+            }
+            // L2 prefetch, lane = element: the row's first elements of the next block, then 32 ahead in this row
+            if (f + 4 <= M && en + lane < en1) {
+                const void* a = BUILD ? (const void*)(ch.Bb32 + lane_base + (size_t)(en + lane) * 32)
+                                      : (const void*)(ch.Bb64 + lane_base + (size_t)(en + lane) * 32);
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
+            }
+            if (rem > 0) S = fma(Raw::wide(bR[0]), xR[0], S);
+            if (rem > 1) S = fma(Raw::wide(bR[1]), xR[1], S);
+            if (rem > 2) S = fma(Raw::wide(bR[2]), xR[2], S);
+            int i = 0;
+            for (; i + 2 <= nb; i += 2) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) bB[k] = Raw::load(B32, B64, q + 4 + k);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) xB[k] = xl[(j + 4 + k) * 32];
+                if (lane < 8 && q + 32 + lane < e1) {
+                    const void* a = BUILD ? (const void*)(ch.Bb32 + lane_base + (size_t)(q + 32 + lane) * 32)
+                                          : (const void*)(ch.Bb64 + lane_base + (size_t)(q + 32 + lane) * 32);
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) S = fma(Raw::wide(bA[k]), xA[k], S);
+                if (i + 2 < nb) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) bA[k] = Raw::load(B32, B64, q + 8 + k);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) xA[k] = xl[(j + 8 + k) * 32];
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) S = fma(Raw::wide(bB[k]), xB[k], S);
+                q += 8;
+                j += 8;
+            }
+            if (i < nb) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) S = fma(Raw::wide(bA[k]), xA[k], S);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (f0 + r > M) break;
+            double X = 0.0;
+            if (w == r) {
+                X = S * ic;
+                if (__double2hiint(ic) == 0 && __double2loint(ic) == 0) {  // zero cooling rate
+                    X = 0.0;
+                    if (__double_as_longlong(S) != 0 && !(PRUNE && stopped)) numeric_bad = true;
+                }
+                if (PRUNE && stopped) X = 0.0;
+                xl[f * 32] = X;
+                epl[f * 32] = (unsigned short)epoch;
+                xs[r][lane] = X;
+            }
+            const bool up = __syncthreads_or(w == r && above_rescale(X));
+            X = xs[r][lane];
+            if constexpr (PRUNE) {  // as recur_task, in every warp
+                if (!stopped) {
+                    const int L = ch.prune, fr = f0 + r;
+                    const int xe = ((__double2hiint(X) >> 20) & 0x7ff) + 800 * epoch;
+                    const int ce = xe + kx[fr];
+                    xmax = max(xmax, xe);
+                    cmax = max(cmax, ce);
+                    if (!(xe < xmax - L && ce < cmax - L)) last_big = fr;
+                    stopped = last_big < fr - (rp[fr + 1] - rp[fr]);
+                }
+            }
+            if (w == 0) {
+                total += X;
+                xmaxb = max(xmaxb, __double_as_longlong(X));
+            }
+            if (r < 3 && w > r && f0 + r >= jb) S = fma(Raw::wide(bt[r < 3 ? r : 0]), X, S);
+            if (up) {  // a cell of the task is above 2^800
+                if (above_rescale(X)) {
+                    ++epoch;
+                    xmaxb = __double_as_longlong(scale_down_800(__longlong_as_double(xmaxb), 1));
+                    total = scale_down_800(total, 1);
+                    S = scale_down_800(S, 1);
+                    // what later blocks read from memory, a quarter of it per warp
+                    const int lo = f0 + 4 <= M ? f0 + 4 - (rp[f0 + 5] - rp[f0 + 4]) : f0 + r + 1;
+                    for (int i = lo + w; i <= f0 + r; i += 4) {
+                        xl[i * 32] = scale_down_800(xl[i * 32], 1);
+                        epl[i * 32] = (unsigned short)epoch;
+                    }
+                }
+                __syncthreads();
+            }
+        }
+        if constexpr (PRUNE) {
+            if (__all_sync(0xffffffffu, stopped)) {
+                f_last = min(f0 + 3, M);
+                break;
+            }
+        }
+        e = en;
+        e1 = en1;
+        ic = ic_n;
+    }
+    __syncthreads();
+    if (w == 0) {
+        xs[0][lane] = total;
+        xs[1][lane] = __longlong_as_double(xmaxb);
+    }
+    __syncthreads();
+    total = xs[0][lane];
+    xmaxb = __double_as_longlong(xs[1][lane]);
+    finish_task(gd, ch, g, cc, M, PRUNE ? f_last : M, PRUNE, total, epoch, xmaxb, xl, epl, w, 4);
+    if (numeric_bad) atomicOr(ch.status, kStatNumeric);
+}
+
+// Resident blocks per SM that take the single warps' tasks first, and only then the four-warp ones: narrow rows wait on
+// their loads and leave the FP64 unit to the wide ones beside them.  32 grains of 512 bins, 4096 cells: 0 9.0 ms, 1 7.4,
+// 2 6.9, 3 6.9.
+constexpr int kSinglesFirst = 2;
 template <int BUILD, bool PRUNE>
 __global__ void __launch_bounds__(128, 5) k_recur(GrainDev gd, ChunkDev ch) {
-    for_each_task(ch, 1, [&](int task, int lane) {
-        const int g = ch.tasks[task].x, grp = ch.tasks[task].y;
+    __shared__ double xs[4][32];
+    __shared__ int next;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto quads = [&] {
+        for (;;) {
+            __syncthreads();
+            if (threadIdx.x == 0) next = atomicAdd(ch.work, 1);
+            __syncthreads();
+            const int task = next;
+            if (task >= ch.n_quad) return;
+            recur_quad<BUILD, PRUNE>(gd, ch, ch.rtasks[task].x, ch.rtasks[task].y, lane, w, xs);
+        }
+    };
+    auto singles = [&](int task) {
+        const int g = ch.rtasks[task].x, grp = ch.rtasks[task].y;
         // window classes 1, 2 and 4 (warp-uniform).  Measured on the batched workload: a class
         // of 8 for rows wider than 4 spilled at the 96 registers of 5 resident blocks (6.26 ms
         // against 6.04-6.10 with 4 the widest; widest 3 or 5 the same, 6 6.33, 7 7.25 ms)
@@ -429,7 +640,22 @@ __global__ void __launch_bounds__(128, 5) k_recur(GrainDev gd, ChunkDev ch) {
             recur_task<BUILD, 2, PRUNE>(gd, ch, g, grp, lane);
         else
             recur_task<BUILD, 4, PRUNE>(gd, ch, g, grp, lane);
-    });
+    };
+    if (!ch.work) {  // a warp per task
+        const int task = blockIdx.x * 4 + w;
+        if (task < ch.n_tasks) singles(task);
+        return;
+    }
+    const bool singles_first = ch.n_quad == 0 || (int)(blockIdx.x / ch.sms) < kSinglesFirst;
+    if (!singles_first) quads();
+    for (;;) {
+        int task = 0;
+        if (lane == 0) task = ch.n_quad + atomicAdd(ch.work + 1, 1);
+        task = __shfl_sync(0xffffffffu, task, 0);
+        if (task >= ch.n_tasks) break;
+        singles(task);
+    }
+    if (singles_first && ch.n_quad > 0) quads();
 }
 
 // ---------------------------------------------------------------------------
@@ -815,8 +1041,8 @@ __global__ void __launch_bounds__(THREADS, THREADS > 256 ? 1 : 2) k_recur_chain(
 // the persistent launches (ch.work set), no more than stay resident on the device at once.
 template <typename K>
 static unsigned task_grid(K kernel, const ChunkDev& ch) {
-    const unsigned full = (unsigned)((ch.n_tasks + 3) / 4);
-    if (!ch.work) return full;
+    if (!ch.work) return (unsigned)((ch.n_tasks + 3) / 4);
+    const unsigned full = (unsigned)(ch.n_quad + (ch.n_tasks - ch.n_quad + 3) / 4);
     int dev = 0, sms = 0, occ = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||

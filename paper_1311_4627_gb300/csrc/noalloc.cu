@@ -132,6 +132,7 @@ extern "C" heat_status heat_solve_noalloc(heat_ctx* ctx, int build, const double
         ch.n_tasks = G * NG;
         int2* tasks = (int2*)take(sizeof(int2) * (size_t)G * NG);
         ch.tasks = tasks;
+        ch.rtasks = tasks;
         if (build == HEAT_BUILD_F64) {
             ch.ua64 = (double*)take(sizeof(double) * (size_t)N * Cc);
             ch.su64 = (double*)take(sizeof(double) * (size_t)N * Cc);
