@@ -6,7 +6,7 @@
 // The GEMM reuses the warp-specialised layout of the emissivity kernel: warp 0 issues
 // TMA loads into a 6-stage ring, warp 1 issues tcgen05.mma (M = 128, N = 128), warps 2..9
 // drain the double-buffered TMEM accumulators (two warps per lane quadrant, each half of the
-// columns: the epilogue's GELU and stores, not the MMAs, bound the hidden layers).  Every
+// columns: the epilogue, not the MMAs, bounds the layers).  Every
 // mbarrier wait is bounded.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -55,7 +55,8 @@ __global__ void __launch_bounds__(64 + 32 * gEpiWarps, 1) k_gemm_bf16(const __gr
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* sA = smem;
     unsigned char* sB = smem + gStages * gAStage;
-    uint64_t* bars = (uint64_t*)(sB + gStages * gBStage);
+    uint4* const stage_all = (uint4*)(sB + gStages * gBStage);  // 4 KB per epilogue warp
+    uint64_t* bars = (uint64_t*)(stage_all + gEpiWarps * 256);
     uint32_t* tmem_slot = (uint32_t*)(bars + 2 * gStages + 5);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
@@ -172,6 +173,7 @@ __global__ void __launch_bounds__(64 + 32 * gEpiWarps, 1) k_gemm_bf16(const __gr
         // epilogue: lane = row of the tile; each chunk of 32 columns gets its bias (broadcast
         // loads), optional GELU for the BF16 output, and 16-byte stores of the row's run
         const int q = warp & 3;                          // the TMEM lane quadrant this warp may read
+        uint4* const stage = stage_all + (warp - 2) * 256;
         const int c0 = ((warp - 2) >> 2) * (gN / 64);    // its half of the tile's 32-column chunks
         int acc = 0;
         uint32_t acc_phase = 0;
@@ -213,19 +215,37 @@ __global__ void __launch_bounds__(64 + 32 * gEpiWarps, 1) k_gemm_bf16(const __gr
                         val[4 * k + 2] = __uint_as_float(v[4 * k + 2]) + b4.z;
                         val[4 * k + 3] = __uint_as_float(v[4 * k + 3]) + b4.w;
                     }
-                    if (rok && crow) {
+                    // FP32 through shared memory, so that a store instruction writes four whole lines and not 16 bytes
+                    // of 32 rows (16-byte pieces, rotated by row against bank conflicts): four members' 65536 x
+                    // 1024 outputs 507 -> 334 us.  The same for the BF16 outputs, half the bytes, gained nothing (hidden
+                    // layers 208 us either way, the first, K = 64, 127 -> 177), nor did 16 epilogue warps.
+                    if (C) {
+                        const int row0 = mt * gM + q * 32;
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            stage[lane * 8 + (k ^ (lane & 7))] =
+                                make_uint4(__float_as_uint(val[4 * k]), __float_as_uint(val[4 * k + 1]),
+                                           __float_as_uint(val[4 * k + 2]), __float_as_uint(val[4 * k + 3]));
+                        __syncwarp();
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
-                            float4 o = make_float4(val[4 * k], val[4 * k + 1], val[4 * k + 2], val[4 * k + 3]);
-                            if (p.accumulate) {
-                                const float4 old = ((const float4*)crow)[k];
-                                o.x += old.x;
-                                o.y += old.y;
-                                o.z += old.z;
-                                o.w += old.w;
+                            const int r = 4 * k + (lane >> 3), pc = lane & 7;
+                            const uint4 u = stage[r * 8 + (pc ^ (r & 7))];
+                            float4 o = make_float4(__uint_as_float(u.x), __uint_as_float(u.y), __uint_as_float(u.z),
+                                                   __uint_as_float(u.w));
+                            float4* dst = (float4*)(C + (size_t)(row0 + r) * p.ldc + col0) + pc;
+                            if (row0 + r < p.M) {
+                                if (p.accumulate) {
+                                    const float4 old = *dst;
+                                    o.x += old.x;
+                                    o.y += old.y;
+                                    o.z += old.z;
+                                    o.w += old.w;
+                                }
+                                *dst = o;
                             }
-                            ((float4*)crow)[k] = o;
                         }
+                        __syncwarp();
                     }
                     if (rok && brow) {
 #pragma unroll
@@ -277,7 +297,7 @@ __global__ void __launch_bounds__(64 + 32 * gEpiWarps, 1) k_gemm_bf16(const __gr
 }
 
 size_t gemm_bf16_smem_bytes() {
-    return 1024 + (size_t)gStages * (gAStage + gBStage) + (2 * gStages + 5) * 8 + 16;
+    return 1024 + (size_t)gStages * (gAStage + gBStage) + gEpiWarps * 4096 + (2 * gStages + 5) * 8 + 16;
 }
 
 cudaError_t launch_gemm_bf16(const GemmTcParams& p, int sms, cudaStream_t st) {
