@@ -85,9 +85,9 @@ int segment_of(const std::vector<double>& lam, double x) {
 }
 
 // offset t in segment n as a fraction of the segment, in Q60 (0 outside the grid's segments)
-int64_t tau_q60(const std::vector<double>& lam, int n, double t) {
-    if (n < 0 || n + 1 >= (int)lam.size()) return 0;
-    const double tau = t / std::log(lam[n + 1] / lam[n]);
+int64_t tau_q60(const std::vector<double>& dln, int n, double t) {
+    if (n < 0 || n >= (int)dln.size()) return 0;
+    const double tau = t / dln[n];
     return (int64_t)(std::min(std::max(tau, 0.0), 1.0) * 0x1p60);
 }
 
@@ -441,6 +441,8 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
     std::vector<PatF64> pat64;
     std::vector<PatF32> pat32;
     std::vector<int> pat_seg;
+    std::vector<double> seg_dln(lam.size() > 1 ? lam.size() - 1 : 0);  // log widths of the segments
+    for (size_t n = 0; n < seg_dln.size(); ++n) seg_dln[n] = std::log(lam[n + 1] / lam[n]);
     std::vector<int> seg_ptr((size_t)G * (N + 1), 0);
     std::vector<int4> pieces, pseg, cpieces;
     std::vector<SoftF64> soft;
@@ -541,7 +543,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
                     pe.n = segment_of(lam, x);
                     pe.t = std::log(x / lam[pe.n]);
                     pe.fac = x * x * x * dE / (kHhost * kHhost * kChost);
-                    pe.tau = tau_q60(lam, pe.n, pe.t);
+                    pe.tau = tau_q60(seg_dln, pe.n, pe.t);
                 } else {
                     pe.n = -1;
                     pe.tau = 0;
@@ -583,7 +585,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
             a.e = en.e;
             a.j = en.diag - 1;
             a.t = en.t;
-            a.tau = tau_q60(lam, en.n, en.t);
+            a.tau = tau_q60(seg_dln, en.n, en.t);
             PatF32 b;
             b.e = en.e;
             b.t = (float)en.t;
@@ -617,7 +619,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
                 sf.n = segment_of(lam, ls);
                 sf.t = std::log(ls / lam[sf.n]);
             }
-            sf.tau = tau_q60(lam, sf.n, sf.t);
+            sf.tau = tau_q60(seg_dln, sf.n, sf.t);
             sg.push_back(sf);
         }
         std::stable_sort(sg.begin(), sg.end(), [](const SoftF64& a, const SoftF64& b) { return a.n > b.n; });
