@@ -22,6 +22,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "gth_tile.cuh"
 #include "internal.h"
 #include "seg64.cuh"
 
@@ -816,7 +817,7 @@ __global__ void __launch_bounds__(kGthThreads, 2) k_gth(GrainDev gd, ChunkDev ch
         const int low = in ? low_of(n) : nb;
 #pragma unroll
         for (int i = warp; i < 32; i += nw)
-            tile[i][lane] = i < lane && n0 + i >= low ? qs[(size_t)(n0 + i) * nb + n] : 0.0;
+            tile[i][lane] = gth_tile_in(i, lane, n0, nb, low) ? qs[(size_t)(n0 + i) * nb + n] : 0.0;
         __syncthreads();
         if (warp == 0) {
             double x = in ? X[n] : 0.0;
