@@ -880,7 +880,9 @@ __global__ void __launch_bounds__(THREADS, THREADS > 256 ? 1 : 2) k_recur_chain(
     using Raw = BandRaw<BUILD>;
     extern __shared__ double xs[];  // X history [max_bins]
     __shared__ double total_s;
-    __shared__ int event_s;  // rescales in the current run
+    // rescales in the current run; two slots in turn: a run without any has one barrier, which does not order the
+    // next run's write after this run's reads
+    __shared__ int event_s[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x, W = T >> 5;
     const int cell = blockIdx.x / gd.G, g = blockIdx.x % gd.G;
     const int grp = cell >> 5, lc = cell & 31;
@@ -918,7 +920,7 @@ __global__ void __launch_bounds__(THREADS, THREADS > 256 ? 1 : 2) k_recur_chain(
         a[k] = 0;
         c[k] = warp == 0 ? load(row, k) : 0;
     }
-    if (tid == 0) total_s = 0.0, event_s = 0;
+    if (tid == 0) total_s = 0.0, event_s[0] = event_s[1] = 0;
     __syncthreads();
     bool numeric_bad = false;
     const int runs = M / 8 + 1;
@@ -989,10 +991,10 @@ __global__ void __launch_bounds__(THREADS, THREADS > 256 ? 1 : 2) k_recur_chain(
 #pragma unroll
             for (int k = 0; k < 8; ++k) mine = lane == k ? x[k] : mine;
             if (lane < 8 && 8 * s + lane <= M) xs[8 * s + lane] = mine;
-            if (lane == 0) event_s = ev;
+            if (lane == 0) event_s[s & 1] = ev;
         }
         __syncthreads();
-        const int ev = event_s;
+        const int ev = event_s[s & 1];
         if (ev) {  // the rest of the block follows the chain's rescales
             if (!chain) acc = scale_down_800(acc, ev);
             for (int i = tid; i < 8 * s; i += T) xs[i] = scale_down_800(xs[i], ev);
