@@ -570,7 +570,6 @@ __device__ __noinline__ void recur_quad(const GrainDev& gd, const ChunkDev& ch, 
                 total += X;
                 xmaxb = max(xmaxb, __double_as_longlong(X));
             }
-            if (r < 3 && w > r && f0 + r >= jb) S = fma(Raw::wide(bt[r < 3 ? r : 0]), X, S);
             if (up) {  // a cell of the task is above 2^800
                 if (above_rescale(X)) {
                     ++epoch;
@@ -583,9 +582,12 @@ __device__ __noinline__ void recur_quad(const GrainDev& gd, const ChunkDev& ch, 
                         xl[i * 32] = scale_down_800(xl[i * 32], 1);
                         epl[i * 32] = (unsigned short)epoch;
                     }
+                    X = scale_down_800(X, 1);
                 }
                 __syncthreads();
             }
+            // (after the rescale: B X of the value before it could overflow)
+            if (r < 3 && w > r && f0 + r >= jb) S = fma(Raw::wide(bt[r < 3 ? r : 0]), X, S);
         }
         if constexpr (PRUNE) {
             if (__all_sync(0xffffffffu, stopped)) {
@@ -978,13 +980,14 @@ __global__ void __launch_bounds__(THREADS, THREADS > 256 ? 1 : 2) k_recur_chain(
                 const double X = __shfl_sync(0xffffffffu, acc * row.ic, f & 31);  // 0 for a zero cooling rate
                 if (icz && row.f == f && f <= M && __double_as_longlong(acc) != 0)
                     numeric_bad = true;  // zero cooling rate with inflow (acc >= 0)
+                const double before = acc;
                 acc = fma(cd[k], X, acc);  // (elements outside a row's band are 0)
                 x[k] = X;
-                if (above_rescale(X)) {
+                if (above_rescale(X)) {  // rare: the sum again, on scaled values (B X could have overflowed)
                     ++ev;
-                    acc = scale_down_800(acc, 1);
 #pragma unroll
                     for (int i = 0; i <= k; ++i) x[i] = scale_down_800(x[i], 1);
+                    acc = fma(cd[k], x[k], scale_down_800(before, 1));
                 }
             }
             double mine = 0.0;  // lane k stores the run's k-th X
