@@ -790,8 +790,11 @@ static heat_status ensure_discrete(heat_ctx* ctx, cudaStream_t st) {
     std::vector<int> order(G);  // grains whose reduction takes longest first (the solve's launch order)
     for (int g = 0; g < G; ++g) order[g] = g;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return info[2 + a] > info[2 + b]; });
-    if (upload(ctx->d_Dtd_order, order))
+    if (ctx->d_Dtd_order.ensure(sizeof(int) * (size_t)G))
         return ctx->fail(HEAT_ENOMEM, "heat_solve: allocation of thermal-discrete rates failed");
+    // on the solve's stream: a copy on the legacy stream is not ordered before the kernels of a non-blocking one
+    CKR(cudaMemcpyAsync(ctx->d_Dtd_order.p, order.data(), sizeof(int) * (size_t)G, cudaMemcpyHostToDevice, st));
+    CKR(cudaStreamSynchronize(st));
     ctx->td_built = true;
     return HEAT_OK;
 }
