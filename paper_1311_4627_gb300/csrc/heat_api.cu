@@ -1154,10 +1154,10 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
                 if (hs != HEAT_OK) return hs;
             } else if (si)
                 CKR(launch_gemm_f64(cells, N, 1, ctx->d_koff_all.as<int>(), ch.P, nbt, ctx->d_Kw.as<double>(), N, jdst,
-                                    N, 0, o.j_dtype == HEAT_F32, ctx->w_nonneg, cs));
+                                    N, 0, o.j_dtype == HEAT_F32, ctx->w_nonneg, ch.small, cs));
             else
                 CKR(launch_gemm_f64(cells, N, G, ctx->d_bin_off.as<int>(), ch.P, nbt, ctx->d_K.as<double>(), N, jdst,
-                                    (long long)G * N, N, o.j_dtype == HEAT_F32, 1, cs));
+                                    (long long)G * N, N, o.j_dtype == HEAT_F32, 1, ch.small, cs));
             if (o.timing) {
                 cudaEvent_t tb = ctx->take_event();
                 CKR(cudaEventRecord(tb, cs));

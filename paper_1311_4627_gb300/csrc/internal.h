@@ -183,9 +183,10 @@ cudaError_t launch_discrete_gth(const GrainDev& g, const ChunkDev& ch, const int
 // ---- emissivity (k_emis.cu)
 // C[z][m][n] = sum_{k in [koff[z], koff[z+1])} A[m][k] B[k][n] for z < nz, m < M, n < N;
 // koff is a device array of nz+1 offsets; C[z] starts at C + z * zstride_c.  A >= 0; b_nonneg: no B is
-// negative either (Planck kernels, unless a size weight is negative).
+// negative either (Planck kernels, unless a size weight is negative).  few: the solve has at most kSmallCells cells
+// (of the whole solve, as for the build and the recursion: a cell's bits do not depend on the chunk it falls in).
 cudaError_t launch_gemm_f64(int M, int N, int nz, const int* koff, const double* A, long long lda,
                             const double* B, long long ldb, void* C, long long ldc, long long zstride_c, int c_is_f32,
-                            int b_nonneg, cudaStream_t st);
+                            int b_nonneg, int few, cudaStream_t st);
 
 }  // namespace heat

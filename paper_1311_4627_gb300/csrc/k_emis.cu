@@ -201,9 +201,9 @@ __global__ void __launch_bounds__(256, 2) k_gemm_i64(int M, int N, const int* __
     }
 }
 
-// Few rows (solves of few cells): a thread per output, threads along n (coalesced rows of K),
-// one accumulator in ascending k as in k_gemm_f64, so both give the same bits; the 64-row
-// tile above would spend 64 FMAs per useful one on a single cell.
+// Solves of few cells: a thread per output, threads along n (coalesced rows of K), one accumulator in
+// ascending k (k_gemm_f64's bits; k_gemm_i64's sums are rounded once and differ in the last bits); the
+// 64-row tiles above would spend 64 products per useful one on a single cell.
 template <typename TC>
 __global__ void __launch_bounds__(128) k_gemv_f64(int N, const int* __restrict__ koff, const double* __restrict__ A,
                                                   long long lda, const double* __restrict__ B, long long ldb,
@@ -219,9 +219,9 @@ __global__ void __launch_bounds__(128) k_gemv_f64(int N, const int* __restrict__
 
 cudaError_t launch_gemm_f64(int M, int N, int nz, const int* koff, const double* A, long long lda, const double* B,
                             long long ldb, void* C, long long ldc, long long zstride_c, int c_is_f32, int b_nonneg,
-                            cudaStream_t st) {
+                            int few, cudaStream_t st) {
     if (M <= 0 || N <= 0 || nz <= 0) return cudaSuccess;
-    if (M <= kSmallCells) {
+    if (few) {
         dim3 g1((N + 127) / 128, M, nz);
         if (c_is_f32)
             k_gemv_f64<float><<<g1, 128, 0, st>>>(N, koff, A, lda, B, ldb, (float*)C, ldc, zstride_c);
