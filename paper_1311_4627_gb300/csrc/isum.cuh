@@ -7,7 +7,7 @@
 // only below that), against FP64's rounding to 2^-53 of the running sum at every addition.  Exponents are
 // plain integers: nothing overflows or underflows between the operands and the rounded result.
 //
-// Compiles for the host too (the arithmetic is checked there).
+// Compiles for the host too (tests/test_fixed_point.py checks the arithmetic there).
 #pragma once
 #include <cstdint>
 #include <cstring>
@@ -52,21 +52,8 @@ HEAT_HD double from_bits64(uint64_t b) {
     return x;
 #endif
 }
-HEAT_HD uint32_t bits32_ftz(float b) {  // the bits of b, 0 where it is subnormal (b >= 0)
-#ifdef __CUDA_ARCH__
-    float r;
-    asm("mul.rn.ftz.f32 %0, %1, 0f3F800000;" : "=f"(r) : "f"(b));  // on the FP32 pipe, which has room
-    return __float_as_uint(r);
-#else
-    uint32_t v;
-    std::memcpy(&v, &b, 4);
-    return v < 0x00800000u ? 0u : v;
-#endif
-}
-
-// A double x >= 0 as mantissa (h, l) with the leading bit at bit 63 and biased exponent e; 0 (and below
-// the normal range) has mantissa 0 and an exponent below every other, so that it raises no sum's
-// exponent.  x = (h:l) 2^(e - 1086).
+// A double x >= 0 as mantissa (h, l) with the leading bit at bit 63 and biased exponent e; 0 has mantissa 0 and an
+// exponent below every other, so that it raises no sum's exponent.  x = (h:l) 2^(e - 1086).
 constexpr int kZeroExp = 4096;
 struct Mant {
     uint32_t h, l;
@@ -82,33 +69,15 @@ HEAT_HD Mant mant(double x) {
     r.e = e ? e : -kZeroExp;
     return r;
 }
+// a b as a 64-bit product p and exponent ep: value p 2^(ep - kProdExp); the low parts' product is below 2^-64 of the
+// whole and left out
+constexpr int kProdExp = 2108;
+HEAT_HD void mul(const Mant& a, const Mant& b, uint64_t& p, int& ep) {
+    p = (uint64_t)a.h * b.h + (((uint64_t)a.h * b.l) >> 32) + (((uint64_t)a.l * b.h) >> 32);
+    ep = a.e + b.e;
+}
 
-// B x as a 64-bit product p and exponent ep: value p 2^(ep - K), K below; p < 2^64.
-template <int BUILD>
-struct Prod;
-template <>
-struct Prod<1> {  // B in FP32: b = (24 bits at the top of 32) 2^(eb - 158)
-    static constexpr int K = 1212;
-    static HEAT_HD void mul(float bf, const Mant& x, uint64_t& p, int& ep) {
-        const uint32_t b = bits32_ftz(bf);
-        const uint32_t hid = b < 0x00800000u ? b : 0x00800000u;  // the leading bit, 0 for b = 0
-        const uint32_t m = ((b & 0x007fffffu) | hid) << 8;
-        p = (uint64_t)m * x.h + (((uint64_t)m * x.l) >> 32);
-        ep = (int)(b >> 23) + (x.e - kZeroExp) + (int)(hid >> 11);  // 0x800000 >> 11 = kZeroExp
-    }
-};
-template <>
-struct Prod<0> {  // B in FP64
-    static constexpr int K = 2108;
-    static HEAT_HD void mul(double bd, const Mant& x, uint64_t& p, int& ep) { mul(mant(bd), x, p, ep); }
-    static HEAT_HD void mul(const Mant& b, const Mant& x, uint64_t& p, int& ep) {
-        // the low parts' product is below 2^-64 of the whole and left out
-        p = (uint64_t)b.h * x.h + (((uint64_t)b.h * x.l) >> 32) + (((uint64_t)b.l * x.h) >> 32);
-        ep = b.e + x.e;
-    }
-};
-
-// The sum: value a 2^(E + 3 - K).  Terms enter shifted to the exponent E (the largest so far) with three
+// The sum: value a 2^(E + 3 - kProdExp).  Terms enter shifted to the exponent E (the largest so far) with three
 // bits of headroom.
 struct ISum {
     uint64_t a = 0;
@@ -123,18 +92,12 @@ struct ISum {
             E += 2;
         }
     }
-    HEAT_HD void add(uint64_t p, int ep) {
-        raise(ep > E ? ep : E);
-        a += shr64(p, E - ep + 3);
-        settle();
-    }
     // rounded to the nearest double (to 0 below the normal range)
-    template <int BUILD>
     HEAT_HD double value() const {
         if (a == 0) return 0.0;
         const int lz = clz64(a);
         uint64_t m = a << lz;
-        int e = E - lz + 1089 - Prod<BUILD>::K;
+        int e = E - lz + 1089 - kProdExp;
         m += 0x400u;  // half of a unit in the 53rd place (ties away from zero)
         const uint64_t carry = m < 0x400u ? 1u : 0u;  // all ones: the next power of two
         e += (int)carry;
@@ -186,7 +149,7 @@ HEAT_HD void add_each4(ISum& s, const Mant (&a)[4], const Mant (&b)[4]) {
     uint64_t p[4];
     int ep[4], En = s.E;
     for (int u = 0; u < 4; ++u) {
-        Prod<0>::mul(a[u], b[u], p[u], ep[u]);
+        mul(a[u], b[u], p[u], ep[u]);
         En = En > ep[u] ? En : ep[u];
     }
     s.raise(En);

@@ -334,7 +334,7 @@ __device__ __forceinline__ void td_spectrum(const ChunkDev& ch, const int* gorde
 // over E_j - E_i.  The window's edges are the band's transition wavelengths (j + 1, i) and (j, i), whose places on
 // the grid do not depend on the cell (edge table).  A row's windows tile the grid: each is its
 // partial end segments plus the segment integrals between them (summed, by eights, not differenced; inside one segment
-// a difference of two Q60 values, exact to 2^-58 of the segment); the soft term is its partial segment plus
+// a difference of two Q60 values, to 2^-53 of the segment); the soft term is its partial segment plus
 // a suffix sum.  A warp per row, a lane per j; neighbouring lanes share their window edge, so a window costs one
 // fixed-point E1 (seg64.cuh).  With the edges and each partial segment's logarithms and exponentials in FP64
 // the fill was bound by the FP64 unit (83 % busy): 8 cells x 64 grains x 1024 wavelengths 8.7 ms, then

@@ -71,8 +71,7 @@ __global__ void __launch_bounds__(256, 2) k_gemm_f64(int M, int N, const int* __
 //   * Four bins whose K values lie within a factor of 2^4 in every column of the tile: both operands are
 //     aligned to the largest of their four (at staging, once per 32 or 64 outputs), a product is three
 //     multiply-adds, and one shift per four products brings them to the sum's exponent: about 18 cycles a
-//     product.  What the alignment drops is below 2^-57 of the largest operands' product, 2^-53 of the
-//     four's sum.
+//     product.  What a four drops is below 17 x 2^-58 of its largest operands' product.
 //   * Otherwise (the Wien side, where K climbs steeply) each product is aligned by itself: 36 cycles.
 //   * Four bins without any emission in the tile's columns (K = 0: the bin's energy or temperature is too low)
 //     are left out.
@@ -196,7 +195,7 @@ __global__ void __launch_bounds__(256, 2) k_gemm_i64(int M, int N, const int* __
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             const int n = n0 + tx + 16 * s;
-            if (n < N) Cz[(size_t)m * ldc + n] = bad[ty + 16 * r] ? (TC)NAN : (TC)S[r][s].value<0>();
+            if (n < N) Cz[(size_t)m * ldc + n] = bad[ty + 16 * r] ? (TC)NAN : (TC)S[r][s].value();
         }
     }
 }

@@ -39,7 +39,7 @@ struct SegF64 {
 };
 // The intra-bin term of a bin whose soft photons begin at offset t (fraction tau) of segment n, with Psi the
 // integral of Omega beyond the segment: c (int from t to the segment's end + Psi) / (E_{j+1} - E_j).  The part of
-// the segment is the difference of two fixed-point values, exact to 2^-58 of the whole segment's.
+// the segment is the difference of two fixed-point values, to 2^-53 of the whole segment's.
 __device__ __forceinline__ double soft_term(const GrainDev& gd, int g, int n, double ua, double su, double t,
                                             int64_t tau, double Psi, double invdE) {
     const double b = ua * gd.ce64[(size_t)g * gd.N + n], q0 = su + gd.sC[(size_t)g * gd.N + n] + 1.0;
