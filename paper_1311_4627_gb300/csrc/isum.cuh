@@ -34,6 +34,7 @@ HEAT_HD int clz64(uint64_t a) {  // a != 0
     return __builtin_clzll(a);
 #endif
 }
+constexpr uint64_t kMag64 = 0x7fffffffffffffffull;  // all but the sign (a -0 counts as 0)
 HEAT_HD uint64_t bits64(double x) {
 #ifdef __CUDA_ARCH__
     return (uint64_t)__double_as_longlong(x);
@@ -60,7 +61,7 @@ struct Mant {
     int e;
 };
 HEAT_HD Mant mant(double x) {
-    const uint64_t b = bits64(x);
+    const uint64_t b = bits64(x) & kMag64;
     const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
     Mant r;
     const int e = (int)(hi >> 20);
@@ -116,7 +117,7 @@ struct Align4 {
 HEAT_HD Align4 align4(const double (&x)[4]) {
     Align4 r;
     int e[4];
-    for (int u = 0; u < 4; ++u) e[u] = (int)(bits64(x[u]) >> 52);
+    for (int u = 0; u < 4; ++u) e[u] = (int)((bits64(x[u]) & kMag64) >> 52);
     const int a = e[0] > e[1] ? e[0] : e[1], b = e[2] > e[3] ? e[2] : e[3];
     r.E = a > b ? a : b;
     for (int u = 0; u < 4; ++u) {

@@ -113,13 +113,13 @@ __global__ void __launch_bounds__(256, 2) k_gemm_i64(int M, int N, const int* __
             Be[q][c] = a.E;
             // compared as integers: the values are not negative (the FP64 unit takes 64 cycles a comparison)
             const int kn = k1 - (kb + 4 * q);  // bins of this four
-            long long lo = __double_as_longlong(x[0]), hi = lo;
+            long long lo = (long long)(bits64(x[0]) & kMag64), hi = lo;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 Bm[q][u][c] = mant(x[u]);
                 if (u < kn) {
-                    lo = min(lo, __double_as_longlong(x[u]));
-                    hi = max(hi, __double_as_longlong(x[u]));
+                    lo = min(lo, (long long)(bits64(x[u]) & kMag64));
+                    hi = max(hi, (long long)(bits64(x[u]) & kMag64));
                 }
             }
             const int f = hi > 0 ? (hi - lo > (3LL << 52) ? 3 : 1) : 0;  // (a difference of 3 exponents: 2^3 to 2^4)

@@ -90,6 +90,13 @@ def test_zeros_and_the_carry(host):
     assert _dot(host, a, np.ones(4), 1) == 2.0 and _dot(host, a, np.ones(4), 0) == 2.0
 
 
+def test_negative_zero(host):
+    a = np.array([1.5, -0.0, 3.0, 0.0, -0.0, -0.0, -0.0, -0.0])
+    for form in (0, 1):
+        assert _dot(host, a, np.array([1.0, 2.0, -0.0, 1.0] * 2), form) == 1.5
+        assert _dot(host, np.abs(a), np.array([1.0, -0.0, -0.0, 1.0] * 2), form) == 1.5
+
+
 def _e1_exact(z, bits=200):
     """E1(z) = sum z^k / (k+1)! for z in Q60, as an integer times 2^-bits."""
     s, t, k = 0, 1 << bits, 0

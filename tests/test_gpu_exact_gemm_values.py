@@ -1,0 +1,36 @@
+"""The exact emissivity's fixed-point contraction on values outside the ordinary: zeros of either sign."""
+import numpy as np
+import pytest
+
+from paper_1311_4627_gb300 import heat
+from paper_1311_4627_gb300 import workloads as W
+
+from .gpu_helpers import Lib
+
+pytestmark = pytest.mark.gpu
+
+EXACT = dict(build=heat.HEAT_BUILD_F64, emis=heat.HEAT_EMIS_F64, j_dtype=heat.HEAT_F64)
+
+
+def _workload(cells, n_lambda=64):
+    return W.grain_subset(W.batched(cells=cells, n_lambda=n_lambda), [0, 30])
+
+
+def test_negative_zeros():
+    """Cross-sections and size weights of -0 count as 0: the same j."""
+    wl = _workload(33)
+    wl.cabs = wl.cabs.copy()
+    wl.cabs[:, ::5] = 0.0
+    wl.size_weight = np.array([0.0, 0.5])
+    out = []
+    for sign in (1.0, -1.0):
+        wl.cabs[:, ::5] = sign * 0.0
+        wl.size_weight[0] = sign * 0.0
+        lib = Lib(wl)
+        try:
+            lib.set_fields(wl.u)
+            out.append((lib.solve(**EXACT)[1], lib.solve(size_integrate=1, **EXACT)[1]))
+        finally:
+            lib.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    assert np.all(out[0][1] >= 0.0) and out[0][1].max() > 0.0
