@@ -64,10 +64,16 @@ HEAT_HD Mant mant(double x) {
     const uint64_t b = bits64(x) & kMag64;
     const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
     Mant r;
-    const int e = (int)(hi >> 20);
-    r.h = e ? ((hi << 11) | (lo >> 21) | 0x80000000u) : 0u;
-    r.l = e ? lo << 11 : 0u;
-    r.e = e ? e : -kZeroExp;
+    r.e = (int)(hi >> 20);
+    r.h = (hi << 11) | (lo >> 21) | 0x80000000u;
+    r.l = lo << 11;
+    if (r.e == 0) {  // zero, or subnormal: normalised
+        const int lz = b ? clz64(b) : 0;
+        const uint64_t m = b << lz;
+        r.h = (uint32_t)(m >> 32);
+        r.l = (uint32_t)m;
+        r.e = b ? 12 - lz : -kZeroExp;
+    }
     return r;
 }
 // a b as a 64-bit product p and exponent ep: value p 2^(ep - kProdExp); the low parts' product is below 2^-64 of the
@@ -93,18 +99,19 @@ struct ISum {
             E += 2;
         }
     }
-    // rounded to the nearest double (to 0 below the normal range)
+    // rounded to the nearest double
     HEAT_HD double value() const {
         if (a == 0) return 0.0;
         const int lz = clz64(a);
         uint64_t m = a << lz;
         int e = E - lz + 1089 - kProdExp;
+        if (e <= 0) return from_bits64((shr64(m, 11 - e) + 1) >> 1);  // below the normal range: to a multiple of 2^-1074
         m += 0x400u;  // half of a unit in the 53rd place (ties away from zero)
         const uint64_t carry = m < 0x400u ? 1u : 0u;  // all ones: the next power of two
         e += (int)carry;
         // the leading bit adds 1 to the exponent field
         const uint64_t r = carry ? 0 : (m >> 11) & 0x000fffffffffffffull;
-        return e > 0 ? from_bits64(((uint64_t)e << 52) | r) : 0.0;
+        return from_bits64(((uint64_t)e << 52) | r);
     }
 };
 
@@ -117,11 +124,15 @@ struct Align4 {
 HEAT_HD Align4 align4(const double (&x)[4]) {
     Align4 r;
     int e[4];
-    for (int u = 0; u < 4; ++u) e[u] = (int)((bits64(x[u]) & kMag64) >> 52);
+    for (int u = 0; u < 4; ++u) {
+        e[u] = (int)((bits64(x[u]) & kMag64) >> 52);
+        e[u] += e[u] == 0;  // zeros and subnormals: the exponent of the smallest normal, no leading bit
+    }
     const int a = e[0] > e[1] ? e[0] : e[1], b = e[2] > e[3] ? e[2] : e[3];
     r.E = a > b ? a : b;
     for (int u = 0; u < 4; ++u) {
-        const uint64_t v = (bits64(x[u]) & 0xfffffffffffffull) | (e[u] > 0 ? 0x10000000000000ull : 0ull);
+        const uint64_t lead = (bits64(x[u]) & 0x7ff0000000000000ull) ? 0x10000000000000ull : 0ull;
+        const uint64_t v = (bits64(x[u]) & 0xfffffffffffffull) | lead;
         const uint64_t y = shr64(v << 4, r.E - e[u]);
         r.h[u] = (uint32_t)(y >> 27);
         r.l[u] = (uint32_t)y & 0x7ffffffu;

@@ -97,6 +97,29 @@ def test_negative_zero(host):
         assert _dot(host, np.abs(a), np.array([1.0, -0.0, -0.0, 1.0] * 2), form) == 1.5
 
 
+# Subnormal operands count at their value, results below the normal range are rounded to its last place (2^-1074).  The
+# aligned form's bound is against the largest of a four, at least 2^-1022 here.
+@pytest.mark.parametrize("seed", range(20))
+def test_subnormals(host, seed):
+    rng = np.random.default_rng(seed)
+    tiny = Fraction(1, 2**1074)
+    n = 16
+    sub = rng.integers(1, 2**52, n).astype(np.float64) * 2.0**-1074 * 2.0 ** -rng.integers(0, 50, n)
+    sub[sub == 0.0] = 2.0**-1074
+    w = rng.uniform(0.5, 1.0, n)
+    for a, b in ((sub, w), (w, sub)):
+        ref = _exact(a, b)
+        assert abs(Fraction(_dot(host, a, b, 1)) - ref) <= ref * (ULP + Fraction(n, 2**59)) + tiny / 2
+        lost = n // 4 * Fraction(17, 2**58) * Fraction(1, 2**1022)
+        assert abs(Fraction(_dot(host, a, b, 0)) - ref) <= ref * (ULP + Fraction(n, 2**59)) + lost + tiny / 2
+    # normal operands, a subnormal product
+    a, b = w * 2.0**-600, rng.uniform(0.5, 1.0, n) * 2.0 ** -rng.integers(421, 480, n)
+    ref = _exact(a, b)
+    assert abs(Fraction(_dot(host, a, b, 1)) - ref) <= ref * (ULP + Fraction(n, 2**59)) + tiny / 2
+    assert _dot(host, np.full(4, 2.0**-600), np.full(4, 2.0**-474), 1) == 2.0**-1072
+    assert _dot(host, np.full(4, 2.0**-600), np.full(4, 2.0**-600), 1) == 0.0
+
+
 def _e1_exact(z, bits=200):
     """E1(z) = sum z^k / (k+1)! for z in Q60, as an integer times 2^-bits."""
     s, t, k = 0, 1 << bits, 0

@@ -1,4 +1,4 @@
-"""The exact emissivity's fixed-point contraction on values outside the ordinary: zeros of either sign."""
+"""The exact emissivity's fixed-point contraction on values outside the ordinary: zeros of either sign, subnormals."""
 import numpy as np
 import pytest
 
@@ -34,3 +34,20 @@ def test_negative_zeros():
             lib.close()
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
     assert np.all(out[0][1] >= 0.0) and out[0][1].max() > 0.0
+
+
+def test_subnormal_emissivities():
+    """Emission far below the normal range (size weights of 1e-300): j as the few-cell kernel's FMA sums give it, to the
+    exact path's 1e-10 and a few units in the last place of a subnormal."""
+    wl = _workload(33)
+    wl.size_weight = np.array([1e-300, 1e-302])
+    lib = Lib(wl)
+    try:
+        lib.set_fields(wl.u)
+        _, j = lib.solve(size_integrate=1, **EXACT)
+        lib.set_fields(wl.u[:3])
+        _, few = lib.solve(size_integrate=1, **EXACT)
+    finally:
+        lib.close()
+    assert np.any((few > 0.0) & (few < 2.0**-1022))
+    assert np.all(np.abs(j[:3] - few) <= 1e-10 * few + 8 * 2.0**-1074)
