@@ -99,7 +99,7 @@ struct ISum {
             E += 2;
         }
     }
-    // rounded to the nearest double
+    // rounded to the nearest double (infinity beyond the range)
     HEAT_HD double value() const {
         if (a == 0) return 0.0;
         const int lz = clz64(a);
@@ -111,7 +111,7 @@ struct ISum {
         e += (int)carry;
         // the leading bit adds 1 to the exponent field
         const uint64_t r = carry ? 0 : (m >> 11) & 0x000fffffffffffffull;
-        return from_bits64(((uint64_t)e << 52) | r);
+        return from_bits64(e < 2047 ? ((uint64_t)e << 52) | r : 0x7ff0000000000000ull);
     }
 };
 

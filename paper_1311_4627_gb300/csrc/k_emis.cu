@@ -66,6 +66,13 @@ __global__ void __launch_bounds__(256, 2) k_gemm_f64(int M, int N, const int* __
     }
 }
 
+// One output's FMA chain, for columns that fixed point cannot hold (an infinite K).
+__device__ __noinline__ double chain_f64(int k0, int k1, const double* a, const double* b, long long ldb) {
+    double acc = 0.0;
+    for (int k = k0; k < k1; ++k) acc = fma(a[k], b[(size_t)k * ldb], acc);
+    return acc;
+}
+
 // The contraction of non-negative operands without the FP64 unit, which takes 64 cycles per warp-wide
 // multiply-add: the sums run in 64-bit fixed point on the integer pipes (isum.cuh), four bins at a time.
 //   * Four bins whose K values lie within a factor of 2^4 in every column of the tile: both operands are
@@ -90,11 +97,13 @@ __global__ void __launch_bounds__(256, 2) k_gemm_i64(int M, int N, const int* __
     __shared__ Mant Am[KB][4][64], Bm[KB][4][32];  // for the one-by-one form
     __shared__ int flag[KB];  // 0: no emission, 1: aligned, 3: one by one
     __shared__ int bad[64];   // rows with a NaN or an infinity
+    __shared__ int badc[32];  // columns with an infinity (or a NaN)
     const int z = blockIdx.z;
     const int k0 = koff[z], k1 = koff[z + 1];
     const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 32;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     if (tid < 64) bad[tid] = 0;
+    if (tid < 32) badc[tid] = 0;
     ISum S[4][2];
     for (int kb = k0; kb < k1; kb += 4 * KB) {
         if (tid < KB) flag[tid] = 0;
@@ -122,6 +131,7 @@ __global__ void __launch_bounds__(256, 2) k_gemm_i64(int M, int N, const int* __
                     hi = max(hi, (long long)(bits64(x[u]) & kMag64));
                 }
             }
+            if (hi >= 0x7ff0000000000000ll) badc[c] = 1;
             const int f = hi > 0 ? (hi - lo > (3LL << 52) ? 3 : 1) : 0;  // (a difference of 3 exponents: 2^3 to 2^4)
             const int any = __reduce_or_sync(0xffffffffu, f);
             if (c == 0) flag[q] = any;
@@ -195,7 +205,11 @@ __global__ void __launch_bounds__(256, 2) k_gemm_i64(int M, int N, const int* __
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             const int n = n0 + tx + 16 * s;
-            if (n < N) Cz[(size_t)m * ldc + n] = bad[ty + 16 * r] ? (TC)NAN : (TC)S[r][s].value();
+            if (n >= N) continue;
+            double v = S[r][s].value();
+            if (bad[ty + 16 * r]) v = NAN;
+            if (badc[tx + 16 * s]) v = chain_f64(k0, k1, A + (size_t)m * lda, B + n, ldb);
+            Cz[(size_t)m * ldc + n] = (TC)v;
         }
     }
 }

@@ -120,6 +120,14 @@ def test_subnormals(host, seed):
     assert _dot(host, np.full(4, 2.0**-600), np.full(4, 2.0**-600), 1) == 0.0
 
 
+def test_overflow(host):
+    big = np.full(8, 2.0**512)
+    for form in (0, 1):
+        assert _dot(host, big, big, form) == np.inf
+        assert _dot(host, big[:4], big[:4] * np.array([0.125, 0.125, 0.125, 0.0625]), form) == 7 * 2.0**1020
+        assert _dot(host, big[:4], big[:4] * 0.25, form) == np.inf  # four quarters of 2^1024
+
+
 def _e1_exact(z, bits=200):
     """E1(z) = sum z^k / (k+1)! for z in Q60, as an integer times 2^-bits."""
     s, t, k = 0, 1 << bits, 0

@@ -1,4 +1,4 @@
-"""The exact emissivity's fixed-point contraction on values outside the ordinary: zeros of either sign, subnormals."""
+"""The exact emissivity's fixed-point contraction on values outside the ordinary: zeros of either sign, subnormals, infinities."""
 import numpy as np
 import pytest
 
@@ -51,3 +51,23 @@ def test_subnormal_emissivities():
         lib.close()
     assert np.any((few > 0.0) & (few < 2.0**-1022))
     assert np.all(np.abs(j[:3] - few) <= 1e-10 * few + 8 * 2.0**-1074)
+
+
+def test_infinite_kernels():
+    """Size weights that take part of the emission kernel, or only sums of it, beyond the range: infinities, NaN and finite j
+    where the few-cell kernel's FMA sums have them."""
+    wl = _workload(33)
+    wl.cabs = wl.cabs * 1e10
+    wl.size_weight = np.array([1e307, 1e308])
+    lib = Lib(wl)
+    try:
+        lib.set_fields(wl.u)
+        _, j = lib.solve(size_integrate=1, **EXACT)
+        lib.set_fields(wl.u[:3])
+        _, few = lib.solve(size_integrate=1, **EXACT)
+    finally:
+        lib.close()
+    assert np.any(~np.isfinite(few)) and np.any(np.isfinite(few))
+    assert np.array_equal(np.isnan(j[:3]), np.isnan(few)) and np.array_equal(np.isinf(j[:3]), np.isinf(few))
+    ok = np.isfinite(few)
+    assert np.all(np.abs(j[:3][ok] - few[ok]) <= 1e-10 * few[ok])
