@@ -81,6 +81,7 @@ struct heat_ctx {
     struct Slot {
         DevBuf ua64, su64, ua32, Bb64, Bb32, phi, xs, ep, pabs, P, j, led, A, rowscale, work, phs, tdq;
         DevBuf P_alt, j_alt, led_alt;   // second staging set of asynchronous host I/O
+        size_t phi_failed = 0;          // size of `phi` that did not fit (0: none)
         cudaStream_t stream = nullptr;  // created on first use
         cudaEvent_t done = nullptr;
         cudaStream_t copy = nullptr;    // asynchronous host I/O: copies to the host

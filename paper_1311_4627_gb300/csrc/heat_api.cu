@@ -799,6 +799,24 @@ static heat_status ensure_discrete(heat_ctx* ctx, cudaStream_t st) {
     return HEAT_OK;
 }
 
+// A table that a solve can do without.  False: no room, or the stream is being captured and the buffer would have to be
+// allocated (which capture does not allow).  `failed`: the size that did not fit last, which is tried again only once
+// that much memory is free.
+static bool ensure_optional(DevBuf& b, size_t& failed, size_t bytes, cudaStream_t st) {
+    if (bytes <= b.cap) return true;
+    if (st) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
+    }
+    if (failed && bytes >= failed) {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || free_b + b.cap < bytes) return false;
+    }
+    failed = b.ensure(bytes) == cudaSuccess ? 0 : bytes;
+    if (failed) (void)cudaGetLastError();
+    return !failed;
+}
+
 // Smallest default chunk worth pipelining host copies against.
 constexpr int kHostIoMinChunk = 1024;
 
@@ -954,13 +972,11 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
     // the integral form's matrix build in two passes (photon prefixes, then the elements): needs the
     // prefix table
     const bool two_pass = !discrete && !fused && count > kSmallCells && o.heating == HEAT_HEATING_INTEGRAL;
-    bool phi_ok[heat_ctx::kMaxSlots] = {};
     // scratch of every slot in use
     bool internal_P = (P_out == nullptr) || o.host_io;
     const bool async_io = o.host_io == 2;
     const int io_set = async_io ? ctx->io_parity : 0;
-    for (int k = 0; k < nslots; ++k) {
-        auto& sl = ctx->slots[k];
+    auto ensure_scratch = [&](heat_ctx::Slot& sl) {
         bool ok = true;
         if (build == 0) {
             ok &= !sl.ua64.ensure(sizeof(double) * (size_t)N * Cc);
@@ -993,10 +1009,21 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
             ok &= !sl.A.ensure((mode_tf32(o.emis) ? 4 : 2) * (size_t)t.aoff_h[Gt]);
             ok &= !sl.rowscale.ensure(sizeof(float) * (size_t)Cc * Gt);
         }
-        if (!ok) return ctx->fail(HEAT_ENOMEM, "heat_solve: scratch allocation failed");
-        // without room for the prefix table the build walks every task's segments once instead
-        phi_ok[k] = two_pass && sl.phi.ensure((build == 0 ? 8 : 4) * (size_t)G * N * Cc) == cudaSuccess;
-        if (two_pass && !phi_ok[k]) (void)cudaGetLastError();
+        return ok;
+    };
+    for (int k = 0; k < nslots; ++k) {
+        if (ensure_scratch(ctx->slots[k])) continue;
+        // the prefix tables are optional: those that earlier solves left give way
+        (void)cudaGetLastError();
+        for (auto& sl : ctx->slots) sl.phi.release();
+        if (!ensure_scratch(ctx->slots[k])) return ctx->fail(HEAT_ENOMEM, "heat_solve: scratch allocation failed");
+    }
+    // after everything that the solve cannot do without; where there is no room for a prefix table the build walks
+    // every task's segments once instead
+    bool phi_ok[heat_ctx::kMaxSlots] = {};
+    for (int k = 0; k < nslots; ++k) {
+        auto& sl = ctx->slots[k];
+        phi_ok[k] = two_pass && ensure_optional(sl.phi, sl.phi_failed, (build == 0 ? 8 : 4) * (size_t)G * N * Cc, st);
         if (nslots > 1 && !sl.stream) {
             CKR(cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking));
             CKR(cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming));
