@@ -820,20 +820,27 @@ static bool ensure_optional(DevBuf& b, size_t& failed, size_t bytes, cudaStream_
 // Smallest default chunk worth pipelining host copies against.
 constexpr int kHostIoMinChunk = 1024;
 
-// Default cells per chunk: as many as 45 % of the device memory the library could use (free
-// memory plus the chunk scratch it already holds) allows for `nslots` chunks in flight (B band,
-// X history, field tables per 32-cell group), at least one group; with several slots the range
-// is also split evenly over them.  More cells per chunk means more warps in flight for the
-// latency-bound build and recursion kernels.
 // Whether a solve of `count` cells with these options runs the fused build + recursion.
 static bool uses_fused(const heat_ctx* ctx, const heat_opts& o, int count) {
     const bool want = o.fused_build == 1 || (o.fused_build == 0 && ctx->tuned_fused);
     return o.build == HEAT_BUILD_F32 && o.heating == HEAT_HEATING_INTEGRAL && count > kSmallCells && want;
 }
 
-static int default_chunk(heat_ctx* ctx, int build, int count, int nslots, bool fused) {
-    const size_t band_bytes = fused ? 0 : (size_t)ctx->band_per_cell * 32 * (build == 0 ? 8 : 4);
-    const size_t phi_bytes = fused ? 0 : (size_t)ctx->G * ctx->N * 32 * (build == 0 ? 8 : 4);
+// Whether its matrix build takes two passes (photon prefixes, then the elements) where the prefix table fits.
+static bool uses_two_pass(const heat_ctx* ctx, const heat_opts& o, int count) {
+    return o.heating == HEAT_HEATING_INTEGRAL && o.cooling != HEAT_COOLING_DISCRETE && count > kSmallCells &&
+           !uses_fused(ctx, o, count);
+}
+
+// Default cells per chunk: as many as 45 % of the device memory the library could use (free
+// memory plus the chunk scratch it already holds) allows for `nslots` chunks in flight (B band, the two-pass
+// build's prefix table, X history, field tables per 32-cell group), at least one group; with several slots the range
+// is also split evenly over them.  More cells per chunk means more warps in flight for the
+// latency-bound build and recursion kernels.
+static int default_chunk(heat_ctx* ctx, const heat_opts& o, int count, int nslots) {
+    const size_t el = o.build == 0 ? 8 : 4;
+    const size_t band_bytes = uses_fused(ctx, o, count) ? 0 : (size_t)ctx->band_per_cell * 32 * el;
+    const size_t phi_bytes = uses_two_pass(ctx, o, count) ? (size_t)ctx->G * ctx->N * 32 * el : 0;
     const size_t per_group = band_bytes + phi_bytes + (size_t)ctx->nbt * 32 * 10 + (size_t)ctx->N * 32 * 16;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = size_t(16) << 30;
@@ -919,7 +926,7 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
     // asynchronous host I/O the copies overlap the next call's kernels, so one chunk
     if (nslots == 0) nslots = (o.host_io == 1 && count >= 2 * kHostIoMinChunk) ? 2 : 1;
     nslots = std::min(nslots, (int)heat_ctx::kMaxSlots);
-    if (chunk == 0) chunk = default_chunk(ctx, build, count, nslots, uses_fused(ctx, o, count));
+    if (chunk == 0) chunk = default_chunk(ctx, o, count, nslots);
     const int n_chunks = (count + chunk - 1) / chunk;
     nslots = std::max(1, std::min(nslots, n_chunks));
     const int span = std::min(count, chunk);
@@ -971,7 +978,7 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
     const bool pack_in_recur = tc && !si && !fused && count > kSmallCells && !discrete;
     // the integral form's matrix build in two passes (photon prefixes, then the elements): needs the
     // prefix table
-    const bool two_pass = !discrete && !fused && count > kSmallCells && o.heating == HEAT_HEATING_INTEGRAL;
+    const bool two_pass = uses_two_pass(ctx, o, count);
     // scratch of every slot in use
     bool internal_P = (P_out == nullptr) || o.host_io;
     const bool async_io = o.host_io == 2;
@@ -1375,8 +1382,7 @@ heat_status heat_graph_create(heat_ctx* ctx, const heat_opts* opts, double* P_ou
     if (o.streams == 0) o.streams = 1;
     if (o.chunk_cells == 0) {
         const int count = o.cell_count > 0 ? o.cell_count : ctx->n_cells - o.cell_begin;
-        o.chunk_cells = default_chunk(ctx, o.build, std::max(count, 1), std::min(o.streams, (int)heat_ctx::kMaxSlots),
-                                      uses_fused(ctx, o, count));
+        o.chunk_cells = default_chunk(ctx, o, std::max(count, 1), std::min(o.streams, (int)heat_ctx::kMaxSlots));
     }
     heat_status h = heat_solve(ctx, &o, P_out, j_out, stream);  // allocations, uploads, streams
     if (h != HEAT_OK) return h;

@@ -100,3 +100,31 @@ def test_the_prefix_table_gives_way(lib_and_P):
         assert np.array_equal(_solve(lib, P, streams=2), ref)
     finally:
         hold.release()
+
+
+# 2 GB of chunk scratch (45 % of 4 GB) hold about 2097 groups of 32 cells by their field tables, 419 with a prefix table
+@pytest.mark.parametrize("opts,chunks", [(dict(heating=heat.HEAT_HEATING_POINT), 1), ({}, 2)])
+def test_only_the_two_pass_build_makes_room_for_its_table(workload, opts, chunks):
+    """The default chunk of a solve without a prefix table (the point rule) does not shrink for one; kernel launches of a
+    captured solve against those of one chunk of all cells."""
+    import torch
+
+    cells = 2 * CELLS
+    P = torch.empty(cells, workload.total_bins, dtype=torch.float64, device="cuda")
+    lib = Lib(workload)
+    s = torch.cuda.Stream()
+    hold = None
+    try:
+        lib.set_fields(np.concatenate([workload.u, workload.u]))
+        hold = _Hold(4 << 30)
+        nodes = []
+        for chunk in (0, cells):
+            g = heat.Graph(lib.ctx, heat.heat_default_opts(**dict(OPTS, streams=1, chunk_cells=chunk, **opts)), P, None,
+                           s.cuda_stream)
+            nodes.append(g.kernel_nodes())
+            g.close()
+        assert nodes[0] == chunks * nodes[1]
+    finally:
+        if hold:
+            hold.release()
+        lib.close()
