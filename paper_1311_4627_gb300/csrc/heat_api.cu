@@ -1041,6 +1041,7 @@ heat_status heat_solve(heat_ctx* ctx, const heat_opts* opts, double* P_out, void
             for (cudaEvent_t& e : sl.copied) CKR(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         }
     }
+    ctx->one_walk = two_pass && !std::all_of(phi_ok, phi_ok + nslots, [](bool v) { return v; });
     if (nslots > 1 && !ctx->ev_fork) CKR(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
 
     GrainDev gd{};
@@ -1331,6 +1332,7 @@ heat_status heat_autotune(heat_ctx* ctx, const heat_opts* opts, double* P_out, v
         if ((hk = time_config(pick, &ms)) != HEAT_OK) return done(hk);
         if (ms < best) best = ms; else ctx->tuned_recur_bps = keep;
     }
+    const bool one_walk = ctx->one_walk;  // of the chosen configuration
     if (opts->emis > HEAT_EMIS_F64 && opts->emis_n_tile == 0) {
         ctx->tuned_emis_nt = 128;
         float ms = 0.0f;
@@ -1343,7 +1345,8 @@ heat_status heat_autotune(heat_ctx* ctx, const heat_opts* opts, double* P_out, v
         if ((hk = time_config(pick, &ms)) != HEAT_OK) return done(hk);
         if (ms < best) best = ms; else ctx->tuned_fused = 0;
     }
-    if (opts->build == HEAT_BUILD_F32 && opts->build_prefetch == 0 && !ctx->tuned_fused) {
+    // (the two-pass build has no prefetch to choose)
+    if (opts->build == HEAT_BUILD_F32 && opts->build_prefetch == 0 && !ctx->tuned_fused && one_walk) {
         ctx->tuned_prefetch = ctx->N <= 1024 ? 2 : 1;  // the other setting than the default
         float ms = 0.0f;
         if ((hk = time_config(pick, &ms)) != HEAT_OK) return done(hk);

@@ -128,3 +128,24 @@ def test_only_the_two_pass_build_makes_room_for_its_table(workload, opts, chunks
         if hold:
             hold.release()
         lib.close()
+
+
+@pytest.mark.parametrize("prefetch", [1, 2])
+def test_one_walk_prefetch_on_and_off(workload, prefetch):
+    """The FP32 build without room for its prefix table (half the bytes of FP64), with and without its pattern prefetch."""
+    import torch
+
+    P = torch.empty(CELLS, workload.total_bins, dtype=torch.float64, device="cuda")
+    lib = Lib(workload)
+    hold = None
+    try:
+        lib.set_fields(workload.u)
+        opts = dict(build=heat.HEAT_BUILD_F32, streams=1)
+        hold = _Hold((FIELDS + PREFIX) // 2 - (60 << 20))
+        a = _solve(lib, P, build_prefetch=prefetch, **opts)
+        hold.release()
+        assert np.array_equal(a, _solve(lib, P, **opts))
+    finally:
+        if hold:
+            hold.release()
+        lib.close()
