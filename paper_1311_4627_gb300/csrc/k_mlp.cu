@@ -409,8 +409,8 @@ __global__ void k_round_bf16(long long n, const float* __restrict__ in, __nv_bfl
     if (i < n) out[i] = __float2bfloat16_rn(in[i]);  // (the caller's pointer: 4-byte alignment only)
 }
 
-// Masked squared error: targets NaN are excluded.  dY = 2 (Y - T) / count (BF16);
-// loss partial sums per block into loss[blockIdx.x].
+// Masked squared error: targets NaN are excluded.  dY = 2 (Y - T) / count (BF16); the loss in compensated FP32 sums
+// per thread (a thread takes as many entries as the batch gives it), FP64 across threads.
 // Weight of the one-sided penalty relative to the fitted entries (it only has to keep the
 // masked tail below the mask, not fit it).
 constexpr float kTailWeight = 0.3f;
@@ -419,17 +419,17 @@ __global__ void k_mse(long long n, int N, const float* __restrict__ Y, const flo
                       const float* __restrict__ tb, const float* __restrict__ ym, const float* __restrict__ ys,
                       const unsigned long long* __restrict__ count, __nv_bfloat16* __restrict__ dY,
                       double* __restrict__ loss_acc) {
-    __shared__ float red[8];
+    __shared__ double red[8];
     const unsigned long long c = *count;
     const float inv = c > 0 ? 1.0f / (float)c : 0.0f;
-    float e2 = 0.0f;
+    Sum32 e2;
     // four entries a thread (rows are multiples of 64), as many rounds as the grid leaves: one atomic addition of
     // the loss a block
     for (long long i4 = (long long)blockIdx.x * blockDim.x + threadIdx.x; i4 < n / 4;
          i4 += (long long)gridDim.x * blockDim.x) {
         const float4 t4 = ((const float4*)T)[i4], y4 = ((const float4*)Y)[i4];
         const float t[4] = {t4.x, t4.y, t4.z, t4.w}, y[4] = {y4.x, y4.y, y4.z, y4.w};
-        float g[4];
+        float g[4], d2[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             float d = 0.0f;
@@ -444,17 +444,19 @@ __global__ void k_mse(long long n, int N, const float* __restrict__ Y, const flo
                 if (bound == bound && over > 0.0f) d = kTailWeight * over / ys[k];
             }
             g[u] = 2.0f * d * inv;
-            e2 += d * d;
+            d2[u] = __fmul_rn(d, d);
         }
+        e2.add((d2[0] + d2[1]) + (d2[2] + d2[3]));
         const __nv_bfloat162 a = __floats2bfloat162_rn(g[0], g[1]), b = __floats2bfloat162_rn(g[2], g[3]);
         ((uint2*)dY)[i4] = make_uint2(*(const uint32_t*)&a, *(const uint32_t*)&b);
     }
-    for (int o = 16; o > 0; o >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e2;
+    double w = isfinite(e2.s) ? e2.wide() : (double)e2.s;
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = w;
     __syncthreads();
     if (threadIdx.x == 0 && loss_acc) {
         double s = 0.0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += (double)red[k];
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += red[k];
         if (s != 0.0) atomicAdd(loss_acc, s * (double)inv);
     }
 }
