@@ -364,8 +364,8 @@ __global__ void __launch_bounds__(128) k_prefix32(GrainDev gd, ChunkDev ch) {
         return;
     }
     float* Bb = ch.Bb32 + (size_t)grp * gd.band_total * 32 + lane;
-    int p[2], p1[2];
-    int4 sf[2], sf_n[2];  // each grain's next two soft-photon records (loaded a record ahead of the test)
+    int p[2] = {0, 0}, p1[2] = {0, 0};
+    int4 sf[2] = {}, sf_n[2] = {};  // each grain's next two soft-photon records (loaded a record ahead of the test)
     auto next = [&](int i) {
         sf[i] = sf_n[i];
         sf_n[i] = __ldg(gd.soft32 + min(p[i] + 1, p1[i]));

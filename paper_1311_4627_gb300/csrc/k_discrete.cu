@@ -317,9 +317,9 @@ constexpr int64_t kNoQ60 = INT64_MIN;
 // Spectrum of block b of a launch that starts at spectrum s0: grains in the order `gorder`
 // (longest state reduction first), every cell of the chunk for each grain in turn, so that the spectra of one
 // launch have similar cost and the largest start first.
-__device__ __forceinline__ void td_spectrum(const ChunkDev& ch, const int* gorder, long long s0, int& cell, int& g,
-                                            int b = -1) {
-    const long long sp = s0 + (b < 0 ? (int)blockIdx.x : b);
+__device__ __forceinline__ void td_spectrum(const ChunkDev& ch, const int* gorder, long long s0, int b, int& cell,
+                                            int& g) {
+    const long long sp = s0 + b;
     cell = (int)(sp % ch.cells);
     g = gorder[sp / ch.cells];
 }
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
     extern __shared__ double fsm[];
     const int bsp = blockIdx.x / S, part = blockIdx.x % S;  // spectrum of the launch, part of its rows
     int cell, g;
-    td_spectrum(ch, gorder, s0, cell, g, bsp);
+    td_spectrum(ch, gorder, s0, bsp, cell, g);
     const int N = gd.N;
     double* A = fsm;
     int64_t* Z = (int64_t*)(A + N);
@@ -403,7 +403,6 @@ __global__ void __launch_bounds__(256) k_td_fill(GrainDev gd, ChunkDev ch, const
     }
     __syncthreads();
     const int off = gd.bin_off[g], nb = gd.bin_off[g + 1] - off;
-    const double* E = gd.E + off;
     const double* Dg = Dt + doff[g];
     const int* rp = gd.rowptr + off + g;
     const int4* ev = env + (off / kGthB + g);
@@ -606,7 +605,7 @@ __global__ void __launch_bounds__(kGthThreads, 2) k_gth(GrainDev gd, ChunkDev ch
     const int rank = CLUSTER ? (int)(blockIdx.x % C) : 0, sp = CLUSTER ? (int)(blockIdx.x / C) : (int)blockIdx.x;
     const int nC = CLUSTER ? C : 1;
     int cell, g;
-    td_spectrum(ch, gorder, s0, cell, g, sp);
+    td_spectrum(ch, gorder, s0, sp, cell, g);
     const int off = gd.bin_off[g], nb = gd.bin_off[g + 1] - off;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     double* Ls = smd;                      // [rcap][kGthB], rcap even

@@ -10,26 +10,6 @@
 
 namespace heat {
 
-// Task loop of the persistent launches: with ch.work set, each warp takes the next task of
-// the list from an atomic counter (dynamic scheduling per warp, in the list's order, as the
-// paper's dynamic OpenMP schedule does per thread); without it, one warp per task.
-template <typename F>
-__device__ __forceinline__ void for_each_task(const ChunkDev& ch, int counter, F&& run) {
-    const int lane = threadIdx.x & 31;
-    if (!ch.work) {
-        const int task = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-        if (task < ch.n_tasks) run(task, lane);
-        return;
-    }
-    for (;;) {
-        int task = 0;
-        if (lane == 0) task = atomicAdd(ch.work + counter, 1);
-        task = __shfl_sync(0xffffffffu, task, 0);
-        if (task >= ch.n_tasks) return;
-        run(task, lane);
-    }
-}
-
 // ---------------------------------------------------------------------------
 // k_recur: the recursion kernel.  X_0 = 1,
 //   X_f = (sum_{j in band(f)} B_fj X_j) / T_{f-1,f}                              (Eq. xf)
@@ -1086,9 +1066,10 @@ cudaError_t launch_recur(const GrainDev& g, const ChunkDev& ch, int build, cudaS
         const size_t smem = base + (staged ? band : 0);
         using KernT = void (*)(GrainDev, ChunkDev, int);
         KernT kern = nullptr;
-#define HEAT_SMALL_PICK(B, P) \
-    kern = warp ? k_recur_small<B, P, 1, true> : (K == 1 ? k_recur_small<B, P, 1, false> : k_recur_small<B, P, 4, false>)
-        if (build == 0) {
+#define HEAT_SMALL_PICK(B, P) kern = K == 1 ? k_recur_small<B, P, 1, false> : k_recur_small<B, P, 4, false>
+        if (warp) {  // (narrow rows without pruning are k_recur_chain's)
+            kern = build == 0 ? k_recur_small<0, true, 1, true> : k_recur_small<1, true, 1, true>;
+        } else if (build == 0) {
             if (ch.prune) HEAT_SMALL_PICK(0, true); else HEAT_SMALL_PICK(0, false);
         } else {
             if (ch.prune) HEAT_SMALL_PICK(1, true); else HEAT_SMALL_PICK(1, false);
