@@ -547,8 +547,8 @@ __global__ void __launch_bounds__(256) k_elem32(GrainDev gd, ChunkDev ch, int gb
 
 // ---------------------------------------------------------------------------
 // Element-parallel build for solves of few cells (ChunkDev::small): the same quantities as
-// k_build with the same expressions; the cumulative sums run in the same order (one thread),
-// so B is bit-identical.
+// k_build with the same expressions.  FP32: the cumulative sums run in the same order (one
+// thread), so B is bit-identical.  FP64: a warp scan, so B differs in the last bits.
 
 // Blocks per (cell, grain): S parts (256 threads each, dynamic shared memory 2 N doubles).
 // Every part forms the segment increments and the cumulative sums; part q writes the

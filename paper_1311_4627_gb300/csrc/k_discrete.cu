@@ -8,6 +8,8 @@
 //       from bin u to bin l, E in [E_u - Ehi_l, E_u - Elo_l] (l = u-1: [0, E_u - Elo_{u-1}],
 //       photons too soft to leave bin u included); the windows tile [0, E_u], so the rates
 //       carry the power Eq. cooling's adjacent rate carries.
+//   k_td_edges, k_td_env  (once per grain set): where the windows' edges fall on the grid, and
+//       which elements of a grain's rate matrix the state reduction touches.
 //   k_td_fill  (per spectrum): the rate matrix q[i][j] (from i to j): heating elements
 //       T_ji, j > i, as closed-form integrals over the target bin's wavelength window of the
 //       log-log interpolant of Omega = u C (plus the intra-bin term on j = i + 1), downward
@@ -16,9 +18,9 @@
 //       removed, their rates redistributed, q_ij += q_in q_nj / s_n with s_n = sum_{j<n} q_nj
 //       (sums and products of non-negative numbers only); then X_0 = 1,
 //       X_n = sum_{i<n} X_i q_in / s_n, power-of-two rescales, P = X / sum X.  About M^3/3
-//       fused multiply-adds per spectrum, on the FP64 unit: one block per spectrum, states
-//       removed eight at a time with one delayed rank-8 update of the rest (q in shared memory
-//       up to 160 bins, else in device memory, read and written once per eight states).
+//       fused multiply-adds per spectrum, on the FP64 unit, less where rates reach few bins: a
+//       block per spectrum, or a cluster of up to eight where a launch has few; states removed
+//       in panels of eight (kGthB), q in device memory, read and written once per panel.
 #include <algorithm>
 
 #include "common.cuh"
