@@ -213,6 +213,14 @@ __device__ __forceinline__ void finish_task(const GrainDev& gd, const ChunkDev& 
     }
 }
 
+// The same as a call.  Pruned kernels carry the pruning state through the row loop; inlined, the epilogue made the FP64
+// ones spill inside it (512 cells x 64 grains 1.24 ms, as a call 1.19).
+__device__ __noinline__ void finish_task_call(const GrainDev& gd, const ChunkDev& ch, int g, int cc, int M, int i_end,
+                                              double total, int epoch, long long xmaxb, const double* xl,
+                                              const unsigned short* epl, int part, int parts) {
+    finish_task(gd, ch, g, cc, M, i_end, true, total, epoch, xmaxb, xl, epl, part, parts);
+}
+
 // One task: the recursion of grain g for the 32 cells of group grp (lane = cell).  W is
 // the register window: the last W values of X, and the window part of each row's band
 // (its last min(width, W) elements), prefetched one row ahead.  The row loop's fixed
@@ -405,7 +413,10 @@ __device__ __forceinline__ void recur_task(const GrainDev& gd, const ChunkDev& c
 #pragma unroll
         for (int k = 0; k < W; ++k) br[k] = br_n[k];
     }
-    finish_task(gd, ch, g, cc, M, PRUNE ? f_last : M, PRUNE, total, epoch, xmaxb, xl, epl, 0, 1);
+    if constexpr (PRUNE)
+        finish_task_call(gd, ch, g, cc, M, f_last, total, epoch, xmaxb, xl, epl, 0, 1);
+    else
+        finish_task(gd, ch, g, cc, M, M, false, total, epoch, xmaxb, xl, epl, 0, 1);
     if (numeric_bad) atomicOr(ch.status, kStatNumeric);
 }
 
@@ -587,7 +598,10 @@ __device__ __noinline__ void recur_quad(const GrainDev& gd, const ChunkDev& ch, 
     __syncthreads();
     total = xs[0][lane];
     xmaxb = __double_as_longlong(xs[1][lane]);
-    finish_task(gd, ch, g, cc, M, PRUNE ? f_last : M, PRUNE, total, epoch, xmaxb, xl, epl, w, 4);
+    if constexpr (PRUNE)
+        finish_task_call(gd, ch, g, cc, M, f_last, total, epoch, xmaxb, xl, epl, w, 4);
+    else
+        finish_task(gd, ch, g, cc, M, M, false, total, epoch, xmaxb, xl, epl, w, 4);
     if (numeric_bad) atomicOr(ch.status, kStatNumeric);
 }
 
@@ -595,12 +609,15 @@ __device__ __noinline__ void recur_quad(const GrainDev& gd, const ChunkDev& ch, 
 // their loads and leave the FP64 unit to the wide ones beside them.  32 grains of 512 bins, 4096 cells: 0 9.0 ms, 1 7.4,
 // 2 6.9, 3 6.9.
 constexpr int kSinglesFirst = 2;
-template <int BUILD, bool PRUNE>
+// QUAD false: without the call of recur_quad, for pruned launches that have no task for a block (4096 cells x 64 grains:
+// 5.59 ms against 5.92 with the call in the kernel).  The unpruned kernels are as fast or faster with it (65536 cells x 32
+// grains of 512 bins: 116.2 ms against 124.8 without).
+template <int BUILD, bool PRUNE, bool QUAD>
 __global__ void __launch_bounds__(128, 5) k_recur(GrainDev gd, ChunkDev ch) {
-    __shared__ double xs[4][32];
-    __shared__ int next;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     auto quads = [&] {
+        __shared__ double xs[4][32];
+        __shared__ int next;
         for (;;) {
             __syncthreads();
             if (threadIdx.x == 0) next = atomicAdd(ch.work, 1);
@@ -628,16 +645,18 @@ __global__ void __launch_bounds__(128, 5) k_recur(GrainDev gd, ChunkDev ch) {
         if (task < ch.n_tasks) singles(task);
         return;
     }
-    const bool singles_first = ch.n_quad == 0 || (int)(blockIdx.x / ch.sms) < kSinglesFirst;
-    if (!singles_first) quads();
+    const bool singles_first = !QUAD || ch.n_quad == 0 || (int)(blockIdx.x / ch.sms) < kSinglesFirst;
+    if constexpr (QUAD)
+        if (!singles_first) quads();
     for (;;) {
         int task = 0;
-        if (lane == 0) task = ch.n_quad + atomicAdd(ch.work + 1, 1);
+        if (lane == 0) task = (QUAD ? ch.n_quad : 0) + atomicAdd(ch.work + 1, 1);
         task = __shfl_sync(0xffffffffu, task, 0);
         if (task >= ch.n_tasks) break;
         singles(task);
     }
-    if (singles_first && ch.n_quad > 0) quads();
+    if constexpr (QUAD)
+        if (singles_first && ch.n_quad > 0) quads();
 }
 
 // ---------------------------------------------------------------------------
@@ -1083,8 +1102,9 @@ cudaError_t launch_recur(const GrainDev& g, const ChunkDev& ch, int build, cudaS
         return cudaGetLastError();
     }
     if (ch.n_tasks == 0) return cudaSuccess;
-    auto kern = build == 0 ? (ch.prune ? k_recur<0, true> : k_recur<0, false>)
-                           : (ch.prune ? k_recur<1, true> : k_recur<1, false>);
+    const bool quad = ch.n_quad > 0;
+    auto kern = build == 0 ? (!ch.prune ? k_recur<0, false, true> : quad ? k_recur<0, true, true> : k_recur<0, true, false>)
+                           : (!ch.prune ? k_recur<1, false, true> : quad ? k_recur<1, true, true> : k_recur<1, true, false>);
     kern<<<task_grid(kern, ch), 128, 0, st>>>(g, ch);
     return cudaGetLastError();
 }
