@@ -552,21 +552,24 @@ __global__ void __launch_bounds__(256) k_elem32(GrainDev gd, ChunkDev ch, int gb
 
 // Blocks per (cell, grain): S parts (256 threads each, dynamic shared memory 2 N doubles).
 // Every part forms the segment increments and the cumulative sums; part q writes the
-// elements of the segments n = q (mod S), and the intra-bin terms whose diagonal element it
-// wrote: the diagonal (j+1, j) and bin j's soft-photon edge are the same wavelength,
-// hc/(Elo_{j+1} - E_j), so both fall in segment sf.n (sf.n < 0: the diagonal is not in the
-// band, part 0).  Few spectra (a single cell) then spread over many SMs.
+// elements of a run of segments, cut so that the parts have about as many elements each, and the
+// intra-bin terms whose diagonal element it wrote: the diagonal (j+1, j) and bin j's soft-photon
+// edge are the same wavelength, hc/(Elo_{j+1} - E_j), so both fall in segment sf.n (sf.n < 0: the
+// diagonal is not in the band, part 0).  Few spectra (a single cell) then spread over many SMs.
 // The sums are the serial part: FP32, one thread in the lane-per-cell kernel's order (its bits), on FP32 values
 // throughout (a conversion to or from FP64 takes the FP64 unit 64 cycles); FP64, a warp, a run of segments a lane
 // and a scan over the lanes.  The elements take a thread each.  Against a warp per segment and FP64 sums on one thread:
-// 5 cells x 64 grains x 1024 wavelengths (FP32) 216 -> 130 us, single cell (FP64) 28 -> 23 us.
+// 5 cells x 64 grains x 1024 wavelengths (FP32) 216 -> 119 us, single cell (FP64) 36 -> 15 us.  With the parts cut as
+// segments n = q (mod S), each part looking through all entries for its own: 130 and 23 us, and a cell of 8 grains of 900
+// bins, all reaching each other, 296 -> 805 us where this takes 258.
 template <int BUILD>
-__global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, int S) {
+__global__ void __launch_bounds__(256, BUILD ? 6 : 5) k_build_small(GrainDev gd, ChunkDev ch, int S) {
     using Real = typename std::conditional<BUILD == 0, double, float>::type;
     extern __shared__ double sm[];
     Real* sPhi = (Real*)sm;     // [N]: Phi before segment n (exclusive prefix)
     Real* sPsi = sPhi + gd.N;   // [N]: Psi after the segments above n (exclusive suffix)
     __shared__ Real sPhiEnd;
+    __shared__ int s_seg[2];
     __shared__ double sPsiTot;
     __shared__ float sPsiEnd32;  // FP32 build: the FP32 value of the compensated total
     const int N = gd.N, Cc = ch.Cc;
@@ -601,6 +604,15 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
         sPsi[n] = dpsi;
     }
     __syncthreads();
+    if (tid >= 64 && tid < 66) {  // beside the sums: the first segment whose entries begin at or after q / S of all
+        const int q = part + tid - 64;
+        int lo = 0, hi = N;
+        while (lo < hi && q < S) {
+            const int mid = (lo + hi) >> 1;
+            if ((long long)(sp[mid] - sp[0]) * S >= (long long)q * (sp[N] - sp[0])) hi = mid; else lo = mid + 1;
+        }
+        s_seg[tid - 64] = q == 0 ? 0 : q < S ? lo : N;
+    }
     // 2. the cumulative sums
     if constexpr (BUILD == 0) {
         if (tid < 64) {  // warp 0 upward over sPhi, warp 1 downward over sPsi
@@ -656,13 +668,15 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
         }
     }
     __syncthreads();
-    // 3. band elements of this part's segments, a thread each
-    for (int k = sp[0] + tid; k < sp[N - 1]; k += blockDim.x) {
-        const int n = gd.pat_seg[k];
-        if (n % S != part) continue;
+    // 3. band elements of this part's segments [n_lo, n_hi), a thread each
+    const int n_lo = s_seg[0], n_hi = s_seg[1];
+    for (int k = sp[n_lo] + tid, k1 = sp[min(n_hi, N - 1)]; k < k1; k += blockDim.x) {
+        const int n = BUILD ? gd.pat_seg[k] : __ldcs(gd.pat_seg + k);
         if (BUILD == 0) {
             const SegF64 s(gd, g, n, ch.ua64[(size_t)n * Cc + cell], ch.su64[(size_t)n * Cc + cell]);
-            const PatF64 pt = gd.pat64[k];
+            PatF64 pt;  // evict first: the recursion reads B next, which alone can fill the L2
+#pragma unroll
+            for (int w = 0; w < 3; ++w) ((int2*)&pt)[w] = __ldcs((const int2*)(gd.pat64 + k) + w);
             ch.Bb64[bb + (size_t)pt.e * 32] = s.element(sPhi[n], pt.t, pt.tau);
         } else {
             const float2 us = uasu[(size_t)n * Cc + cell];
@@ -672,7 +686,7 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
             ch.Bb32[bb + (size_t)a0.e * 32] = fmaf(us.x * a0.cat, sh ? e1f_small(z) : e1f(z), (float)sPhi[n]);
         }
     }
-    if ((N - 1) % S == part)
+    if (n_lo <= N - 1 && N - 1 < n_hi)
         for (int k = sp[N - 1] + tid; k < sp[N]; k += blockDim.x) {
             if (BUILD == 0)
                 ch.Bb64[bb + (size_t)gd.pat64[k].e * 32] = sPhiEnd;
@@ -683,7 +697,7 @@ __global__ void __launch_bounds__(256) k_build_small(GrainDev gd, ChunkDev ch, i
     // 4. intra-bin terms, one per soft entry (each has its own diagonal element)
     for (int p = gd.soft_off[g] + tid; p < gd.soft_off[g + 1]; p += blockDim.x) {
         const SoftF64 sf = gd.soft[p];
-        if ((sf.n < 0 ? 0 : sf.n % S) != part) continue;
+        if (sf.n < 0 ? part != 0 : sf.n < n_lo || sf.n >= n_hi) continue;
         if (BUILD == 0) {
             double v = 0.0;
             if (sf.n == N - 1) {
