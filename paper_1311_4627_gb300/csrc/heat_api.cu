@@ -457,6 +457,8 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
         double t;
         int diag;  // for a diagonal element, 1 + the lower bin's index over all grains, else 0
     };
+    std::vector<Ent> ents, sorted;
+    std::vector<size_t> ent_at(2 * (size_t)N + 1);
     std::vector<int> diag_e(nbt, 0), diag_ok(nbt, 0);
     std::vector<PointEnt> pent;  // point-rule entries (Eq. heating), column by column
     std::vector<RowEnt32> rent;  // every band element in row order (fused kernel)
@@ -473,7 +475,7 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
             invdE32[off + j] = (float)invdE[off + j];
         }
         long long band = 0;
-        std::vector<Ent> ents;
+        ents.clear();
         std::vector<int> row_e(nb, 0), row_jlo(nb, 0);  // band index of (f, jlo(f)) and jlo(f)
         // row 0 has no elements
         rowptr.push_back((int)band_total);
@@ -556,8 +558,13 @@ heat_status heat_set_grains(heat_ctx* ctx, int n_grains, const double* radius_cm
         cpieces.push_back(make_int4(g, cp0, nb, 0));
         // pattern: the grain's elements grouped by segment, the diagonal ones (which also carry an
         // intra-bin term) last in each
-        std::stable_sort(ents.begin(), ents.end(),
-                         [](const Ent& a, const Ent& b) { return a.n != b.n ? a.n < b.n : (a.diag > 0) < (b.diag > 0); });
+        // (by counting; equal ones keep their order)
+        std::fill(ent_at.begin(), ent_at.end(), 0);
+        for (const Ent& en : ents) ++ent_at[2 * (size_t)en.n + (en.diag > 0) + 1];
+        for (size_t b = 1; b < ent_at.size(); ++b) ent_at[b] += ent_at[b - 1];
+        sorted.resize(ents.size());
+        for (const Ent& en : ents) sorted[ent_at[2 * (size_t)en.n + (en.diag > 0)]++] = en;
+        ents.swap(sorted);
         size_t base = pat64.size();
         size_t k = 0;
         for (int n = 0; n <= N; ++n) {
