@@ -84,7 +84,8 @@ __device__ __noinline__ double chain_f64(int k0, int k1, const double* a, const 
 //     are left out.
 // Which form a column's bins take depends on K alone, so a cell's result does not depend on the others'.
 // Errors are below the FMA chain's (each row is rounded to FP64 once).  Measured at 512 cells x 64 grains x
-// 1024 wavelengths (36864 bins): 31.3 -> 10.7 ms.
+// 1024 wavelengths (36864 bins): 31.3 -> 10.7 ms; both operands are staged in the one form that their four takes (in both,
+// 11.3 ms).
 // Tile 64 rows x 32 columns per 256 threads, 4 x 2 outputs a thread, 16 bins staged at a time.
 template <typename TC>
 __global__ void __launch_bounds__(256, 2) k_gemm_i64(int M, int N, const int* __restrict__ koff,
@@ -116,24 +117,27 @@ __global__ void __launch_bounds__(256, 2) k_gemm_i64(int M, int N, const int* __
                 const int k = kb + 4 * q + u;
                 x[u] = (k < k1 && n < N) ? B[(size_t)k * ldb + n] : 0.0;
             }
-            const Align4 a = align4(x);
-            Bh[q][c] = make_uint4(a.h[0], a.h[1], a.h[2], a.h[3]);
-            Bl[q][c] = make_uint4(a.l[0], a.l[1], a.l[2], a.l[3]);
-            Be[q][c] = a.E;
             // compared as integers: the values are not negative (the FP64 unit takes 64 cycles a comparison)
             const int kn = k1 - (kb + 4 * q);  // bins of this four
             long long lo = (long long)(bits64(x[0]) & kMag64), hi = lo;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                Bm[q][u][c] = mant(x[u]);
+            for (int u = 1; u < 4; ++u)
                 if (u < kn) {
                     lo = min(lo, (long long)(bits64(x[u]) & kMag64));
                     hi = max(hi, (long long)(bits64(x[u]) & kMag64));
                 }
-            }
             if (hi >= 0x7ff0000000000000ll) badc[c] = 1;
             const int f = hi > 0 ? (hi - lo > (3LL << 52) ? 3 : 1) : 0;  // (a difference of 3 exponents: 2^3 to 2^4)
             const int any = __reduce_or_sync(0xffffffffu, f);
+            if (any == 1) {  // only the form that the four's columns take
+                const Align4 a = align4(x);
+                Bh[q][c] = make_uint4(a.h[0], a.h[1], a.h[2], a.h[3]);
+                Bl[q][c] = make_uint4(a.l[0], a.l[1], a.l[2], a.l[3]);
+                Be[q][c] = a.E;
+            } else if (any) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) Bm[q][u][c] = mant(x[u]);
+            }
             if (c == 0) flag[q] = any;
         }
         __syncthreads();
@@ -149,12 +153,16 @@ __global__ void __launch_bounds__(256, 2) k_gemm_i64(int M, int N, const int* __
                 x[u] = (m < M && k < k1) ? A[(size_t)m * lda + k] : 0.0;
                 nan |= (__double2hiint(x[u]) & 0x7ff00000) == 0x7ff00000;
             }
-            const Align4 a = align4(x);
-            Ah[q][r] = make_uint4(a.h[0], a.h[1], a.h[2], a.h[3]);
-            Al[q][r] = make_uint4(a.l[0], a.l[1], a.l[2], a.l[3]);
-            Ae[q][r] = a.E;
+            const int f = flag[q];
+            if (f == 1) {
+                const Align4 a = align4(x);
+                Ah[q][r] = make_uint4(a.h[0], a.h[1], a.h[2], a.h[3]);
+                Al[q][r] = make_uint4(a.l[0], a.l[1], a.l[2], a.l[3]);
+                Ae[q][r] = a.E;
+            } else if (f) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) Am[q][u][r] = mant(x[u]);
+                for (int u = 0; u < 4; ++u) Am[q][u][r] = mant(x[u]);
+            }
             if (nan) bad[r] = 1;
         }
         __syncthreads();
