@@ -840,22 +840,25 @@ static bool uses_two_pass(const heat_ctx* ctx, const heat_opts& o, int count) {
 }
 
 // Default cells per chunk: as many as 45 % of the device memory the library could use (free
-// memory plus the chunk scratch it already holds) allows for `nslots` chunks in flight (B band, the two-pass
-// build's prefix table, X history, field tables per 32-cell group), at least one group; with several slots the range
-// is also split evenly over them.  More cells per chunk means more warps in flight for the
-// latency-bound build and recursion kernels.
+// memory plus the chunk scratch it already holds) allows for `nslots` chunks in flight (B band,
+// X history, field tables per 32-cell group) and 60 % with the two-pass build's prefix table, at least one group; with
+// several slots the range is also split evenly over them.  More cells per chunk means more warps in flight for the
+// latency-bound build and recursion kernels; a table that is small beside the band does not make the chunks smaller
+// (65536 cells x 32 grains of 512 bins, 2048 wavelengths: within the 45 % it took 4 chunks instead of 3).
 static int default_chunk(heat_ctx* ctx, const heat_opts& o, int count, int nslots) {
     const size_t el = o.build == 0 ? 8 : 4;
     const size_t band_bytes = uses_fused(ctx, o, count) ? 0 : (size_t)ctx->band_per_cell * 32 * el;
     const size_t phi_bytes = uses_two_pass(ctx, o, count) ? (size_t)ctx->G * ctx->N * 32 * el : 0;
-    const size_t per_group = band_bytes + phi_bytes + (size_t)ctx->nbt * 32 * 10 + (size_t)ctx->N * 32 * 16;
+    const size_t per_group = band_bytes + (size_t)ctx->nbt * 32 * 10 + (size_t)ctx->N * 32 * 16;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = size_t(16) << 30;
     size_t held = 0;
     for (auto& sl : ctx->slots) held += sl.ua64.cap + sl.su64.cap + sl.ua32.cap + sl.Bb64.cap + sl.Bb32.cap + sl.phi.cap +
                                         sl.xs.cap + sl.ep.cap;
-    const size_t budget = std::max<size_t>(size_t(2) << 30, (size_t)(0.45 * (double)(free_b + held)));
-    size_t groups = std::max<size_t>(1, budget / (size_t)nslots / per_group);
+    auto budget = [&](double part) { return std::max<size_t>(size_t(2) << 30, (size_t)(part * (double)(free_b + held))); };
+    size_t groups = budget(0.45) / (size_t)nslots / per_group;
+    if (phi_bytes) groups = std::min(groups, budget(0.6) / (size_t)nslots / (per_group + phi_bytes));
+    groups = std::max<size_t>(1, groups);
     size_t want = ((size_t)count + 31) / 32;
     if (nslots > 1) want = (want + nslots - 1) / nslots;
     return (int)(std::min(groups, std::max<size_t>(1, want)) * 32);

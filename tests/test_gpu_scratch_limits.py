@@ -130,6 +130,33 @@ def test_only_the_two_pass_build_makes_room_for_its_table(workload, opts, chunks
         lib.close()
 
 
+def test_a_small_table_does_not_shrink_the_chunk():
+    """A prefix table of a tenth of the rest (one grain of 180 bins that all reach each other, 2000 wavelengths: 5.2 MB per 32
+    cells, 0.5 MB of table): 2 GB hold 412 groups without it, 375 with it; 395 are still one chunk."""
+    import torch
+
+    cells, lam = 395 * 32, W.wavelength_grid(2000)
+    u = W.three_bb_fields(lam, np.full(cells, 10.0), np.zeros(cells), np.full((cells, 3), 0.3))
+    wl = W.custom(lam, np.array([3.5e-8]), ["carbonaceous"], [180], u)
+    P = torch.empty(cells, wl.total_bins, dtype=torch.float64, device="cuda")
+    lib = Lib(wl)
+    s = torch.cuda.Stream()
+    hold = None
+    try:
+        lib.set_fields(wl.u)
+        hold = _Hold(4 << 30)
+        nodes = []
+        for chunk in (0, cells):
+            g = heat.Graph(lib.ctx, heat.heat_default_opts(**dict(OPTS, streams=1, chunk_cells=chunk)), P, None, s.cuda_stream)
+            nodes.append(g.kernel_nodes())
+            g.close()
+        assert nodes[0] == nodes[1]
+    finally:
+        if hold:
+            hold.release()
+        lib.close()
+
+
 @pytest.mark.parametrize("prefetch", [1, 2])
 def test_one_walk_prefetch_on_and_off(workload, prefetch):
     """The FP32 build without room for its prefix table (half the bytes of FP64), with and without its pattern prefetch."""
