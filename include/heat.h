@@ -110,7 +110,8 @@ typedef struct heat_opts {
     int cell_begin;     /* first cell solved (0-based)                                             */
     int cell_count;     /* cells solved; <= 0 means all cells from cell_begin                      */
     int chunk_cells;    /* cells per internal chunk (multiple of 32; 0 = library default: as many
-                           as 45 % of the usable device memory holds)                             */
+                           as 45 % of the usable device memory holds, 60 % with the prefix table
+                           of the two-pass matrix build)                                          */
     int host_io;        /* 1: P_out, j_out and ledger_out are host pointers; the library stages
                            through device memory and the call returns after the results are on
                            the host.  2: the same, asynchronous: the call returns once the work is
